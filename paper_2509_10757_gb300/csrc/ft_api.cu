@@ -615,9 +615,9 @@ ft_status build_table(ft_ctx *ctx, const ft_params &params, const std::vector<Jo
                 fill_cam_out(C, c ? j.so.right : j.so.left);
                 C.cell_ptr = reinterpret_cast<int *>(carve(sizeof(int) * (kCells + 1)));
                 C.cell16 = reinterpret_cast<uint16_t *>(carve(sizeof(uint16_t) * (kCells + 1)));
-                C.gkp = reinterpret_cast<float4 *>(carve(sizeof(float4) * (size_t)C.nk));
-                C.gdesc = reinterpret_cast<uint4 *>(carve(sizeof(uint4) * 2 * (size_t)C.nk));
-                C.gpos = reinterpret_cast<int *>(carve(sizeof(int) * (size_t)C.nk));
+                C.gq = reinterpret_cast<unsigned *>(carve(sizeof(unsigned) * (size_t)C.nk));
+                if (C.nk < 65536) C.gk16 = reinterpret_cast<uint16_t *>(carve(sizeof(uint16_t) * (size_t)C.nk));
+                else C.gk32 = reinterpret_cast<int *>(carve(sizeof(int) * (size_t)C.nk));
                 C.owner = reinterpret_cast<unsigned long long *>(carve(sizeof(unsigned long long) * (size_t)C.nk));
                 // a pinhole frame whose stereo step runs in the same launch splits
                 // its search around it (search items need not wait for it)

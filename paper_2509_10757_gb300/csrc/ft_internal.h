@@ -90,15 +90,16 @@ struct CamDev {
     int8_t *level;
     float4 *proj;
     int *mp_kp, *mp_d1, *mp_d2, *kp_mp;
-    int *cell_ptr;                 // [kCells + 1]
+    // the keypoint grid (scratch), in cell order; keypoints already taken
+    // are left out
+    int *cell_ptr;                 // [kCells + 1] cell starts
     uint16_t *cell16;              // [kCells + 1] the same starts in 16 bits (nk < 65536), 16-byte aligned
-    float4 *gkp;                   // [nk] keypoints in cell order: x, y,
-                                   // index | octave << 20 | taken << 28, right coordinate (or -1)
-    uint4 *gdesc;                  // [2 * nk]
-    int *gpos;                     // [nk] cell-order position of keypoint k (-1: outside the grid)
+    unsigned *gq;                  // [nk] packed place and octave of each placed keypoint (see pack_place)
+    uint16_t *gk16;                // [nk] its index (nk < 65536)
+    int *gk32;                     // [nk] its index (nk >= 65536, else NULL)
     unsigned long long *owner;     // [nk] (distance << 32) | map index
     uint4 *scan;                   // [2 * nm] split search: per map point its four smallest candidate keys,
-                                   // then (right coordinate, radius, their octaves, how many passed)
+                                   // then (right coordinate, radius, how many passed, 0)
 };
 
 struct FrameDev {

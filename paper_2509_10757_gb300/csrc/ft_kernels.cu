@@ -47,7 +47,8 @@ constexpr int kStripW = 2 * (kW + kL) + 1;                      // 21
 constexpr int kShifts = 2 * kL + 1;                             // 11
 constexpr int kBatch = 4;                                       // loads issued ahead per thread
 constexpr int kScatter = 3;                                     // keypoints per thread per scatter batch
-constexpr int kGridScatter = 2;
+constexpr int kGridBatch = 8;                                   // the same in the grid build
+constexpr float kPlaceX = 16383.0f, kPlaceY = 4095.0f;          // largest packed places (14 and 12 bits)
 
 // resident CTAs per SM the register budget is sized for
 #ifndef FT_MIN_CTAS_PER_SM
@@ -101,14 +102,14 @@ __device__ __forceinline__ void top2_push(unsigned key, unsigned &best, unsigned
 __device__ float atan_series(float a)
 {
     const float a2 = fmul(a, a);
-    float p = fdiv(1.0f, 17.0f);
-    p = fadd(-fdiv(1.0f, 15.0f), fmul(a2, p));
-    p = fadd(fdiv(1.0f, 13.0f), fmul(a2, p));
-    p = fadd(-fdiv(1.0f, 11.0f), fmul(a2, p));
-    p = fadd(fdiv(1.0f, 9.0f), fmul(a2, p));
-    p = fadd(-fdiv(1.0f, 7.0f), fmul(a2, p));
-    p = fadd(fdiv(1.0f, 5.0f), fmul(a2, p));
-    p = fadd(-fdiv(1.0f, 3.0f), fmul(a2, p));
+    float p = (1.0f / 17.0f);
+    p = fadd(-(1.0f / 15.0f), fmul(a2, p));
+    p = fadd((1.0f / 13.0f), fmul(a2, p));
+    p = fadd(-(1.0f / 11.0f), fmul(a2, p));
+    p = fadd((1.0f / 9.0f), fmul(a2, p));
+    p = fadd(-(1.0f / 7.0f), fmul(a2, p));
+    p = fadd((1.0f / 5.0f), fmul(a2, p));
+    p = fadd(-(1.0f / 3.0f), fmul(a2, p));
     p = fadd(1.0f, fmul(a2, p));
     return fmul(a, p);
 }
@@ -206,7 +207,6 @@ struct SmemStereo {
         PatchBuf patch;                // (a strip with a second pass stages its window again)
     } u;
     RefineJob ref[kThreads];
-    int gp[kSadChunk];                 // grid record of each match of the round (-1: none)
     int sad[kSadChunk][12];
     int bptr[kOctBuckets * kWinRows + 1];   // start of each (octave, window row) bucket
     int warp_sums[kWarps];
@@ -243,19 +243,36 @@ struct SmemMedian {
     int hist[256], hist2[256];          // high bytes; low bytes within the median's high byte
     int count, bin, before;
     int vals[kMedianSmem];
-    int gp[kMedianSmem];               // grid record of each left keypoint (searched frames)
 };
 
-constexpr int kSearchStage = 1536;              // keypoints of one camera the search keeps on chip
-
 constexpr int kCell16Bytes = (2 * (kCells + 1) + 15) / 16 * 16;   // 16-bit cell starts, whole chunks
+constexpr int kPool = 128;                      // candidates a warp collects before it compares them
+constexpr int kStep = 2;                        // candidates a lane tests per step
+constexpr int kPoolFull = kPool - 2 - 32 * kStep;   // collected candidates beyond which another step might not fit
+constexpr unsigned kPoolEnd = 127u;             // end of a point's chain of candidates
+constexpr int kSearchBuf = 64 * 1024;           // bytes for the staged grid and the split search's records
 
-// a camera's keypoints in cell order, staged for the search of one tile:
-// records (x, y, index | octave << 20 | taken << 28, right coordinate or -1)
-// then descriptors, and, when they fit behind them, the 16-bit cell starts
+// Where a keypoint lies, for the search's first test: x and y over the grid's
+// span (one cell more at each side, so that every placed keypoint is inside)
+// in 14 and 12 bits, and the octave in 4.
+struct PlaceScale {
+    float x0, y0, sx, sy;
+};
+
+// what a search item keeps on chip: the camera's pose, each warp's candidate
+// pool with the compared keys, then (buf) the staged grid (16-bit cell
+// starts, packed places, 16-bit indices) and, in a split search, its points'
+// records
 struct SmemSearch {
     float pose[12];
-    uint4 buf[kSearchStage * 3];
+    PlaceScale ps;
+    float iw, ih;                   // grid cells per pixel
+    int motion;                     // of a last-frame search (f2)
+    int staged;                     // the grid lies in buf
+    int qb;                         // bytes of the staged packed places
+    unsigned pool[kWarps][kPool];
+    unsigned key[kWarps][kPool];
+    uint4 buf[kSearchBuf / 16];
 };
 
 union Smem {
@@ -353,6 +370,35 @@ __device__ __forceinline__ int grid_cell(const CamDev &C, float iw, float ih, fl
     return cy * FT_GRID_COLS + cx;
 }
 
+__device__ __forceinline__ PlaceScale place_scale(const CamDev &C)
+{
+    PlaceScale s;
+    const float w = fsub(C.maxx, C.minx), h = fsub(C.maxy, C.miny);
+    s.x0 = fsub(C.minx, fdiv(w, (float)FT_GRID_COLS));
+    s.y0 = fsub(C.miny, fdiv(h, (float)FT_GRID_ROWS));
+    s.sx = fdiv(kPlaceX * (float)FT_GRID_COLS / (float)(FT_GRID_COLS + 2), w);
+    s.sy = fdiv(kPlaceY * (float)FT_GRID_ROWS / (float)(FT_GRID_ROWS + 2), h);
+    // a span too small to scale: every place is 0 and passes the first test
+    if (!(s.sx < 1e30f)) s.sx = 0.0f;
+    if (!(s.sy < 1e30f)) s.sy = 0.0f;
+    return s;
+}
+
+__device__ __forceinline__ unsigned place_of(float t, float top) { return (unsigned)f2i(fminf(fmaxf(t, 0.0f), top)); }
+
+__device__ __forceinline__ unsigned pack_place(const PlaceScale &s, float x, float y, unsigned oct)
+{
+    return place_of(fmul(fsub(x, s.x0), s.sx), kPlaceX) | place_of(fmul(fsub(y, s.y0), s.sy), kPlaceY) << 16 |
+           oct << 28;
+}
+
+// The keypoints that can be matched (in the grid, not taken, an octave below
+// 16) in cell order: 6 bytes each, so that a search item's staging of a whole
+// camera is short; coordinates, descriptors and right coordinates are read
+// from the frame's own arrays, for the few candidates that pass the first
+// test.  One block per camera; 8 keypoints' loads in flight per thread
+// (1200 keypoints: 6 us; with 48-byte records copied in cell order 10 us;
+// 8000 keypoints: 16 against 44 us).
 __device__ void grid_item(const BatchHeader &B, const FrameDev &F, int cam, SmemGrid &G,
                           int *s_flag)
 {
@@ -360,22 +406,37 @@ __device__ void grid_item(const BatchHeader &B, const FrameDev &F, int cam, Smem
     const int tid = threadIdx.x;
     const float iw = fdiv((float)FT_GRID_COLS, fsub(C.maxx, C.minx));
     const float ih = fdiv((float)FT_GRID_ROWS, fsub(C.maxy, C.miny));
+    const PlaceScale ps = place_scale(C);
     for (int c = tid; c < kCells; c += kThreads) G.cnt[c] = 0;
     __syncthreads();
-    for (int base = 0; base < C.nk; base += kBatch * kThreads) {
-        float x[kBatch], y[kBatch];
+    auto pass = [&](bool place) {
+        for (int base = 0; base < C.nk; base += kGridBatch * kThreads) {
+            float x[kGridBatch], y[kGridBatch];
+            unsigned oct[kGridBatch], tk[kGridBatch];
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-            const int k = base + u * kThreads + tid;
-            x[u] = k < C.nk ? __ldg(C.kx + k) : 0.0f;
-            y[u] = k < C.nk ? __ldg(C.ky + k) : 0.0f;
-        }
+            for (int u = 0; u < kGridBatch; ++u) {
+                const int k = min(base + u * kThreads + tid, C.nk - 1);
+                x[u] = __ldg(C.kx + k);
+                y[u] = __ldg(C.ky + k);
+                oct[u] = (unsigned)(int)__ldg(C.koct + k);
+                tk[u] = C.taken ? (unsigned)__ldg(C.taken + k) : 0u;
+            }
 #pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-            const int c = grid_cell(C, iw, ih, x[u], y[u]);
-            if (base + u * kThreads + tid < C.nk && c >= 0) atomicAdd(&G.cnt[c], 1);
+            for (int u = 0; u < kGridBatch; ++u) {
+                const int k = base + u * kThreads + tid;
+                if (k >= C.nk) continue;
+                if (!place) C.owner[k] = ~0ull;
+                const int c = grid_cell(C, iw, ih, x[u], y[u]);
+                if (c < 0 || tk[u] || oct[u] > 15u) continue;
+                const int pos = atomicAdd(&G.cnt[c], 1);
+                if (!place) continue;
+                C.gq[pos] = pack_place(ps, x[u], y[u], oct[u]);
+                if (C.gk32) C.gk32[pos] = k;
+                else C.gk16[pos] = (uint16_t)k;
+            }
         }
-    }
+    };
+    pass(false);
     __syncthreads();
     mark(B, 0);
     const int total = block_scan(G.cnt, G.cnt, kCells, G.warp_sums);
@@ -389,42 +450,7 @@ __device__ void grid_item(const BatchHeader &B, const FrameDev &F, int cam, Smem
     }
     __syncthreads();
     mark(B, 1);
-    // the record's right coordinate: a stereo step in this launch fills it
-    // in later (pinhole frames that wait for their stereo); otherwise it is
-    // the caller's u_right input, or -1 (no consistency check)
-    const bool ur_in = C.model == FT_CAMERA_PINHOLE && F.u_right_in != nullptr && !F.wait_stereo;
-    for (int base = 0; base < C.nk; base += kGridScatter * kThreads) {
-        float x[kGridScatter], y[kGridScatter], ur[kGridScatter];
-        unsigned oct[kGridScatter], tk[kGridScatter];
-        uint4 d0[kGridScatter], d1[kGridScatter];
-#pragma unroll
-        for (int u = 0; u < kGridScatter; ++u) {
-            const int k = min(base + u * kThreads + tid, C.nk - 1);
-            x[u] = __ldg(C.kx + k);
-            y[u] = __ldg(C.ky + k);
-            oct[u] = (unsigned)__ldg(C.koct + k) & 0xffu;
-            tk[u] = C.taken ? (__ldg(C.taken + k) != 0) : 0u;
-            ur[u] = ur_in ? __ldg(F.u_right_in + k) : -1.0f;
-            d0[u] = __ldg(C.kdesc + 2 * k);
-            d1[u] = __ldg(C.kdesc + 2 * k + 1);
-        }
-#pragma unroll
-        for (int u = 0; u < kGridScatter; ++u) {
-            const int k = base + u * kThreads + tid;
-            if (k >= C.nk) continue;
-            const int c = grid_cell(C, iw, ih, x[u], y[u]);
-            int pos = -1;
-            if (c >= 0) {
-                pos = atomicAdd(&G.cnt[c], 1);
-                C.gkp[pos] = make_float4(x[u], y[u], __uint_as_float((unsigned)k | (oct[u] << 20) | (tk[u] << 28)),
-                                         ur[u]);
-                C.gdesc[2 * pos] = d0[u];
-                C.gdesc[2 * pos + 1] = d1[u];
-            }
-            C.gpos[k] = pos;
-            C.owner[k] = ~0ull;
-        }
-    }
+    pass(true);
     mark(B, 2);
     signal_count(&F.ctr[C_GRID_DONE], (unsigned)F.n_grid_items, s_flag);
     mark(B, 3);
@@ -701,7 +727,7 @@ __device__ void hamming_phase(const DevParams &P, const FrameDev &F, SmemStereo 
 //     row's part of the 11 SADs of centre-subtracted patches; then per match
 //     the first strict minimum over the shifts, the parabola, disparity and
 //     depth.
-__device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &S, int r0, int nc, bool rec)
+__device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &S, int r0, int nc)
 {
     const int tid = threadIdx.x;
     constexpr int kRows = 2 * kW + 1;
@@ -730,12 +756,6 @@ __device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + row * dstep),
                          "l"(src + (size_t)row * pitch)
                          : "memory");
-    }
-    // the grid record of each match (the search reads the right coordinate there)
-    if (rec && tid < nc) {
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(&S.gp[tid]);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(F.cam[0].gpos + S.ref[r0 + tid].i)
-                     : "memory");
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
@@ -804,7 +824,6 @@ __device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &
             }
         }
         write_stereo(F, J.i, J.j, J.d, shift, sadb, ur, dep);
-        if (rec && sadb >= 0 && S.gp[m] >= 0) reinterpret_cast<float *>(F.cam[0].gkp + S.gp[m])[3] = ur;
     }
     __syncthreads();
 }
@@ -849,38 +868,30 @@ __device__ __forceinline__ int median_value(const FrameDev &F, const SmemMedian 
 
 constexpr int kMedianBatch = 8;   // values a thread loads at once in the median's first pass
 
-__device__ void median_reject(const BatchHeader &B, const FrameDev &F, SmemMedian &M, bool grid_ok)
+__device__ void median_reject(const BatchHeader &B, const FrameDev &F, SmemMedian &M)
 {
     const DevParams &P = B.p;
     const int tid = threadIdx.x;
-    // a search in this launch reads the final right coordinates from the
-    // grid records (the strip waited for the grid step): a rejected match
-    // takes its coordinate back there too
-    const bool rec = F.wait_stereo && F.u_right_in != nullptr && grid_ok;
     const bool on_chip = F.nl <= kMedianSmem;
     for (int b = tid; b < 256; b += kThreads) M.hist[b] = M.hist2[b] = 0;
     if (tid == 0) M.count = 0;
     __syncthreads();
-    // one pass over the values (kept on chip with each keypoint's grid
-    // record when they fit): the count and the histogram of the high bytes;
-    // a thread loads kMedianBatch values before it stores or counts any
+    // one pass over the values (kept on chip when they fit): the count and
+    // the histogram of the high bytes; a thread loads kMedianBatch values
+    // before it stores or counts any
     int local = 0;
     for (int i0 = tid; i0 < F.nl; i0 += kThreads * kMedianBatch) {
-        int xv[kMedianBatch], gv[kMedianBatch];
+        int xv[kMedianBatch];
 #pragma unroll
         for (int u = 0; u < kMedianBatch; ++u) {
             const int i = i0 + u * kThreads;
             xv[u] = i < F.nl ? __ldcg(F.sad_best + i) : -1;
-            gv[u] = on_chip && rec && i < F.nl ? __ldcg(F.cam[0].gpos + i) : -1;
         }
 #pragma unroll
         for (int u = 0; u < kMedianBatch; ++u) {
             const int i = i0 + u * kThreads;
             if (i >= F.nl) continue;
-            if (on_chip) {
-                M.vals[i] = xv[u];
-                if (rec) M.gp[i] = gv[u];
-            }
+            if (on_chip) M.vals[i] = xv[u];
             if (xv[u] >= 0) {
                 atomicAdd(&M.hist[(xv[u] >> 8) & 255], 1);
                 ++local;
@@ -906,17 +917,12 @@ __device__ void median_reject(const BatchHeader &B, const FrameDev &F, SmemMedia
     __syncthreads();
     const int median = (hi << 8) | M.bin;
     const float th = fmul(P.median_factor, (float)median);
-    const CamDev &C = F.cam[0];
     for (int i = tid; i < F.nl; i += kThreads) {
         const int x = median_value(F, M, on_chip, i);
         if (x < 0) continue;
         if ((float)x >= th) {
             F.u_right[i] = -1.0f;
             F.depth[i] = -1.0f;
-            if (rec) {
-                const int pos = on_chip ? M.gp[i] : __ldcg(C.gpos + i);
-                if (pos >= 0) reinterpret_cast<float *>(C.gkp + pos)[3] = -1.0f;
-            }
         }
     }
 }
@@ -964,11 +970,7 @@ __device__ void stereo_pinhole_item(const BatchHeader &B, const FrameDev &F, int
     SmemStereo &S = U.s;
     const DevParams &P = B.p;
     const int tid = threadIdx.x;
-    // a search in this launch reads each refined match's right coordinate
-    // from the grid record, written once the grid step is done
-    const bool rec = F.wait_stereo && F.u_right_in != nullptr;
-    bool ready = wait_geq(B, &F.ctr[C_ROWS_DONE], (unsigned)F.rowsort, s_flag);
-    if (ready) {
+    if (wait_geq(B, &F.ctr[C_ROWS_DONE], (unsigned)F.rowsort, s_flag)) {
         const int H = F.H;
         const int r_lo = strip * F.strip_rows;
         const int r_hi = min(H, r_lo + F.strip_rows);
@@ -997,23 +999,18 @@ __device__ void stereo_pinhole_item(const BatchHeader &B, const FrameDev &F, int
             __syncthreads();
             mark(B, 0);
             hamming_phase(P, F, S, npass, staged, w_a, nrows);
-            // the refinement writes the grid records: the grid step must be done
-            if (rec && pass == l_lo) ready = wait_geq(B, &F.ctr[C_GRID_DONE], (unsigned)F.n_grid_items, s_flag);
-            else __syncthreads();
+            __syncthreads();
             mark(B, 1);
             const int nref = S.nref;
             for (int r0 = 0; r0 < nref; r0 += kSadChunk)
-                refine_round(P, F, S, r0, min(kSadChunk, nref - r0), rec && ready);
+                refine_round(P, F, S, r0, min(kSadChunk, nref - r0));
             if (tid == 0) S.nref = 0;
             __syncthreads();
             mark(B, 2);
         }
     }
     if (signal_count(&F.ctr[C_STEREO_DONE], (unsigned)F.n_stereo_items, s_flag)) {
-        // the rejection writes grid records too (this strip may have had no
-        // keypoints to refine, so it has not waited for the grid step yet)
-        if (rec && ready) ready = wait_geq(B, &F.ctr[C_GRID_DONE], (unsigned)F.n_grid_items, s_flag);
-        median_reject(B, F, U.m, ready);
+        median_reject(B, F, U.m);
         __threadfence();
         __syncthreads();
         mark(B, 3);
@@ -1321,219 +1318,204 @@ __device__ bool project(const DevParams &P, const CamDev &C, const float *pose, 
     return project_uv(C, pose, pos, u, v, ur) && distance_scale(P, C.O, pos, nrm, vc, level);
 }
 
-// One map point against the keypoints of its search window.  kStaged: the
-// camera's cell-ordered records and descriptors sit in shared memory.
+// The search of one map point, as its lane holds it: the projection, the
+// radius and the window of grid cells (active: the point is in view and its
+// window meets the grid), the same window in packed places (widened by a
+// place, so that it keeps every keypoint the exact test keeps) and the
+// octaves searched (bit o).
+struct PointWindow {
+    bool active;
+    int level, x0, x1, y0, y1;
+    unsigned lo, hi, octs;
+    float u, v, ur, vc, r;
+};
+
 // motion: for a last-frame search, +1 / -1 / 0 for a camera that moved
 // forward / backward / neither along its viewing axis (f2).
-// kScan: the first half of a search split around the stereo step.  Every
-// test but the stereo consistency is applied; the four smallest keys
-// (distance << 20 | keypoint) that pass, their octaves, the number that
-// passed and the projection's right coordinate and radius go to C.scan for
-// finish_point, which applies the consistency once the stereo step is done.
-// The consistency test drops candidates and keys are unique, so the two
-// smallest consistent keys among the four smallest candidates are the two
-// smallest consistent candidates, unless fewer than two of the four are
-// consistent while more than four passed: only then is the point searched
-// again.
-template <bool kStaged, bool kScan = false>
-__device__ void search_point(const DevParams &P, const FrameDev &F, const CamDev &C, const SmemSearch &Q,
-                             const uint16_t *scell, float iw, float ih, int m, int motion)
+__device__ __forceinline__ PointWindow point_window(const DevParams &P, const FrameDev &F, const CamDev &C,
+                                                    const SmemSearch &Q, int m)
 {
     const float *pose = Q.pose;
-    const float4 *srec = reinterpret_cast<const float4 *>(Q.buf);
-    const uint4 *sdesc = Q.buf + C.nk;
+    const PlaceScale &ps = Q.ps;
+    const float iw = Q.iw, ih = Q.ih;
+    const int motion = Q.motion;
+    PointWindow W;
+    W.active = false;
+    W.level = -1;
+    W.u = W.v = W.ur = W.vc = W.r = 0.0f;
+    W.x0 = W.x1 = W.y0 = W.y1 = 0;
+    W.lo = W.hi = W.octs = 0u;
     const bool last = F.search_mode != 0;
-    int lvl = -1, d1 = -1, d2 = -1, kp = -1;
-    float4 pj = make_float4(0.f, 0.f, 0.f, 0.f);
-    unsigned sk[4] = {kNoKey, kNoKey, kNoKey, kNoKey};   // kScan: four smallest keys, ascending
-    unsigned soct = 0, scount = 0;                          // their octaves (a byte each), how many passed
-    float sr = 0.0f, sur = 0.0f;
     const int loct = last ? (int)__ldg(F.last_oct + m) : 0;
-    const bool skipped = (F.skip != nullptr && __ldg(F.skip + m) != 0) || (last && (loct < 0 || loct >= P.nlevels));
-    if (!skipped) {
-        const float4 pos = __ldg(F.pos + m);
-        float u, v, ur, vc = 0.0f;
-        int level = loct;
-        const bool in_view = last ? project_uv(C, pose, pos, u, v, ur)
-                                  : project(P, C, pose, pos, __ldg(F.nrm + m), u, v, ur, vc, level);
-        if (in_view) {
-            lvl = level;
-            pj = make_float4(u, v, ur, vc);
-            float r;
-            int min_oct = level - 1, max_oct = level;
-            if (last) {
-                // f2: radius of the last octave, octave window by the motion
-                r = fmul(P.th_last, P.sc[level]);
-                min_oct = motion > 0 ? level : (motion < 0 ? 0 : level - 1);
-                max_oct = motion > 0 ? P.nlevels - 1 : (motion < 0 ? level : level + 1);
-            } else {
-                r = (vc > P.view_cos_narrow) ? P.radius_narrow : P.radius_wide;
-                r = fmul(r, P.search_th);
-                r = fmul(r, P.sc[level]);
-            }
-            const float du = fsub(u, C.minx), dv = fsub(v, C.miny);
-            const int x0 = max(f2i(floorf(fmul(fsub(du, r), iw))), 0);
-            const int x1 = min(f2i(ceilf(fmul(fadd(du, r), iw))), FT_GRID_COLS - 1);
-            const int y0 = max(f2i(floorf(fmul(fsub(dv, r), ih))), 0);
-            const int y1 = min(f2i(ceilf(fmul(fadd(dv, r), ih))), FT_GRID_ROWS - 1);
-            sr = r;
-            sur = ur;
-            if (!(x0 >= FT_GRID_COLS || x1 < 0 || y0 >= FT_GRID_ROWS || y1 < 0)) {
-                const uint4 q0 = __ldg(F.mdesc + 2 * m), q1 = __ldg(F.mdesc + 2 * m + 1);
-                const bool check_ur = C.model == FT_CAMERA_PINHOLE;
-                unsigned best = kNoKey, second = kNoKey;
-                int oct1 = -1, oct2 = -1;
-                for (int cy = y0; cy <= y1; ++cy) {
-                    int e0, e1;
-                    if (kStaged && scell != nullptr) {
-                        e0 = scell[cy * FT_GRID_COLS + x0];
-                        e1 = scell[cy * FT_GRID_COLS + x1 + 1];
-                    } else {
-                        e0 = __ldcg(C.cell_ptr + cy * FT_GRID_COLS + x0);
-                        e1 = __ldcg(C.cell_ptr + cy * FT_GRID_COLS + x1 + 1);
-                    }
-                    // records in device memory arrive kBatchRec at a time (one
-                    // round trip), the descriptors of those that pass the tests after
-                    constexpr int kBatchRec = kStaged ? 1 : 4;
-                    for (int eb = e0; eb < e1; eb += kBatchRec) {
-                        float4 gb[kBatchRec];
-#pragma unroll
-                        for (int q = 0; q < kBatchRec; ++q) {
-                            if (kStaged) gb[q] = srec[eb + q];
-                            else gb[q] = eb + q < e1 ? __ldcg(C.gkp + eb + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-#pragma unroll
-                        for (int q = 0; q < kBatchRec; ++q) {
-                            const int e = eb + q;
-                            if (e >= e1) break;
-                            const float4 g = gb[q];
-                            const unsigned z = __float_as_uint(g.z);
-                            const int k = (int)(z & 0xfffffu);
-                            const int oct = (int)(int8_t)((z >> 20) & 0xffu);
-                            if (oct < min_oct || oct > max_oct) continue;
-                            const float distx = fsub(g.x, u), disty = fsub(g.y, v);
-                            if (!(fabsf(distx) < r && fabsf(disty) < r)) continue;
-                            if (z >> 28) continue;                         // taken
-                            if (!kScan && check_ur && g.w > 0.0f && fabsf(fsub(ur, g.w)) > r) continue;
-                            const uint4 b0 = kStaged ? sdesc[2 * e] : __ldcg(C.gdesc + 2 * e);
-                            const uint4 b1 = kStaged ? sdesc[2 * e + 1] : __ldcg(C.gdesc + 2 * e + 1);
-                            const unsigned key = ((unsigned)ham8(q0, q1, b0, b1) << 20) | (unsigned)k;
-                            if (kScan) {
-                                scount = min(scount + 1u, 255u);
-                                const unsigned ob = (unsigned)oct & 0xffu;
-                                if (key < sk[3]) {
-                                    if (key < sk[2]) {
-                                        sk[3] = sk[2];
-                                        if (key < sk[1]) {
-                                            sk[2] = sk[1];
-                                            if (key < sk[0]) {
-                                                sk[1] = sk[0];
-                                                sk[0] = key;
-                                                soct = (soct << 8) | ob;
-                                            } else {
-                                                sk[1] = key;
-                                                soct = (soct & 0xffu) | ((soct << 8) & 0xff0000u) |
-                                                       ((soct << 8) & 0xff000000u) | ob << 8;
-                                            }
-                                        } else {
-                                            sk[2] = key;
-                                            soct = (soct & 0xffffu) | ((soct << 8) & 0xff000000u) | ob << 16;
-                                        }
-                                    } else {
-                                        sk[3] = key;
-                                        soct = (soct & 0xffffffu) | ob << 24;
-                                    }
-                                }
-                                continue;
-                            }
-                            if (key < best) {
-                                second = best;
-                                oct2 = oct1;
-                                best = key;
-                                oct1 = oct;
-                            } else if (key < second) {
-                                second = key;
-                                oct2 = oct;
-                            }
-                        }
-                    }
-                }
-                if (best != kNoKey) {
-                    d1 = (int)(best >> 20);
-                    d2 = second != kNoKey ? (int)(second >> 20) : 256;
-                    if (d1 <= P.th_search) {
-                        const int k1 = (int)(best & 0xfffffu);
-                        const bool ratio = !last && (P.ratio_any_octave || oct1 == oct2);
-                        if (!(ratio && (float)d1 > fmul(P.nn_ratio, (float)d2))) {
-                            atomicMin(C.owner + k1, ((unsigned long long)d1 << 32) | (unsigned)m);
-                            kp = k1;
-                        }
-                    }
-                }
-            }
-        }
+    if ((F.skip != nullptr && __ldg(F.skip + m) != 0) || (last && (loct < 0 || loct >= P.nlevels))) return W;
+    const float4 pos = __ldg(F.pos + m);
+    float u, v, ur, vc = 0.0f;
+    int level = loct;
+    const bool in_view = last ? project_uv(C, pose, pos, u, v, ur)
+                              : project(P, C, pose, pos, __ldg(F.nrm + m), u, v, ur, vc, level);
+    if (!in_view) return W;
+    W.level = level;
+    W.u = u;
+    W.v = v;
+    W.ur = ur;
+    W.vc = vc;
+    float r;
+    int min_oct = level - 1, max_oct = level;
+    if (last) {
+        // f2: radius of the last octave, octave window by the motion
+        r = fmul(P.th_last, P.sc[level]);
+        min_oct = motion > 0 ? level : (motion < 0 ? 0 : level - 1);
+        max_oct = motion > 0 ? P.nlevels - 1 : (motion < 0 ? level : level + 1);
+    } else {
+        r = (vc > P.view_cos_narrow) ? P.radius_narrow : P.radius_wide;
+        r = fmul(r, P.search_th);
+        r = fmul(r, P.sc[level]);
     }
-    C.level[m] = (int8_t)lvl;
-    if (C.proj) C.proj[m] = pj;
-    if (kScan) {
-        C.scan[2 * m] = make_uint4(sk[0], sk[1], sk[2], sk[3]);
-        C.scan[2 * m + 1] = make_uint4(__float_as_uint(sur), __float_as_uint(sr), soct, scount);
-        return;
-    }
-    C.mp_d1[m] = d1;
-    C.mp_d2[m] = d2;
-    C.mp_kp[m] = kp;
+    W.r = r;
+    const float du = fsub(u, C.minx), dv = fsub(v, C.miny);
+    W.x0 = max(f2i(floorf(fmul(fsub(du, r), iw))), 0);
+    W.x1 = min(f2i(ceilf(fmul(fadd(du, r), iw))), FT_GRID_COLS - 1);
+    W.y0 = max(f2i(floorf(fmul(fsub(dv, r), ih))), 0);
+    W.y1 = min(f2i(ceilf(fmul(fadd(dv, r), ih))), FT_GRID_ROWS - 1);
+    W.active = !(W.x0 >= FT_GRID_COLS || W.x1 < 0 || W.y0 >= FT_GRID_ROWS || W.y1 < 0);
+    const float pu = fsub(u, ps.x0), pv = fsub(v, ps.y0);
+    W.lo = place_of(fsub(fmul(fsub(pu, r), ps.sx), 1.0f), kPlaceX) |
+           place_of(fsub(fmul(fsub(pv, r), ps.sy), 1.0f), kPlaceY) << 16;
+    W.hi = place_of(fadd(fmul(fadd(pu, r), ps.sx), 1.0f), kPlaceX) |
+           place_of(fadd(fmul(fadd(pv, r), ps.sy), 1.0f), kPlaceY) << 16;
+    W.octs = (0xffffu >> (15 - clampi(max_oct, 0, 15))) & ~((1u << clampi(min_oct, 0, 15)) - 1u);
+    return W;
 }
 
-// The second half of a split search (see search_point): the stereo
-// consistency applied to the four smallest candidates of map point m, then
-// the top-2 rules and the claim, exactly as the unsplit search takes them.
-// A point that needs more than its four smallest candidates is searched
-// again from the device-memory records (whose right coordinates are final).
-__device__ void finish_point(const DevParams &P, const FrameDev &F, const CamDev &C, const SmemSearch &Q, float iw,
-                             float ih, int m, int motion)
+// The grid as a search item reads it: staged in shared memory, or in device
+// memory.
+__device__ __forceinline__ int grid_start(const CamDev &C, const SmemSearch &Q, int c)
 {
-    const uint4 ks = __ldcg(C.scan + 2 * m), aux = __ldcg(C.scan + 2 * m + 1);
-    const unsigned sk[4] = {ks.x, ks.y, ks.z, ks.w};
-    const float ur = __uint_as_float(aux.x), r = __uint_as_float(aux.y);
-    const unsigned count = aux.w;
-    const bool check_ur = C.model == FT_CAMERA_PINHOLE;
-    const bool last = F.search_mode != 0;
-    unsigned best = kNoKey, second = kNoKey;
-    int oct1 = -1, oct2 = -1;
+    return Q.staged ? (int)reinterpret_cast<const uint16_t *>(Q.buf)[c] : __ldcg(C.cell_ptr + c);
+}
+__device__ __forceinline__ unsigned grid_place(const CamDev &C, const SmemSearch &Q, int e)
+{
+    return Q.staged ? reinterpret_cast<const unsigned *>(Q.buf)[kCell16Bytes / 4 + e] : __ldcg(C.gq + e);
+}
+__device__ __forceinline__ int grid_index(const CamDev &C, const SmemSearch &Q, int e)
+{
+    if (Q.staged)
+        return (int)*reinterpret_cast<const uint16_t *>(reinterpret_cast<const unsigned char *>(Q.buf) + kCell16Bytes +
+                                                        Q.qb + 2 * e);
+    return C.gk32 ? __ldcg(C.gk32 + e) : (int)__ldcg(C.gk16 + e);
+}
+
+// A warp's 32 map points (point mw + lane in lane `lane`) against the
+// keypoints of their windows.  Each lane walks the cell rows of its own point
+// and applies the first test (packed place and octave: one shared-memory
+// word a candidate, 19 in 20 of which fail); what passes goes to the warp's
+// pool.  The pool's candidates are then shared out over the lanes, whichever
+// point they belong to, and get the exact tests and the Hamming distance
+// from the frame's own arrays, all their loads in flight at once; then each
+// lane takes its own point's keys (distance << 20 | keypoint) from its chain
+// in the pool and keeps the four smallest and their number.  What bounds it
+// is latency: a point has one or two candidates behind the first test, so
+// comparing them lane by lane as they are found leaves most lanes idle and
+// pays a round trip for each (1280x720, 4000 keypoints, 20000 points: 13 us
+// a point and thread that way).
+// check_ur: the stereo consistency is among the tests (the first half of a
+// search split around the stereo step leaves it out).
+__device__ __forceinline__ void gather(const FrameDev &F, const CamDev &C, SmemSearch &Q, const PointWindow &W, int mw,
+                                       bool check_ur, unsigned (&sk)[4], unsigned &count)
+{
+    const int lane = threadIdx.x & 31;
+    unsigned *const pool = Q.pool[threadIdx.x >> 5], *const pkey = Q.key[threadIdx.x >> 5];
+    bool active = W.active;
+    int cy = W.y0, e = 0, e1 = 0;
+    if (active) {
+        e = grid_start(C, Q, cy * FT_GRID_COLS + W.x0);
+        e1 = grid_start(C, Q, cy * FT_GRID_COLS + W.x1 + 1);
+    }
+    unsigned head = kPoolEnd;
+    int n = 0;                          // candidates in the pool (the same in every lane)
+    for (;;) {
+        if (active && e >= e1) {
+            if (cy < W.y1) {
+                ++cy;
+                e = grid_start(C, Q, cy * FT_GRID_COLS + W.x0);
+                e1 = grid_start(C, Q, cy * FT_GRID_COLS + W.x1 + 1);
+            } else {
+                active = false;
+            }
+        }
+        unsigned w[kStep];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        if ((unsigned)q >= count) break;
-        const unsigned key = sk[q];
-        const int k = (int)(key & 0xfffffu);
-        if (k >= C.nk) continue;                     // never: keys name keypoints of the window
-        if (check_ur) {
-            const int e = __ldcg(C.gpos + k);
-            if (e < 0) continue;                     // never: window keypoints lie in the grid
-            const float w = __ldcg(&C.gkp[e].w);
-            if (w > 0.0f && fabsf(fsub(ur, w)) > r) continue;
+        for (int s = 0; s < kStep; ++s) w[s] = active && e + s < e1 ? grid_place(C, Q, e + s) : 0u;
+#pragma unroll
+        for (int s = 0; s < kStep; ++s) {
+            const unsigned place = w[s] & 0x0fff3fffu;
+            const bool pass = active && e + s < e1 && __vminu2(__vmaxu2(place, W.lo), W.hi) == place &&
+                              ((W.octs >> (w[s] >> 28)) & 1u);
+            const unsigned hit = __ballot_sync(kFull, pass);
+            if (pass) {
+                const unsigned slot = (unsigned)(n + __popc(hit & ((1u << lane) - 1u)));
+                pool[slot] = (unsigned)(e + s) | ((unsigned)lane << 20) | (head << 25);
+                head = slot;
+            }
+            n += __popc(hit);
         }
-        const int oct = (int)(int8_t)((aux.z >> (8 * q)) & 0xffu);
-        if (best == kNoKey) {
-            best = key;
-            oct1 = oct;
-        } else {
-            second = key;
-            oct2 = oct;
-            break;
+        e += kStep;
+        const bool more = __any_sync(kFull, active);
+        if (more && n <= kPoolFull) continue;
+        __syncwarp();
+        for (int p = lane; p - lane < n; p += 32) {
+            const bool have = p < n;
+            const unsigned ent = have ? pool[p] : 0u;
+            const int o = (int)((ent >> 20) & 31u);
+            const float uo = __shfl_sync(kFull, W.u, o), vo = __shfl_sync(kFull, W.v, o);
+            const float ro = __shfl_sync(kFull, W.r, o), uro = __shfl_sync(kFull, W.ur, o);
+            if (!have) continue;
+            const int k = grid_index(C, Q, (int)(ent & 0xfffffu));
+            const float x = __ldg(C.kx + k), y = __ldg(C.ky + k);
+            const float w1 = check_ur ? __ldcg(F.u_right_in + k) : -1.0f;
+            const uint4 b0 = __ldg(C.kdesc + 2 * k), b1 = __ldg(C.kdesc + 2 * k + 1);
+            const uint4 q0 = __ldg(F.mdesc + 2 * (size_t)(mw + o)), q1 = __ldg(F.mdesc + 2 * (size_t)(mw + o) + 1);
+            bool ok = fabsf(fsub(x, uo)) < ro && fabsf(fsub(y, vo)) < ro;
+            if (w1 > 0.0f && fabsf(fsub(uro, w1)) > ro) ok = false;
+            pkey[p] = ok ? ((unsigned)ham8(q0, q1, b0, b1) << 20) | (unsigned)k : kNoKey;
         }
+        __syncwarp();
+        while (head != kPoolEnd) {
+            unsigned key = pkey[head];
+            head = pool[head] >> 25;
+            if (key == kNoKey) continue;
+            ++count;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const unsigned lo = min(sk[q], key);
+                key = max(sk[q], key);
+                sk[q] = lo;
+            }
+        }
+        __syncwarp();
+        n = 0;
+        if (!more) break;
     }
-    if (count > 4u && second == kNoKey) {
-        search_point<false>(P, F, C, Q, nullptr, iw, ih, m, motion);
-        return;
-    }
+}
+
+// The top-2 rules (threshold, ratio test) on a point's two smallest keys, the
+// claim of the keypoint, and the point's outputs.
+__device__ __forceinline__ void claim_point(const DevParams &P, const FrameDev &F, const CamDev &C, int m,
+                                            unsigned best, unsigned second)
+{
     int d1 = -1, d2 = -1, kp = -1;
     if (best != kNoKey) {
         d1 = (int)(best >> 20);
         d2 = second != kNoKey ? (int)(second >> 20) : 256;
         if (d1 <= P.th_search) {
             const int k1 = (int)(best & 0xfffffu);
-            const bool ratio = !last && (P.ratio_any_octave || oct1 == oct2);
+            bool ratio = F.search_mode == 0;
+            if (ratio && !P.ratio_any_octave) {
+                // the ratio test applies if both share an octave
+                const int o1 = __ldg(C.koct + k1);
+                const int o2 = second != kNoKey ? (int)__ldg(C.koct + (second & 0xfffffu)) : -1;
+                ratio = o1 == o2;
+            }
             if (!(ratio && (float)d1 > fmul(P.nn_ratio, (float)d2))) {
                 atomicMin(C.owner + k1, ((unsigned long long)d1 << 32) | (unsigned)m);
                 kp = k1;
@@ -1545,9 +1527,82 @@ __device__ void finish_point(const DevParams &P, const FrameDev &F, const CamDev
     C.mp_kp[m] = kp;
 }
 
+// How a search item passes over its points: the whole search; the first half
+// of a search split around the stereo step (each point's four smallest keys,
+// their number and the projection's right coordinate and radius go to its
+// record); or the whole search of the points that the second half left.
+enum SearchPass { kWhole, kFirstHalf, kLeftOver };
+
+// Map points [m0, m1), 32 a warp at a time; scan: their records (2 a point).
+__device__ __forceinline__ void search_points(const DevParams &P, const FrameDev &F, const CamDev &C, SmemSearch &Q,
+                                              uint4 *scan, int m0, int m1, SearchPass pass)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool check_ur = pass != kFirstHalf && C.model == FT_CAMERA_PINHOLE && F.u_right_in != nullptr;
+    for (int mw = m0 + 32 * warp; mw < m1; mw += kThreads) {
+        const int m = mw + lane;
+        const bool mine = m < m1 && (pass != kLeftOver || scan[2 * (m - m0) + 1].w != 0u);
+        PointWindow W;
+        W.active = false;
+        if (mine) {
+            W = point_window(P, F, C, Q, m);
+            C.level[m] = (int8_t)W.level;
+            if (C.proj) C.proj[m] = make_float4(W.u, W.v, W.ur, W.vc);
+        }
+        unsigned sk[4] = {kNoKey, kNoKey, kNoKey, kNoKey}, count = 0;
+        __syncwarp();
+        gather(F, C, Q, W, mw, check_ur, sk, count);
+        if (!mine) continue;
+        if (pass == kFirstHalf) {
+            scan[2 * (m - m0)] = make_uint4(sk[0], sk[1], sk[2], sk[3]);
+            scan[2 * (m - m0) + 1] = make_uint4(__float_as_uint(W.ur), __float_as_uint(W.r), count, 0u);
+        } else {
+            claim_point(P, F, C, m, sk[0], sk[1]);
+        }
+    }
+}
+
+// The second half of a split search, after the stereo step: the stereo
+// consistency applied to each point's four smallest candidates, then the
+// top-2 rules and the claim, exactly as the unsplit search takes them.  The
+// consistency test drops candidates and keys are unique, so the two smallest
+// consistent keys among the four smallest candidates are the two smallest
+// consistent candidates, unless fewer than two of the four are consistent
+// while more than four passed: only those points are left to be searched
+// again, with the consistency among the tests (true: there are some).
+__device__ __forceinline__ bool finish_points(const DevParams &P, const FrameDev &F, const CamDev &C, uint4 *scan,
+                                              int m0, int m1)
+{
+    const bool check_ur = C.model == FT_CAMERA_PINHOLE && F.u_right_in != nullptr;
+    bool left = false;
+    for (int m = m0 + (int)threadIdx.x; m < m1; m += kThreads) {
+        const uint4 ks = scan[2 * (m - m0)], aux = scan[2 * (m - m0) + 1];
+        const unsigned sk[4] = {ks.x, ks.y, ks.z, ks.w};
+        const float ur = __uint_as_float(aux.x), r = __uint_as_float(aux.y);
+        unsigned best = kNoKey, second = kNoKey;
+        float w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            w[q] = check_ur && sk[q] != kNoKey ? __ldcg(F.u_right_in + (sk[q] & 0xfffffu)) : -1.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (sk[q] == kNoKey || (w[q] > 0.0f && fabsf(fsub(ur, w[q])) > r)) continue;
+            if (best == kNoKey) best = sk[q];
+            else if (second == kNoKey) second = sk[q];
+        }
+        if (aux.z > 4u && second == kNoKey) {
+            scan[2 * (m - m0) + 1].w = 1u;
+            left = true;
+        } else {
+            claim_point(P, F, C, m, best, second);
+        }
+    }
+    return left;
+}
+
 // The camera pose of a search item in shared memory (the right fisheye
-// camera's composed from the rig), the grid scale and the last-frame motion.
-__device__ void search_setup(const FrameDev &F, int cam, SmemSearch &Q, float &iw, float &ih, int &motion)
+// camera's composed from the rig), the grid scales and the last-frame motion.
+__device__ void search_setup(const FrameDev &F, int cam, SmemSearch &Q)
 {
     const CamDev &C = F.cam[cam];
     const int tid = threadIdx.x;
@@ -1568,16 +1623,20 @@ __device__ void search_setup(const FrameDev &F, int cam, SmemSearch &Q, float &i
         }
         Q.pose[tid] = v;
     }
-    iw = fdiv((float)FT_GRID_COLS, fsub(C.maxx, C.minx));
-    ih = fdiv((float)FT_GRID_ROWS, fsub(C.maxy, C.miny));
-    motion = 0;
-    if (F.search_mode != 0) {
-        // the current (left) camera centre in the last frame's camera
-        // coordinates; its z against the baseline (f2)
-        const float *O = F.cam[0].O;
-        const float cz = fadd(fadd(fadd(fmul(F.last_R[6], O[0]), fmul(F.last_R[7], O[1])), fmul(F.last_R[8], O[2])),
-                              F.last_t[2]);
-        motion = cz > F.base ? 1 : (-cz > F.base ? -1 : 0);
+    if (tid == 32) {
+        Q.iw = fdiv((float)FT_GRID_COLS, fsub(C.maxx, C.minx));
+        Q.ih = fdiv((float)FT_GRID_ROWS, fsub(C.maxy, C.miny));
+        Q.ps = place_scale(C);
+        Q.motion = 0;
+        if (F.search_mode != 0) {
+            // the current (left) camera centre in the last frame's camera
+            // coordinates; its z against the baseline (f2)
+            const float *O = F.cam[0].O;
+            const float cz = fadd(fadd(fadd(fmul(F.last_R[6], O[0]), fmul(F.last_R[7], O[1])),
+                                       fmul(F.last_R[8], O[2])),
+                                  F.last_t[2]);
+            Q.motion = cz > F.base ? 1 : (-cz > F.base ? -1 : 0);
+        }
     }
 }
 
@@ -1619,52 +1678,49 @@ __device__ void search_item(const BatchHeader &B, const FrameDev &F, int tile, S
     if (ok) {
         SmemSearch &Q = U.q;
         const int tid = threadIdx.x;
-        float iw, ih;
-        int motion;
-        search_setup(F, cam, Q, iw, ih, motion);
-        // stage the camera's cell-ordered keypoint records and descriptors
-        // by asynchronous copies when they fit (the tail past the placed
-        // records is copied but never read)
+        search_setup(F, cam, Q);
+        // the camera's grid on chip by asynchronous copies when it fits (6
+        // bytes a keypoint and the cell starts: up to about 9900 keypoints;
+        // the tails past the placed keypoints are copied but never read)
         const int nk = C.nk;
-        const bool staged = F.search_stage == 0 && nk <= kSearchStage;
-        // the 16-bit cell starts too when they fit behind the descriptors
-        const bool cells = staged && 48 * nk + kCell16Bytes <= (int)sizeof(Q.buf);
-        const uint16_t *scell = cells ? reinterpret_cast<const uint16_t *>(Q.buf + 3 * nk) : nullptr;
+        const int qb = (4 * nk + 15) & ~15, kb = (2 * nk + 15) & ~15;
+        const bool staged = F.search_stage == 0 && nk < 65536 && kCell16Bytes + qb + kb <= kSearchBuf;
+        unsigned char *buf = reinterpret_cast<unsigned char *>(Q.buf);
+        const int used = staged ? kCell16Bytes + qb + kb : 0;
+        if (tid == 0) {
+            Q.qb = qb;
+            Q.staged = staged;
+        }
         if (staged) {
-            for (int e = tid; e < nk; e += kThreads) cp_async16(Q.buf + e, C.gkp + e);
-            for (int e = tid; e < 2 * nk; e += kThreads) cp_async16(Q.buf + nk + e, C.gdesc + e);
-            if (cells)
-                for (int c = tid; c < kCell16Bytes / 16; c += kThreads)
-                    cp_async16(Q.buf + 3 * nk + c, reinterpret_cast<const uint4 *>(C.cell16) + c);
+            auto stage = [&](unsigned char *dst, const void *src, int bytes) {
+                for (int c = 16 * tid; c < bytes; c += 16 * kThreads)
+                    cp_async16(dst + c, reinterpret_cast<const unsigned char *>(src) + c);
+            };
+            stage(buf, C.cell16, kCell16Bytes);
+            stage(buf + kCell16Bytes, C.gq, qb);
+            stage(buf + kCell16Bytes + qb, C.gk16, kb);
             asm volatile("cp.async.wait_all;" ::: "memory");
         }
         __syncthreads();
         mark(B, 0);
-        if (split) {
-            // first halves (the staged records' right coordinates are not
-            // read: they may not be final yet), then the stereo step, then
-            // the second halves; each thread finishes the points it scanned
-            if (staged) {
-                for (int m = m0 + tid; m < m1; m += kThreads)
-                    search_point<true, true>(B.p, F, C, Q, scell, iw, ih, m, motion);
-            } else {
-                for (int m = m0 + tid; m < m1; m += kThreads)
-                    search_point<false, true>(B.p, F, C, Q, nullptr, iw, ih, m, motion);
-            }
+        // a split search runs its first halves (the right coordinates are not
+        // read: they may not be final yet), then waits for the stereo step,
+        // then runs the second halves; each thread finishes the points it
+        // scanned, whose records stay on chip when they fit behind the grid
+        uint4 *scan = used + 32 * (m1 - m0) <= kSearchBuf ? reinterpret_cast<uint4 *>(buf + used) : C.scan + 2 * (size_t)m0;
+        SearchPass pass = split ? kFirstHalf : kWhole;
+        for (;;) {
+            search_points(B.p, F, C, Q, scan, m0, m1, pass);
             mark(B, 1);
-            if (wait_geq(B, &F.ctr[C_STEREO_READY], 1u, s_flag)) {
-                for (int m = m0 + tid; m < m1; m += kThreads) finish_point(B.p, F, C, Q, iw, ih, m, motion);
-            } else {
+            if (pass != kFirstHalf) break;
+            if (!wait_geq(B, &F.ctr[C_STEREO_READY], 1u, s_flag)) {
                 search_abandon(C, m0, m1);
+                break;
             }
+            const bool left = finish_points(B.p, F, C, scan, m0, m1);
             mark(B, 2);
-        } else if (staged) {
-            for (int m = m0 + tid; m < m1; m += kThreads) search_point<true>(B.p, F, C, Q, scell, iw, ih, m, motion);
-            mark(B, 1);
-        } else {
-            for (int m = m0 + tid; m < m1; m += kThreads)
-                search_point<false>(B.p, F, C, Q, nullptr, iw, ih, m, motion);
-            mark(B, 1);
+            if (!__syncthreads_or(left)) break;
+            pass = kLeftOver;
         }
     } else {
         search_abandon(C, m0, m1);
@@ -1750,7 +1806,6 @@ __device__ __forceinline__ void copy_words(void *dst, const void *src, size_t by
 __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(const BatchHeader *__restrict__ hdr)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem &U = *reinterpret_cast<Smem *>(smem_raw);
     __shared__ int s_item;
     __shared__ int s_flag;
     // the launch header and the current frame's descriptor live in shared
@@ -1760,13 +1815,18 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(
     __shared__ __align__(16) FrameDev sF;
     copy_words(&sB, hdr, sizeof(BatchHeader));
     __syncthreads();
-    const BatchHeader &B = sB;
     for (;;) {
-        if (threadIdx.x == 0) s_item = (int)atomicAdd(B.queue, 1u);
+        if (threadIdx.x == 0) s_item = (int)atomicAdd(sB.queue, 1u);
         __syncthreads();
         const int item = s_item;
         __syncthreads();
-        if (item >= B.total_items) break;
+        if (item >= sB.total_items) break;
+        // zero (items are not negative), which the compiler does not know: the
+        // roles' addresses then depend on the item, and their arithmetic is not
+        // hoisted out of this loop, all roles' at once, and spilled
+        const unsigned zero = (unsigned)item >> 31;
+        const BatchHeader &B = *reinterpret_cast<const BatchHeader *>(reinterpret_cast<const char *>(&sB) + 16 * zero);
+        Smem &U = *reinterpret_cast<Smem *>(smem_raw + 16 * zero);
         int kind = 0;
         while (kind < K_KINDS - 1 && item >= B.kind_begin[kind + 1]) ++kind;
         const int local = item - B.kind_begin[kind];
@@ -1779,7 +1839,7 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(
         }
         copy_words(&sF, B.frames + lo, sizeof(FrameDev));
         __syncthreads();
-        const FrameDev &F = sF;
+        const FrameDev &F = *reinterpret_cast<const FrameDev *>(reinterpret_cast<const char *>(&sF) + 16 * zero);
         const int tile = local - pre[lo];
         unsigned long long t_start = 0;
         if (B.trace != nullptr && threadIdx.x == 0) {
