@@ -588,7 +588,6 @@ ft_status build_table(ft_ctx *ctx, const ft_params &params, const std::vector<Jo
             for (int i = 0; i < 3; ++i) F.last_t[i] = j.last_pose.t[i];
             F.base = j.camera == FT_CAMERA_PINHOLE ? j.pin.b : j.rig.b;
             F.search_tile = std::max(kThreads, tune.search_tile / kThreads * kThreads);
-            F.search_stage = tune.search_stage ? 1 : 0;
             F.resolve_tile = std::max(kThreads, tune.resolve_tile / kThreads * kThreads);
             for (int c = 0; c < F.ncam; ++c) {
                 CamDev &C = F.cam[c];
@@ -614,7 +613,6 @@ ft_status build_table(ft_ctx *ctx, const ft_params &params, const std::vector<Jo
                 fill_cam_kps(C, c ? j.right : j.left, c ? j.taken_r : j.taken_l);
                 fill_cam_out(C, c ? j.so.right : j.so.left);
                 C.cell_ptr = reinterpret_cast<int *>(carve(sizeof(int) * (kCells + 1)));
-                C.cell16 = reinterpret_cast<uint16_t *>(carve(sizeof(uint16_t) * (kCells + 1)));
                 C.gq = reinterpret_cast<unsigned *>(carve(sizeof(unsigned) * (size_t)C.nk));
                 if (C.nk < 65536) C.gk16 = reinterpret_cast<uint16_t *>(carve(sizeof(uint16_t) * (size_t)C.nk));
                 else C.gk32 = reinterpret_cast<int *>(carve(sizeof(int) * (size_t)C.nk));
@@ -1428,8 +1426,8 @@ ft_status ft_get_tuning(ft_ctx *ctx, const ft_batch *batch, ft_tuning *t)
 
 // The launch shapes both autotuners try: strip rows 16/32/64, search tile
 // 256/512/1024, fisheye tile 64/128, every count of CTAs per SM from the
-// resident maximum down to one (fewer leave room for a concurrent launch),
-// both search staging modes and the search in one pass or two halves.
+// resident maximum down to one (fewer leave room for a concurrent launch)
+// and the search in one pass or two halves.
 static std::vector<ft_tuning> tuning_candidates(int occ)
 {
     const int strips[] = {16, 32, 64};
@@ -1442,17 +1440,15 @@ static std::vector<ft_tuning> tuning_candidates(int occ)
         for (int b : tiles)
             for (int c : fish)
                 for (int o : occs)
-                    for (int st = 0; st < 2; ++st)
-                        for (int sp : {1, -1}) {
-                            ft_tuning t = default_tuning();
-                            t.strip_rows = a;
-                            t.search_tile = b;
-                            t.fisheye_tile = c;
-                            t.ctas_per_sm = o;
-                            t.search_stage = st;
-                            t.split_search = sp;
-                            cand.push_back(t);
-                        }
+                    for (int sp : {1, -1}) {
+                        ft_tuning t = default_tuning();
+                        t.strip_rows = a;
+                        t.search_tile = b;
+                        t.fisheye_tile = c;
+                        t.ctas_per_sm = o;
+                        t.split_search = sp;
+                        cand.push_back(t);
+                    }
     return cand;
 }
 

@@ -92,10 +92,9 @@ struct CamDev {
     int *mp_kp, *mp_d1, *mp_d2, *kp_mp;
     // the keypoint grid (scratch), in cell order; keypoints already taken
     // are left out
-    int *cell_ptr;                 // [kCells + 1] cell starts
-    uint16_t *cell16;              // [kCells + 1] the same starts in 16 bits (nk < 65536), 16-byte aligned
+    int *cell_ptr;                 // [kCells + 1] cell starts, 16-byte aligned
     unsigned *gq;                  // [nk] packed place and octave of each placed keypoint (see pack_place)
-    uint16_t *gk16;                // [nk] its index (nk < 65536)
+    uint16_t *gk16;                // [nk] its index (nk < 65536, else NULL); this and gq in whole 16-byte chunks
     int *gk32;                     // [nk] its index (nk >= 65536, else NULL)
     unsigned long long *owner;     // [nk] (distance << 32) | map index
     uint4 *scan;                   // [2 * nm] split search: per map point its four smallest candidate keys,
@@ -144,7 +143,6 @@ struct FrameDev {
     // work decomposition
     int strip_rows, n_stereo_items, fisheye_tile;
     int search_tile, resolve_tile;
-    int search_stage;              // 0: stage the camera's records on chip when they fit; 1: read from L2
     int rowsort;                   // row-sort index items (kRowSortItems: the first half the left
                                    // keypoints, the second half the right ones), 0 without stereo
     int fold_resolve;              // 1: the last search item of a camera writes the final tables

@@ -246,11 +246,10 @@ struct SmemMedian {
 };
 
 constexpr int kCell16Bytes = (2 * (kCells + 1) + 15) / 16 * 16;   // 16-bit cell starts, whole chunks
-constexpr int kPool = 128;                      // candidates a warp collects before it compares them
-constexpr int kStep = 2;                        // candidates a lane tests per step
-constexpr int kPoolFull = kPool - 2 - 32 * kStep;   // collected candidates beyond which another step might not fit
-constexpr unsigned kPoolEnd = 127u;             // end of a point's chain of candidates
-constexpr int kSearchBuf = 64 * 1024;           // bytes for the staged grid and the split search's records
+constexpr int kStep = 4;                        // candidates a lane tests per step
+constexpr int kList = 8;                        // candidates a lane collects before its warp compares them
+constexpr int kSearchBuf = 56 * 1024;           // bytes for the staged grid and the split search's records
+constexpr int kGridStage = (kSearchBuf - kCell16Bytes) / 6 / 8 * 8;   // keypoints of a camera's grid on chip at a time
 
 // Where a keypoint lies, for the search's first test: x and y over the grid's
 // span (one cell more at each side, so that every placed keypoint is inside)
@@ -259,19 +258,17 @@ struct PlaceScale {
     float x0, y0, sx, sy;
 };
 
-// what a search item keeps on chip: the camera's pose, each warp's candidate
-// pool with the compared keys, then (buf) the staged grid (16-bit cell
-// starts, packed places, 16-bit indices) and, in a split search, its points'
-// records
+// what a search item keeps on chip: the camera's pose, each warp's
+// candidates, then (buf) the staged part of the grid (cell starts, packed
+// places, indices) and, in a split search, its points' records
 struct SmemSearch {
     float pose[12];
     PlaceScale ps;
     float iw, ih;                   // grid cells per pixel
     int motion;                     // of a last-frame search (f2)
-    int staged;                     // the grid lies in buf
-    int qb;                         // bytes of the staged packed places
-    unsigned pool[kWarps][kPool];
-    unsigned key[kWarps][kPool];
+    int e0, wide;                   // first staged keypoint of the grid; its indices are left in device memory
+    unsigned list[kWarps][kList][32];   // candidates by lane, then the warp's pool of them
+    unsigned pool[kWarps][kList * 32];
     uint4 buf[kSearchBuf / 16];
 };
 
@@ -440,14 +437,8 @@ __device__ void grid_item(const BatchHeader &B, const FrameDev &F, int cam, Smem
     __syncthreads();
     mark(B, 0);
     const int total = block_scan(G.cnt, G.cnt, kCells, G.warp_sums);
-    for (int c = tid; c < kCells; c += kThreads) {
-        C.cell_ptr[c] = G.cnt[c];
-        C.cell16[c] = (uint16_t)G.cnt[c];      // read only for frames of fewer than 65536 keypoints
-    }
-    if (tid == 0) {
-        C.cell_ptr[kCells] = total;
-        C.cell16[kCells] = (uint16_t)total;
-    }
+    for (int c = tid; c < kCells; c += kThreads) C.cell_ptr[c] = G.cnt[c];
+    if (tid == 0) C.cell_ptr[kCells] = total;
     __syncthreads();
     mark(B, 1);
     pass(true);
@@ -1347,12 +1338,14 @@ __device__ __forceinline__ PointWindow point_window(const DevParams &P, const Fr
     W.lo = W.hi = W.octs = 0u;
     const bool last = F.search_mode != 0;
     const int loct = last ? (int)__ldg(F.last_oct + m) : 0;
-    if ((F.skip != nullptr && __ldg(F.skip + m) != 0) || (last && (loct < 0 || loct >= P.nlevels))) return W;
+    const bool skipped = F.skip != nullptr && __ldg(F.skip + m) != 0;
     const float4 pos = __ldg(F.pos + m);
+    const float4 nrm = last ? pos : __ldg(F.nrm + m);
+    if (skipped || (last && (loct < 0 || loct >= P.nlevels))) return W;
     float u, v, ur, vc = 0.0f;
     int level = loct;
     const bool in_view = last ? project_uv(C, pose, pos, u, v, ur)
-                              : project(P, C, pose, pos, __ldg(F.nrm + m), u, v, ur, vc, level);
+                              : project(P, C, pose, pos, nrm, u, v, ur, vc, level);
     if (!in_view) return W;
     W.level = level;
     W.u = u;
@@ -1387,104 +1380,138 @@ __device__ __forceinline__ PointWindow point_window(const DevParams &P, const Fr
     return W;
 }
 
-// The grid as a search item reads it: staged in shared memory, or in device
-// memory.
-__device__ __forceinline__ int grid_start(const CamDev &C, const SmemSearch &Q, int c)
+// The staged part of the grid: keypoints [e0, e0 + kGridStage) in cell order,
+// which is all of them for a camera of up to kGridStage keypoints (8528);
+// cell starts are relative to e0 and clamped to the part.
+__device__ __forceinline__ int grid_start(const SmemSearch &Q, int c)
 {
-    return Q.staged ? (int)reinterpret_cast<const uint16_t *>(Q.buf)[c] : __ldcg(C.cell_ptr + c);
+    return (int)reinterpret_cast<const uint16_t *>(Q.buf)[c];
 }
-__device__ __forceinline__ unsigned grid_place(const CamDev &C, const SmemSearch &Q, int e)
+__device__ __forceinline__ const unsigned *grid_places(const SmemSearch &Q)
 {
-    return Q.staged ? reinterpret_cast<const unsigned *>(Q.buf)[kCell16Bytes / 4 + e] : __ldcg(C.gq + e);
+    return reinterpret_cast<const unsigned *>(Q.buf) + kCell16Bytes / 4;
 }
-__device__ __forceinline__ int grid_index(const CamDev &C, const SmemSearch &Q, int e)
+__device__ __forceinline__ int grid_index(const CamDev &C, const SmemSearch &Q, int n, int e)
 {
-    if (Q.staged)
-        return (int)*reinterpret_cast<const uint16_t *>(reinterpret_cast<const unsigned char *>(Q.buf) + kCell16Bytes +
-                                                        Q.qb + 2 * e);
-    return C.gk32 ? __ldcg(C.gk32 + e) : (int)__ldcg(C.gk16 + e);
+    if (Q.wide) return __ldcg(C.gk32 + Q.e0 + e);
+    return (int)reinterpret_cast<const uint16_t *>(grid_places(Q) + n)[e];
+}
+
+// entries of a staged part, rounded up to whole 16-byte chunks of indices
+__device__ __forceinline__ int grid_part(const CamDev &C) { return min((C.nk + 7) & ~7, kGridStage); }
+
+// Copies part `part` of a camera's grid on chip (the caller synchronizes).
+// Every chunk read lies inside the arrays, whose sizes are whole chunks.
+__device__ void stage_grid(const CamDev &C, SmemSearch &Q, int part)
+{
+    const int tid = threadIdx.x;
+    const int e0 = part * kGridStage, n = grid_part(C);
+    const int have = min(n, ((C.nk + 7) & ~7) - e0);         // entries of this part
+    unsigned char *buf = reinterpret_cast<unsigned char *>(Q.buf);
+    auto copy = [&](unsigned char *dst, const void *src, int bytes) {
+        for (int c = 16 * tid; c < bytes; c += 16 * kThreads)
+            cp_async16(dst + c, reinterpret_cast<const unsigned char *>(src) + c);
+    };
+    copy(buf + kCell16Bytes, C.gq + e0, 4 * have);
+    if (C.gk16) copy(buf + kCell16Bytes + 4 * n, C.gk16 + e0, 2 * have);
+    uint16_t *start = reinterpret_cast<uint16_t *>(buf);
+    for (int c = 4 * tid; c < kCells; c += 4 * kThreads) {
+        const int4 v = __ldcg(reinterpret_cast<const int4 *>(C.cell_ptr + c));
+        const unsigned a = (unsigned)clampi(v.x - e0, 0, n) | (unsigned)clampi(v.y - e0, 0, n) << 16;
+        const unsigned b = (unsigned)clampi(v.z - e0, 0, n) | (unsigned)clampi(v.w - e0, 0, n) << 16;
+        *reinterpret_cast<uint2 *>(start + c) = make_uint2(a, b);
+    }
+    if (tid == 0) {
+        start[kCells] = (uint16_t)clampi(__ldcg(C.cell_ptr + kCells) - e0, 0, n);
+        Q.e0 = e0;
+        Q.wide = C.gk16 == nullptr;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // A warp's 32 map points (point mw + lane in lane `lane`) against the
 // keypoints of their windows.  Each lane walks the cell rows of its own point
 // and applies the first test (packed place and octave: one shared-memory
-// word a candidate, 19 in 20 of which fail); what passes goes to the warp's
-// pool.  The pool's candidates are then shared out over the lanes, whichever
+// word a candidate, four in flight; 19 in 20 fail), listing what passes.  The
+// warp's listed candidates are then shared out over its lanes, whichever
 // point they belong to, and get the exact tests and the Hamming distance
 // from the frame's own arrays, all their loads in flight at once; then each
-// lane takes its own point's keys (distance << 20 | keypoint) from its chain
-// in the pool and keeps the four smallest and their number.  What bounds it
-// is latency: a point has one or two candidates behind the first test, so
-// comparing them lane by lane as they are found leaves most lanes idle and
-// pays a round trip for each (1280x720, 4000 keypoints, 20000 points: 13 us
-// a point and thread that way).
+// lane takes its own point's keys (distance << 20 | keypoint) and keeps the
+// four smallest and their number.  What bounds it is latency: a point has one
+// or two candidates behind the first test, so comparing them lane by lane as
+// they are found leaves most lanes idle and pays a round trip for each
+// (1280x720, 4000 keypoints, 20000 points: 13 us a point and thread that
+// way; 7 us with the candidates voted into the pool one step at a time).
 // check_ur: the stereo consistency is among the tests (the first half of a
 // search split around the stereo step leaves it out).
 __device__ __forceinline__ void gather(const FrameDev &F, const CamDev &C, SmemSearch &Q, const PointWindow &W, int mw,
                                        bool check_ur, unsigned (&sk)[4], unsigned &count)
 {
     const int lane = threadIdx.x & 31;
-    unsigned *const pool = Q.pool[threadIdx.x >> 5], *const pkey = Q.key[threadIdx.x >> 5];
+    unsigned *const list = &Q.list[threadIdx.x >> 5][0][lane], *const pool = Q.pool[threadIdx.x >> 5];
+    const unsigned *const places = grid_places(Q);
+    const int part = grid_part(C);
     bool active = W.active;
     int cy = W.y0, e = 0, e1 = 0;
     if (active) {
-        e = grid_start(C, Q, cy * FT_GRID_COLS + W.x0);
-        e1 = grid_start(C, Q, cy * FT_GRID_COLS + W.x1 + 1);
+        e = grid_start(Q, cy * FT_GRID_COLS + W.x0);
+        e1 = grid_start(Q, cy * FT_GRID_COLS + W.x1 + 1);
     }
-    unsigned head = kPoolEnd;
-    int n = 0;                          // candidates in the pool (the same in every lane)
-    for (;;) {
-        if (active && e >= e1) {
-            if (cy < W.y1) {
-                ++cy;
-                e = grid_start(C, Q, cy * FT_GRID_COLS + W.x0);
-                e1 = grid_start(C, Q, cy * FT_GRID_COLS + W.x1 + 1);
-            } else {
-                active = false;
+    do {
+        int n = 0;
+        while (active && n <= kList - kStep) {
+            if (e >= e1) {
+                if (cy < W.y1) {
+                    ++cy;
+                    e = grid_start(Q, cy * FT_GRID_COLS + W.x0);
+                    e1 = grid_start(Q, cy * FT_GRID_COLS + W.x1 + 1);
+                } else {
+                    active = false;
+                }
             }
-        }
-        unsigned w[kStep];
+            unsigned w[kStep];
 #pragma unroll
-        for (int s = 0; s < kStep; ++s) w[s] = active && e + s < e1 ? grid_place(C, Q, e + s) : 0u;
+            for (int s = 0; s < kStep; ++s) w[s] = e + s < e1 ? places[e + s] : 0u;
 #pragma unroll
-        for (int s = 0; s < kStep; ++s) {
-            const unsigned place = w[s] & 0x0fff3fffu;
-            const bool pass = active && e + s < e1 && __vminu2(__vmaxu2(place, W.lo), W.hi) == place &&
-                              ((W.octs >> (w[s] >> 28)) & 1u);
-            const unsigned hit = __ballot_sync(kFull, pass);
-            if (pass) {
-                const unsigned slot = (unsigned)(n + __popc(hit & ((1u << lane) - 1u)));
-                pool[slot] = (unsigned)(e + s) | ((unsigned)lane << 20) | (head << 25);
-                head = slot;
+            for (int s = 0; s < kStep; ++s) {
+                const unsigned place = w[s] & 0x0fff3fffu;
+                const bool pass = e + s < e1 & __vminu2(__vmaxu2(place, W.lo), W.hi) == place &
+                                  ((W.octs >> (w[s] >> 28)) & 1u);
+                list[32 * n] = (unsigned)(e + s) | ((unsigned)lane << 20);   // kept if it passes
+                n += pass;
             }
-            n += __popc(hit);
+            e += kStep;
         }
-        e += kStep;
-        const bool more = __any_sync(kFull, active);
-        if (more && n <= kPoolFull) continue;
         __syncwarp();
-        for (int p = lane; p - lane < n; p += 32) {
-            const bool have = p < n;
+        int end = n;                    // of this lane's candidates in the pool
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int t = __shfl_up_sync(kFull, end, d);
+            if (lane >= d) end += t;
+        }
+        const int total = __shfl_sync(kFull, end, 31);
+        for (int i = 0; i < n; ++i) pool[end - n + i] = list[32 * i];
+        __syncwarp();
+        for (int p = lane; p - lane < total; p += 32) {
+            const bool have = p < total;
             const unsigned ent = have ? pool[p] : 0u;
-            const int o = (int)((ent >> 20) & 31u);
+            const int o = (int)(ent >> 20);
             const float uo = __shfl_sync(kFull, W.u, o), vo = __shfl_sync(kFull, W.v, o);
             const float ro = __shfl_sync(kFull, W.r, o), uro = __shfl_sync(kFull, W.ur, o);
             if (!have) continue;
-            const int k = grid_index(C, Q, (int)(ent & 0xfffffu));
+            const int k = grid_index(C, Q, part, (int)(ent & 0xfffffu));
             const float x = __ldg(C.kx + k), y = __ldg(C.ky + k);
             const float w1 = check_ur ? __ldcg(F.u_right_in + k) : -1.0f;
             const uint4 b0 = __ldg(C.kdesc + 2 * k), b1 = __ldg(C.kdesc + 2 * k + 1);
             const uint4 q0 = __ldg(F.mdesc + 2 * (size_t)(mw + o)), q1 = __ldg(F.mdesc + 2 * (size_t)(mw + o) + 1);
             bool ok = fabsf(fsub(x, uo)) < ro && fabsf(fsub(y, vo)) < ro;
             if (w1 > 0.0f && fabsf(fsub(uro, w1)) > ro) ok = false;
-            pkey[p] = ok ? ((unsigned)ham8(q0, q1, b0, b1) << 20) | (unsigned)k : kNoKey;
+            pool[p] = ok ? ((unsigned)ham8(q0, q1, b0, b1) << 20) | (unsigned)k : kNoKey;
         }
         __syncwarp();
-        while (head != kPoolEnd) {
-            unsigned key = pkey[head];
-            head = pool[head] >> 25;
-            if (key == kNoKey) continue;
-            ++count;
+        for (int p = end - n; p < end; ++p) {
+            unsigned key = pool[p];
+            count += key != kNoKey;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const unsigned lo = min(sk[q], key);
@@ -1492,10 +1519,7 @@ __device__ __forceinline__ void gather(const FrameDev &F, const CamDev &C, SmemS
                 sk[q] = lo;
             }
         }
-        __syncwarp();
-        n = 0;
-        if (!more) break;
-    }
+    } while (__any_sync(kFull, active));
 }
 
 // The top-2 rules (threshold, ratio test) on a point's two smallest keys, the
@@ -1539,8 +1563,12 @@ __device__ __forceinline__ void search_points(const DevParams &P, const FrameDev
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool check_ur = pass != kFirstHalf && C.model == FT_CAMERA_PINHOLE && F.u_right_in != nullptr;
-    for (int mw = m0 + 32 * warp; mw < m1; mw += kThreads) {
-        const int m = mw + lane;
+    // a grid of several parts is staged part by part for every 256 points (all
+    // warps take part in each)
+    const int parts = (C.nk + kGridStage - 1) / kGridStage;
+    for (int mb = m0; mb < m1; mb += kThreads) {
+        const int mw = mb + 32 * warp, m = mw + lane;
+        if (parts <= 1 && mw >= m1) break;
         const bool mine = m < m1 && (pass != kLeftOver || scan[2 * (m - m0) + 1].w != 0u);
         PointWindow W;
         W.active = false;
@@ -1550,8 +1578,15 @@ __device__ __forceinline__ void search_points(const DevParams &P, const FrameDev
             if (C.proj) C.proj[m] = make_float4(W.u, W.v, W.ur, W.vc);
         }
         unsigned sk[4] = {kNoKey, kNoKey, kNoKey, kNoKey}, count = 0;
-        __syncwarp();
-        gather(F, C, Q, W, mw, check_ur, sk, count);
+        for (int part = 0; part < parts; ++part) {
+            if (parts > 1) {
+                __syncthreads();
+                stage_grid(C, Q, part);
+                __syncthreads();
+            }
+            __syncwarp();
+            gather(F, C, Q, W, mw, check_ur, sk, count);
+        }
         if (!mine) continue;
         if (pass == kFirstHalf) {
             scan[2 * (m - m0)] = make_uint4(sk[0], sk[1], sk[2], sk[3]);
@@ -1679,35 +1714,16 @@ __device__ void search_item(const BatchHeader &B, const FrameDev &F, int tile, S
         SmemSearch &Q = U.q;
         const int tid = threadIdx.x;
         search_setup(F, cam, Q);
-        // the camera's grid on chip by asynchronous copies when it fits (6
-        // bytes a keypoint and the cell starts: up to about 9900 keypoints;
-        // the tails past the placed keypoints are copied but never read)
-        const int nk = C.nk;
-        const int qb = (4 * nk + 15) & ~15, kb = (2 * nk + 15) & ~15;
-        const bool staged = F.search_stage == 0 && nk < 65536 && kCell16Bytes + qb + kb <= kSearchBuf;
-        unsigned char *buf = reinterpret_cast<unsigned char *>(Q.buf);
-        const int used = staged ? kCell16Bytes + qb + kb : 0;
-        if (tid == 0) {
-            Q.qb = qb;
-            Q.staged = staged;
-        }
-        if (staged) {
-            auto stage = [&](unsigned char *dst, const void *src, int bytes) {
-                for (int c = 16 * tid; c < bytes; c += 16 * kThreads)
-                    cp_async16(dst + c, reinterpret_cast<const unsigned char *>(src) + c);
-            };
-            stage(buf, C.cell16, kCell16Bytes);
-            stage(buf + kCell16Bytes, C.gq, qb);
-            stage(buf + kCell16Bytes + qb, C.gk16, kb);
-            asm volatile("cp.async.wait_all;" ::: "memory");
-        }
+        if (C.nk <= kGridStage) stage_grid(C, Q, 0);
         __syncthreads();
         mark(B, 0);
         // a split search runs its first halves (the right coordinates are not
         // read: they may not be final yet), then waits for the stereo step,
         // then runs the second halves; each thread finishes the points it
         // scanned, whose records stay on chip when they fit behind the grid
-        uint4 *scan = used + 32 * (m1 - m0) <= kSearchBuf ? reinterpret_cast<uint4 *>(buf + used) : C.scan + 2 * (size_t)m0;
+        const int used = kCell16Bytes + 6 * grid_part(C);
+        uint4 *scan = used + 32 * (m1 - m0) <= kSearchBuf ? reinterpret_cast<uint4 *>(reinterpret_cast<char *>(Q.buf) + used)
+                                                          : C.scan + 2 * (size_t)m0;
         SearchPass pass = split ? kFirstHalf : kWhole;
         for (;;) {
             search_points(B.p, F, C, Q, scan, m0, m1, pass);
