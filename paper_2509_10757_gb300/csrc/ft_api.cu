@@ -785,7 +785,7 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         pyr_blocks = most;
     }
     // frames that optimize their pose run the pose kernel after the fused
-    // kernel, one block per frame up to the last such frame
+    // kernel, one cluster per frame up to the last such frame
     int pose_frames = 0;
     for (size_t f = 0; f < jobs.size(); ++f)
         if (jobs[f].do_pose) pose_frames = (int)f + 1;

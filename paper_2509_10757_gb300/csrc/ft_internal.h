@@ -151,7 +151,7 @@ struct FrameDev {
     int n_grid_items, n_index_items, n_search_items[2], n_resolve_items[2];
     unsigned *ctr;                 // [kCounters]
     // pose optimization (next row f4): the pose kernel, launched after the
-    // fused kernel, takes one block per frame with do_pose (pinhole frames)
+    // fused kernel, takes one cluster per frame with do_pose (pinhole frames)
     int do_pose;
     const int *po_mp_kp;           // [nm] matches: map point -> keypoint (cam[0])
     float *po_Rt;                  // [12] out: R row-major, t
@@ -219,7 +219,7 @@ struct OrbHeader {
 // Launch helpers implemented in ft_kernels.cu (host-callable).
 namespace ft {
 cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stream);
-// pose optimization of the frames with do_pose (one block per frame of the
+// pose optimization of the frames with do_pose (one cluster per frame of the
 // first nframes; after the fused kernel on the same stream)
 cudaError_t launch_pose(const BatchHeader *dev_hdr, int nframes, cudaStream_t stream);
 // levels 1.. of the pyramids of the frames that build them (before the fused
