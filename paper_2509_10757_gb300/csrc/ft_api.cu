@@ -56,6 +56,8 @@ int next_pow2(int v)
     return p;
 }
 
+int next_pow2_or_zero(int v) { return v > 0 ? next_pow2(v) : 0; }
+
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 struct TableLayout {
@@ -157,8 +159,8 @@ struct ft_ctx {
     bool use_graphs = false;
     cudaStream_t capture_stream = nullptr;
     // graphs by (bucket frames, CTAs/SM, slot, pyramid frames, pyramid
-    // blocks per image, pyramid levels, pose frames)
-    std::map<std::tuple<int, int, int, int, int, int, int>, cudaGraphExec_t> graphs;
+    // blocks per image, pyramid levels, pose frames, fisheye blocks per frame)
+    std::map<std::tuple<int, int, int, int, int, int, int, int>, cudaGraphExec_t> graphs;
     std::map<Bucket, ft_tuning> tuning;
     uint64_t launches = 0;
     unsigned debug_flags = 0;
@@ -567,8 +569,6 @@ ft_status build_table(ft_ctx *ctx, const ft_params &params, const std::vector<Jo
                 F.fd2 = j.fo.d2;
                 F.fdepth = j.fo.depth;
                 F.fxyz = reinterpret_cast<float4 *>(j.fo.depth ? j.fo.xyz : nullptr);
-                F.fisheye_tile = tune.fisheye_tile >= kFishTileMax ? kFishTileMax : kFishTileMax / 2;
-                n_stereo = (F.nl + F.fisheye_tile - 1) / F.fisheye_tile;
             }
         }
         F.n_stereo_items = n_stereo;
@@ -702,10 +702,10 @@ ft_status finish_call(ft_ctx *ctx, cudaStream_t s)
 
 ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int slot, int grid,
                     size_t copy_bytes, int pyr_frames, int pyr_blocks, int pyr_levels, int pose_frames,
-                    cudaGraphExec_t *out)
+                    int fish_blocks, cudaGraphExec_t *out)
 {
     // the pyramid launch's shared memory depends on the level count
-    const auto key = std::make_tuple(frames_p2, cps, slot, pyr_frames, pyr_blocks, pyr_levels, pose_frames);
+    const auto key = std::make_tuple(frames_p2, cps, slot, pyr_frames, pyr_blocks, pyr_levels, pose_frames, fish_blocks);
     auto it = ctx->graphs.find(key);
     if (it != ctx->graphs.end()) {
         *out = it->second;
@@ -718,8 +718,9 @@ ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int sl
     const cudaError_t e1 = cudaMemcpyAsync(table_dev, ctx->staging[slot], copy_bytes, cudaMemcpyHostToDevice, cs);
     const cudaError_t e0 =
         launch_pyramids(reinterpret_cast<const BatchHeader *>(table_dev), pyr_frames, pyr_levels, pyr_blocks, cs);
-    cudaError_t e2 = e0 != cudaSuccess ? e0 : launch_fused(reinterpret_cast<const BatchHeader *>(table_dev),
-                                                           grid, cs);
+    cudaError_t e2 = e0 != cudaSuccess ? e0 : launch_fisheye(reinterpret_cast<const BatchHeader *>(table_dev),
+                                                             frames_p2, fish_blocks, cs);
+    if (e2 == cudaSuccess) e2 = launch_fused(reinterpret_cast<const BatchHeader *>(table_dev), grid, cs);
     if (e2 == cudaSuccess) e2 = launch_pose(reinterpret_cast<const BatchHeader *>(table_dev), pose_frames, cs);
     const cudaError_t e3 = cudaStreamEndCapture(cs, &g);
     if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
@@ -784,19 +785,28 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
             }
         pyr_blocks = most;
     }
+    // fisheye frames run their stereo step in a kernel of its own, as many
+    // blocks per frame as the one with the most left keypoints needs (the
+    // blocks past a smaller frame's keypoints, and other frames', exit)
+    int fish_frames = 0, fish_blocks = 0;
+    for (size_t f = 0; f < jobs.size(); ++f) {
+        if (jobs[f].camera != FT_CAMERA_FISHEYE || !jobs[f].do_stereo || jobs[f].left.n == 0) continue;
+        fish_frames = (int)f + 1;
+        fish_blocks = std::max(fish_blocks, fisheye_blocks(jobs[f].left.n));
+    }
     // frames that optimize their pose run the pose kernel after the fused
     // kernel, one cluster per frame up to the last such frame
     int pose_frames = 0;
     for (size_t f = 0; f < jobs.size(); ++f)
         if (jobs[f].do_pose) pose_frames = (int)f + 1;
-    if (items > 0 || pyr_frames > 0 || pose_frames > 0) {
+    if (items > 0 || pyr_frames > 0 || pose_frames > 0 || fish_frames > 0) {
         if (allow_graph && ctx->use_graphs && items > 0) {
             const int fp2 = bk.frames_p2;
             const size_t copy = std::max(bytes, table_layout(fp2).total);
             cudaGraphExec_t exec = nullptr;
             if ((s = get_graph(ctx, table_dev, fp2, cps, slot, grid_max, std::min(copy, ctx->table_cap),
                                pyr_frames > 0 ? fp2 : 0, pyr_blocks, params.nlevels, pose_frames > 0 ? fp2 : 0,
-                               &exec)) != FT_OK)
+                               next_pow2_or_zero(fish_blocks), &exec)) != FT_OK)
                 return s;
             FT_CUDA(cudaGraphLaunch(exec, stream));
         } else {
@@ -805,13 +815,15 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
                 FT_CUDA(launch_pyramids(reinterpret_cast<const BatchHeader *>(table_dev), pyr_frames, params.nlevels,
                                         pyr_blocks,
                                         stream));
+            FT_CUDA(launch_fisheye(reinterpret_cast<const BatchHeader *>(table_dev), fish_frames, fish_blocks, stream));
             if (items > 0)
                 FT_CUDA(launch_fused(reinterpret_cast<const BatchHeader *>(table_dev), std::min(items, grid_max),
                                      stream));
             if (pose_frames > 0)
                 FT_CUDA(launch_pose(reinterpret_cast<const BatchHeader *>(table_dev), pose_frames, stream));
         }
-        ctx->launches += (items > 0 ? 1 : 0) + (pyr_frames > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0);
+        ctx->launches += (items > 0 ? 1 : 0) + (pyr_frames > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) +
+                         (fish_frames > 0 ? 1 : 0);
     }
     FT_CUDA(cudaEventRecord(ctx->slot_done[slot], stream));
     return finish_call(ctx, stream);
@@ -914,6 +926,7 @@ ft_status ft_create(ft_ctx **out, const ft_ctx_desc *desc)
     cudaError_t e = cudaGetDeviceProperties(&prop, d.device);
     if (e == cudaSuccess) e = fused_occupancy(&c->occ);
     if (e == cudaSuccess) e = pyramid_setup();
+    if (e == cudaSuccess) e = fisheye_setup();
     c->sm_count = prop.multiProcessorCount;
     if (c->occ < 1) c->occ = 1;
     // the table region holds a batch table of max_frames frames or an

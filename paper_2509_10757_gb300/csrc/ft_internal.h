@@ -26,9 +26,6 @@ constexpr int kStageCap = 512;                      // right keypoints staged pe
 constexpr int kMaxRows = 4096;                      // image rows the row sort handles
 constexpr int kWinRows = 192;                       // rows of a stereo item's staged window
 constexpr int kOctBuckets = 8;                      // octaves a staged window separates
-constexpr int kRefineChunk = 64;                    // matches refined per SAD round
-constexpr int kFishChunk = 512;                     // right descriptors staged per chunk
-constexpr int kFishTileMax = 128;                   // left keypoints per fisheye item, at most
 constexpr int kFoldResolveMax = 8192;               // frames up to this size resolve in their last search item
 constexpr int kCounters = 8;                        // per-frame counters (u32)
 constexpr int kRowSortItems = 4;                    // row-sort work items per pinhole frame (2 per side)
@@ -141,7 +138,7 @@ struct FrameDev {
     const uint4 *mdesc;
     const uint8_t *skip;
     // work decomposition
-    int strip_rows, n_stereo_items, fisheye_tile;
+    int strip_rows, n_stereo_items;
     int search_tile, resolve_tile;
     int rowsort;                   // row-sort index items (kRowSortItems: the first half the left
                                    // keypoints, the second half the right ones), 0 without stereo
@@ -226,6 +223,12 @@ cudaError_t launch_pose(const BatchHeader *dev_hdr, int nframes, cudaStream_t st
 // launch); blocks_per_image blocks stride over each image's virtual blocks
 cudaError_t launch_pyramids(const BatchHeader *dev_hdr, int nframes, int nlevels, int tiles_per_image,
                             cudaStream_t stream);
+// brute-force matching and triangulation of the fisheye frames among the first
+// nframes (any order with the fused kernel: neither reads the other's
+// outputs); blocks: of the frame with the most left keypoints
+cudaError_t launch_fisheye(const BatchHeader *dev_hdr, int nframes, int blocks, cudaStream_t stream);
+int fisheye_blocks(int nl);    // blocks of a frame of nl left keypoints
+cudaError_t fisheye_setup();   // the fisheye kernel's shared-memory attribute (once per context)
 cudaError_t pyramid_setup();   // the pyramid kernel's shared-memory attribute (once per context)
 int fused_smem_bytes();
 // device set-up of the fused and pose kernels (shared-memory attributes),

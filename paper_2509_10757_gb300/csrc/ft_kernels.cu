@@ -16,9 +16,8 @@
 //              centre-subtracted patches, then per match the best shift,
 //              parabola, disparity and depth (kernel 2 of section IV-C).  The
 //              frame's last strip runs the median rejection.
-//              fisheye: one tile of left keypoints, one thread each, against
-//              the right overlap descriptors staged in shared memory chunks;
-//              best/second best kept as packed (distance, index) keys.
+//              (Fisheye frames' brute force is a kernel of its own:
+//              ft_fisheye.cu.)
 //   K_SEARCH   one tile of map points, one thread each: frustum test, FP32
 //              projection, predicted level, grid-window gather, top-2 Hamming,
 //              ratio test; accepted claims go to an atomicMin per keypoint.
@@ -86,14 +85,6 @@ __device__ __forceinline__ unsigned long long global_ns()
 }
 
 __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? lo : (v > hi ? hi : v); }
-
-// Top-2 of packed (distance << 20 | index) keys: the smallest and the
-// smallest of the rest.
-__device__ __forceinline__ void top2_push(unsigned key, unsigned &best, unsigned &second)
-{
-    second = min(second, max(best, key));
-    best = min(best, key);
-}
 
 // atan2 for y >= 0, x >= 0, from the mathematics: atan2(y, x) = atan(y/x)
 // when y <= x, else pi/2 - atan(x/y); atan(t) = pi/4 + atan((t-1)/(t+1)) for
@@ -227,17 +218,6 @@ struct SmemGrid {
     int warp_sums[kWarps];
 };
 
-constexpr int kFishGroup = 4;                    // lanes sharing one left keypoint (each scans a quarter)
-constexpr int kFishSlots = kThreads / kFishGroup; // left keypoints per pass
-static_assert(kFishTileMax % kFishSlots == 0, "a fisheye item is a whole number of passes");
-
-struct SmemFish {
-    uint4 desc[2 * kFishChunk];
-    int idx[kFishChunk];
-    int act[kFishTileMax];   // the item's left keypoints inside the overlap
-    int count, nact;
-};
-
 constexpr int kMedianSmem = 8192;               // left keypoints whose SADs the median keeps on chip
 
 struct SmemMedian {
@@ -277,7 +257,6 @@ union Smem {
     SmemStereo s;
     SmemRows r;
     SmemGrid g;
-    SmemFish f;
     SmemMedian m;
     SmemSearch q;
 };
@@ -1011,229 +990,6 @@ __device__ void stereo_pinhole_item(const BatchHeader &B, const FrameDev &F, int
     }
 }
 
-// ---------------------------------------------------------------- f1: fisheye triangulation
-// sin and cos by their Taylor series (to t^13 and t^14; |t| <= 2 keeps the
-// remainder under 2e-8), Horner in t^2, every operation explicitly rounded
-__device__ __forceinline__ float sin_series(float t)
-{
-    const float t2 = fmul(t, t);
-    float s = 1.60590444e-10f;               //  1/13!
-    s = fadd(-2.50521079e-08f, fmul(t2, s)); // -1/11!
-    s = fadd(2.75573188e-06f, fmul(t2, s));  //  1/9!
-    s = fadd(-1.98412701e-04f, fmul(t2, s)); // -1/7!
-    s = fadd(8.33333377e-03f, fmul(t2, s));  //  1/5!
-    s = fadd(-1.66666672e-01f, fmul(t2, s)); // -1/3!
-    s = fadd(1.0f, fmul(t2, s));
-    return fmul(t, s);
-}
-
-__device__ __forceinline__ float cos_series(float t)
-{
-    const float t2 = fmul(t, t);
-    float c = -1.14707454e-11f;              // -1/14!
-    c = fadd(2.08767559e-09f, fmul(t2, c));  //  1/12!
-    c = fadd(-2.75573200e-07f, fmul(t2, c)); // -1/10!
-    c = fadd(2.48015876e-05f, fmul(t2, c));  //  1/8!
-    c = fadd(-1.38888892e-03f, fmul(t2, c)); // -1/6!
-    c = fadd(4.16666679e-02f, fmul(t2, c));  //  1/4!
-    c = fadd(-0.5f, fmul(t2, c));            // -1/2!
-    return fadd(1.0f, fmul(t2, c));
-}
-
-// Ray of a Kannala-Brandt pixel (kb = fx, fy, cx, cy, k1..k4): theta solves
-// theta * (1 + k1 t + k2 t^2 + k3 t^3 + k4 t^4) = |m| (t = theta^2) by
-// `iters` Newton steps from theta = |m|; false if the residual stays above
-// 2e-6 rad, the model no longer rises there, or theta leaves [0, 2].
-__device__ bool unproject_kb8(const float *kb, int iters, float u, float v, float *ray)
-{
-    const float mx = fdiv(fsub(u, kb[2]), kb[0]);
-    const float my = fdiv(fsub(v, kb[3]), kb[1]);
-    const float thd = fsqrt(fadd(fmul(mx, mx), fmul(my, my)));
-    if (thd == 0.0f) {
-        ray[0] = 0.0f;
-        ray[1] = 0.0f;
-        ray[2] = 1.0f;
-        return true;
-    }
-    float th = thd, f = 0.0f, dp = 1.0f;
-    for (int it = 0; it <= iters; ++it) {
-        const float t2 = fmul(th, th);
-        float poly = kb[7];
-        poly = fadd(kb[6], fmul(t2, poly));
-        poly = fadd(kb[5], fmul(t2, poly));
-        poly = fadd(kb[4], fmul(t2, poly));
-        poly = fadd(1.0f, fmul(t2, poly));
-        f = fsub(fmul(th, poly), thd);
-        dp = fmul(9.0f, kb[7]);
-        dp = fadd(fmul(7.0f, kb[6]), fmul(t2, dp));
-        dp = fadd(fmul(5.0f, kb[5]), fmul(t2, dp));
-        dp = fadd(fmul(3.0f, kb[4]), fmul(t2, dp));
-        dp = fadd(1.0f, fmul(t2, dp));
-        if (it == iters) break;             // the last pass only measures the residual
-        th = fsub(th, fdiv(f, dp));
-    }
-    if (!(fabsf(f) <= 2e-6f && dp > 0.0f && th >= 0.0f && th <= 2.0f)) return false;
-    const float sn = fdiv(sin_series(th), thd);
-    ray[0] = fmul(mx, sn);
-    ray[1] = fmul(my, sn);
-    ray[2] = cos_series(th);
-    return true;
-}
-
-__device__ __forceinline__ float dot3f(const float *a, const float *b)
-{
-    return fadd(fadd(fmul(a[0], b[0]), fmul(a[1], b[1])), fmul(a[2], b[2]));
-}
-
-__device__ __forceinline__ void cross3f(const float *a, const float *b, float *c)
-{
-    c[0] = fsub(fmul(a[1], b[2]), fmul(a[2], b[1]));
-    c[1] = fsub(fmul(a[2], b[0]), fmul(a[0], b[2]));
-    c[2] = fsub(fmul(a[0], b[1]), fmul(a[1], b[0]));
-}
-
-// Midpoint of the common perpendicular of the left ray l (from the left
-// centre) and the right ray r (right camera coordinates; X_r = R_rl X_l +
-// t_rl), in left-camera coordinates: with C = -R^T t, d = R^T r and
-// n = l x d, s = ((C x d).n)/(n.n), t = ((C x l).n)/(n.n).  Kept if the rays
-// are not parallel, both parameters are positive and the depth exceeds
-// min_depth.
-__device__ bool triangulate(const float *l, const float *r, const float *R, const float *t, float min_depth,
-                            float *X)
-{
-    float C[3], d[3], n[3], cd[3], cl[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        C[i] = -fadd(fadd(fmul(R[i], t[0]), fmul(R[3 + i], t[1])), fmul(R[6 + i], t[2]));
-        d[i] = fadd(fadd(fmul(R[i], r[0]), fmul(R[3 + i], r[1])), fmul(R[6 + i], r[2]));
-    }
-    cross3f(l, d, n);
-    const float nn = dot3f(n, n);
-    if (!(nn > fmul(1e-10f, fmul(dot3f(l, l), dot3f(d, d))))) return false;
-    cross3f(C, d, cd);
-    cross3f(C, l, cl);
-    const float s = fdiv(dot3f(cd, n), nn);
-    const float tt = fdiv(dot3f(cl, n), nn);
-    if (!(s > 0.0f && tt > 0.0f)) return false;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) X[i] = fmul(0.5f, fadd(fmul(s, l[i]), fadd(C[i], fmul(tt, d[i]))));
-    return X[2] > min_depth;
-}
-
-// f1 for left keypoint i with accepted right keypoint j (j < 0: none)
-__device__ void triangulate_match(const DevParams &P, const FrameDev &F, int i, int j)
-{
-    float X[3] = {0.0f, 0.0f, 0.0f}, rl[3], rr[3];
-    bool ok = false;
-    if (j >= 0 && unproject_kb8(F.kbl, P.kb_iters, __ldg(F.lx + i), __ldg(F.ly + i), rl) &&
-        unproject_kb8(F.kbr, P.kb_iters, __ldg(F.rx + j), __ldg(F.ry + j), rr))
-        ok = triangulate(rl, rr, F.R_rl, F.t_rl, P.min_depth, X);
-    F.fdepth[i] = ok ? X[2] : -1.0f;
-    if (F.fxyz) F.fxyz[i] = ok ? make_float4(X[0], X[1], X[2], 1.0f) : make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-// ---------------------------------------------------------------- K_STEREO, fisheye
-__device__ void stereo_fisheye_item(const BatchHeader &B, const FrameDev &F, int tile, Smem &U,
-                                    int *s_flag)
-{
-    // The item's left keypoints inside the overlap are compacted into a list;
-    // kFishGroup lanes share each one, lane g comparing it with the staged
-    // right overlap descriptors g, g + kFishGroup, ...; the lanes' top-2 keys
-    // (distance << 20 | right index, all distinct) merge by shuffles into the
-    // top-2 of the whole scan.
-    SmemFish &S = U.f;
-    const DevParams &P = B.p;
-    const int tid = threadIdx.x;
-    const int g = tid & (kFishGroup - 1), slot = tid / kFishGroup;
-    const int i0 = tile * F.fisheye_tile, i1 = min(F.nl, i0 + F.fisheye_tile);
-    if (tid == 0) S.nact = 0;
-    __syncthreads();
-    for (int i = i0 + tid; i < i1; i += kThreads) {
-        const float x = __ldg(F.lx + i);
-        if (x >= F.lap_l0 && x <= F.lap_l1) S.act[atomicAdd(&S.nact, 1)] = i;
-    }
-    __syncthreads();
-    const int nact = S.nact;
-    constexpr int Q = kFishTileMax / kFishSlots;    // passes: left keypoints per lane group
-    int idx[Q];
-    uint4 a0[Q], a1[Q];
-    unsigned best[Q], second[Q];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int a = q * kFishSlots + slot;
-        idx[q] = a < nact ? S.act[a] : -1;
-        best[q] = second[q] = kNoKey;
-        if (idx[q] >= 0) {
-            a0[q] = __ldg(F.ldesc + 2 * idx[q]);
-            a1[q] = __ldg(F.ldesc + 2 * idx[q] + 1);
-        }
-    }
-    if (nact > 0) {
-        for (int c0 = 0; c0 < F.nr; c0 += kFishChunk) {
-            if (tid == 0) S.count = 0;
-            __syncthreads();
-            const int c1 = min(F.nr, c0 + kFishChunk);
-            for (int j = c0 + tid; j < c1; j += kThreads) {
-                const float x = __ldg(F.rx + j);
-                if (x >= F.lap_r0 && x <= F.lap_r1) {
-                    const int pos = atomicAdd(&S.count, 1);
-                    S.idx[pos] = j;
-                    S.desc[2 * pos] = __ldg(F.rdesc + 2 * j);
-                    S.desc[2 * pos + 1] = __ldg(F.rdesc + 2 * j + 1);
-                }
-            }
-            __syncthreads();
-            const int cnt = S.count;
-            if (idx[0] >= 0) {
-                for (int e = g; e < cnt; e += kFishGroup) {
-                    const uint4 b0 = S.desc[2 * e], b1 = S.desc[2 * e + 1];
-                    const unsigned j = (unsigned)S.idx[e];
-#pragma unroll
-                    for (int q = 0; q < Q; ++q)
-                        if (idx[q] >= 0) top2_push(((unsigned)ham8(a0[q], a1[q], b0, b1) << 20) | j, best[q], second[q]);
-                }
-            }
-            __syncthreads();
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-#pragma unroll
-        for (int off = 1; off < kFishGroup; off <<= 1) {
-            const unsigned ob = __shfl_xor_sync(kFull, best[q], off), os = __shfl_xor_sync(kFull, second[q], off);
-            second[q] = min(min(second[q], os), max(best[q], ob));
-            best[q] = min(best[q], ob);
-        }
-        if (idx[q] >= 0 && g == 0) {
-            int r = -1, d2 = 256;
-            const int d1 = best[q] != kNoKey ? (int)(best[q] >> 20) : -1;
-            if (best[q] != kNoKey) {
-                d2 = second[q] != kNoKey ? (int)(second[q] >> 20) : 256;
-                if ((float)d1 < fmul(P.fisheye_ratio, (float)d2)) r = (int)(best[q] & 0xfffffu);
-            } else {
-                d2 = -1;
-            }
-            F.r_idx[idx[q]] = r;
-            F.fd1[idx[q]] = d1;
-            F.fd2[idx[q]] = d2;
-            if (F.fdepth) triangulate_match(P, F, idx[q], r);
-        }
-    }
-    // the item's keypoints outside the overlap: no match
-    for (int i = i0 + tid; i < i1; i += kThreads) {
-        const float x = __ldg(F.lx + i);
-        if (x >= F.lap_l0 && x <= F.lap_l1) continue;
-        F.r_idx[i] = -1;
-        F.fd1[i] = -1;
-        F.fd2[i] = -1;
-        if (F.fdepth) triangulate_match(P, F, i, -1);
-    }
-    if (signal_count(&F.ctr[C_STEREO_DONE], (unsigned)F.n_stereo_items, s_flag)) {
-        if (tid == 0 && !(B.debug_flags & kDebugWithholdStereoReady))
-            atomicExch(&F.ctr[C_STEREO_READY], 1u);
-    }
-}
-
 // ---------------------------------------------------------------- K_SEARCH
 __device__ void resolve_range(const CamDev &C, int nm, int i0, int i1);
 
@@ -1873,8 +1629,7 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(
             }
             break;
         case K_STEREO:
-            if (F.camera == FT_CAMERA_PINHOLE) stereo_pinhole_item(B, F, tile, U, &s_flag);
-            else stereo_fisheye_item(B, F, tile, U, &s_flag);
+            stereo_pinhole_item(B, F, tile, U, &s_flag);
             break;
         case K_SEARCH: search_item(B, F, tile, U, &s_flag); break;
         default: resolve_item(B, F, tile, &s_flag); break;
