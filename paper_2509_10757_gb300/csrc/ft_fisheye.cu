@@ -11,7 +11,9 @@
 // an item of 128 keypoints while three shared an SM).
 //
 // One block of 256 threads per 128 left keypoints of the overlap (compacted in
-// index order).  It expands their descriptors into shared memory once (128
+// index order), or a cluster of two or four that share the right keypoints
+// step by step where the blocks would not fill the chip (one frame of 1500
+// keypoints has eight).  It expands their descriptors into shared memory once (128
 // rows x 256 bytes, K-major, 128-byte swizzle), then takes the right overlap
 // keypoints 128 at a time: all threads expand the next 128 into one of two
 // buffers while the tensor core multiplies the other (eight tcgen05.mma of
@@ -36,9 +38,10 @@ constexpr int kFishRows = 128;          // left keypoints of a block (rows of th
 constexpr int kFishCols = 128;          // right keypoints of a step (columns)
 constexpr int kFishThreads = 256;
 constexpr int kFishWarps = kFishThreads / 32;
-constexpr int kFishWindow = 4096;       // keypoints scanned for the overlap at a time
+constexpr int kFishWindow = 2048;       // keypoints scanned for the overlap at a time
 constexpr int kFishRowBytes = 256;      // an expanded descriptor
 constexpr int kFishTile = kFishRows * kFishRowBytes;
+constexpr int kFishSplit = 4;           // blocks that share a row's columns, at most (a cluster)
 constexpr unsigned kTmemCols = 2 * kFishCols;
 static_assert(kFishRows == kFishCols, "both operands share the tile layout");
 static_assert(kFishThreads == 2 * kFishRows, "two threads expand a row, two warps read a row");
@@ -48,8 +51,9 @@ struct SmemFish {
     uint8_t b[2][kFishTile];                // right rows of this step and the next
     uint16_t list[kFishWindow];             // right overlap keypoints of the window, relative to its start
     int row[kFishRows];                     // left keypoint of each row
-    unsigned best[kFishRows], second[kFishRows];
+    unsigned best[2 * kFishSplit][kFishRows], second[2 * kFishSplit][kFishRows];  // by block of the cluster and half
     int count[kFishWarps];
+    float rig[28];                          // kb of both cameras, R_rl, t_rl
     unsigned long long mbar[2];
     unsigned tmem;
 };
@@ -121,7 +125,11 @@ __device__ bool unproject_kb8(const float *kb, int iters, float u, float v, floa
         dp = fadd(fmul(3.0f, kb[4]), fmul(t2, dp));
         dp = fadd(1.0f, fmul(t2, dp));
         if (it == iters) break;             // the last pass only measures the residual
-        th = fsub(th, fdiv(f, dp));
+        // a step that changes nothing leaves nothing to the later ones: the
+        // residual is that of this pass (about 4 steps instead of 10)
+        const float next = fsub(th, fdiv(f, dp));
+        if (next == th) break;
+        th = next;
     }
     if (!(fabsf(f) <= 2e-6f && dp > 0.0f && th >= 0.0f && th <= 2.0f)) return false;
     const float sn = fdiv(sin_series(th), thd);
@@ -171,14 +179,18 @@ __device__ bool triangulate(const float *l, const float *r, const float *R, cons
     return X[2] > min_depth;
 }
 
-// f1 for left keypoint i with accepted right keypoint j (j < 0: none)
-__device__ void triangulate_match(const DevParams &P, const FrameDev &F, int i, int j)
+// f1 for left keypoint i with accepted right keypoint j (j < 0: none); rig:
+// the left and right cameras' kb, R_rl, t_rl (on chip)
+__device__ void triangulate_match(const DevParams &P, const FrameDev &F, const float *rig, int i, int j)
 {
     float X[3] = {0.0f, 0.0f, 0.0f}, rl[3], rr[3];
     bool ok = false;
-    if (j >= 0 && unproject_kb8(F.kbl, P.kb_iters, __ldg(F.lx + i), __ldg(F.ly + i), rl) &&
-        unproject_kb8(F.kbr, P.kb_iters, __ldg(F.rx + j), __ldg(F.ry + j), rr))
-        ok = triangulate(rl, rr, F.R_rl, F.t_rl, P.min_depth, X);
+    if (j >= 0) {
+        const float ul = __ldg(F.lx + i), vl = __ldg(F.ly + i), ur = __ldg(F.rx + j), vr = __ldg(F.ry + j);
+        const bool left = unproject_kb8(rig, P.kb_iters, ul, vl, rl);
+        const bool right = unproject_kb8(rig + 8, P.kb_iters, ur, vr, rr);
+        if (left && right) ok = triangulate(rl, rr, rig + 16, rig + 25, P.min_depth, X);
+    }
     F.fdepth[i] = ok ? X[2] : -1.0f;
     if (F.fxyz) F.fxyz[i] = ok ? make_float4(X[0], X[1], X[2], 1.0f) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
@@ -310,6 +322,15 @@ __device__ __forceinline__ int compact(const float *xs, int j0, int n, float lo,
     return total;
 }
 
+// Stores v at this shared-memory location of the cluster's first block.
+__device__ __forceinline__ void store_first(unsigned *p, unsigned v)
+{
+    asm volatile("{\n\t.reg .u32 a;\n\tmapa.shared::cluster.u32 a, %0, 0;\n\t"
+                 "st.shared::cluster.u32 [a], %1;\n\t}" ::"r"(smem_addr(p)),
+                 "r"(v)
+                 : "memory");
+}
+
 __device__ __forceinline__ void top2_push(unsigned key, unsigned &best, unsigned &second)
 {
     second = min(second, max(best, key));
@@ -318,15 +339,18 @@ __device__ __forceinline__ void top2_push(unsigned key, unsigned &best, unsigned
 
 // The two smallest keys of 32 accumulator columns in each 16-bit lane (even
 // and odd columns): (256 - v) / 2 << 7 | column is 16384 - 64 v + column,
-// formed in the low mantissa bits of 2^23 + it (exact).
+// formed in the low mantissa bits of 2^23 + it (exact; the column is a
+// constant, so a key is one instruction).  n: columns that count, from col0 = 0.
 template <bool kAll>
-__device__ __forceinline__ void scan_columns(const unsigned (&v)[32], int col0, int n, unsigned &best, unsigned &second)
+__device__ __forceinline__ void scan_columns(const unsigned (&v)[32], const int col0, int n, unsigned &best,
+                                             unsigned &second)
 {
 #pragma unroll
     for (int i = 0; i < 32; i += 2) {
-        const float c = 8388608.0f + 16384.0f + (float)(col0 + i);
-        const unsigned k0 = __float_as_uint(__fmaf_rn(__uint_as_float(v[i]), -64.0f, c));
-        const unsigned k1 = __float_as_uint(__fmaf_rn(__uint_as_float(v[i + 1]), -64.0f, c + 1.0f));
+        const unsigned k0 =
+            __float_as_uint(__fmaf_rn(__uint_as_float(v[i]), -64.0f, 8388608.0f + 16384.0f + (float)(col0 + i)));
+        const unsigned k1 =
+            __float_as_uint(__fmaf_rn(__uint_as_float(v[i + 1]), -64.0f, 8388608.0f + 16384.0f + (float)(col0 + i + 1)));
         unsigned k = __byte_perm(k0, k1, 0x5410);
         if (!kAll) {
             if (col0 + i >= n) k |= 0xffffu;
@@ -351,16 +375,20 @@ __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const Batch
     const float *const rx = F.rx;
     const uint4 *const rdesc = F.rdesc;
     const float lap_r0 = F.lap_r0, lap_r1 = F.lap_r1;
+    const unsigned long long timeout_ns = hdr->timeout_ns;
+
+    if (tid < 28) S.rig[tid] = tid < 8 ? F.kbl[tid] : tid < 16 ? F.kbr[tid - 8] : tid < 25 ? F.R_rl[tid - 16] : F.t_rl[tid - 25];
+    const int split = (int)blockIdx.z, splits = (int)gridDim.z;     // of the cluster
 
     // this block's share of the left keypoints outside the overlap: no match
     const int i_out = tile * kFishRows + tid;
-    if (tid < kFishRows && i_out < nl) {
+    if (split == 0 && tid < kFishRows && i_out < nl) {
         const float x = __ldg(F.lx + i_out);
         if (!(x >= F.lap_l0 && x <= F.lap_l1)) {
             F.r_idx[i_out] = -1;
             F.fd1[i_out] = -1;
             F.fd2[i_out] = -1;
-            if (F.fdepth) triangulate_match(P, F, i_out, -1);
+            if (F.fdepth) triangulate_match(P, F, nullptr, i_out, -1);
         }
     }
     // the rows: left keypoints of the overlap with ranks [128 tile, 128 tile + 128)
@@ -373,7 +401,7 @@ __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const Batch
         });
     }
     const int rows = min(seen - tile * kFishRows, kFishRows);
-    if (rows <= 0) return;                          // the whole block
+    if (rows <= 0) return;                          // the whole cluster
 
     __syncwarp();
     if (warp == 0) {
@@ -405,68 +433,89 @@ __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const Batch
                                 [&](int rank, int e) { S.list[rank] = (uint16_t)e; });
         __syncthreads();
         const int steps = (cnt + kFishCols - 1) / kFishCols;
-        auto stage = [&](int s) {
-            const int c = s * kFishCols + er;
-            if (c < cnt) expand(S.b[s & 1], er, eh, __ldg(rdesc + 2 * (j0 + S.list[c]) + eh));
+        // this block's steps: split, split + splits, ...; its i-th uses buffers i & 1
+        const int mine = steps > split ? (steps - split + splits - 1) / splits : 0;
+        uint4 next = make_uint4(0, 0, 0, 0);        // what this thread expands next
+        auto fetch = [&](int i) {
+            const int c = (split + i * splits) * kFishCols + er;
+            if (i < mine && c < cnt) next = __ldg(rdesc + 2 * (j0 + S.list[c]) + eh);
+        };
+        auto stage = [&](int i) {
+            if ((split + i * splits) * kFishCols + er < cnt) expand(S.b[i & 1], er, eh, next);
             // the tensor core reads shared memory through the async proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-            __syncthreads();
+            ok = __syncthreads_and(ok);
+            if (!ok) return;
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                mma_step(tmem + (unsigned)(s & 1) * kFishCols, smem_addr(S.a), smem_addr(S.b[s & 1]),
-                         smem_addr(&S.mbar[s & 1]));
+                mma_step(tmem + (unsigned)(i & 1) * kFishCols, smem_addr(S.a), smem_addr(S.b[i & 1]),
+                         smem_addr(&S.mbar[i & 1]));
             }
+            fetch(i + 1);
         };
-        if (steps > 0) stage(0);
-        for (int s = 0; s < steps && ok; ++s) {
-            // the buffer of step s + 1 was read by step s - 1, whose product
-            // was waited for; its accumulators were read before stage()'s
-            // block-wide synchronization
-            if (s + 1 < steps) stage(s + 1);
-            ok = mbar_wait(smem_addr(&S.mbar[s & 1]), phase[s & 1], hdr->timeout_ns);
-            ok = __syncthreads_and(ok);
-            phase[s & 1] ^= 1u;
-            if (!ok) break;
+        fetch(0);
+        if (mine > 0) stage(0);
+        for (int i = 0; i < mine; ++i) {
+            // the buffer of step i + 1 was read by step i - 1, whose product
+            // every thread has waited for; its accumulators were read before
+            // stage()'s block-wide synchronization
+            if (i + 1 < mine) stage(i + 1);
+            if (!ok) break;                         // a wait ran out: known to the whole block
+            const int s = split + i * splits;
+            ok = __all_sync(kFull, mbar_wait(smem_addr(&S.mbar[i & 1]), phase[i & 1], timeout_ns));
+            phase[i & 1] ^= 1u;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            const int n = min(kFishCols, cnt - s * kFishCols);
+            const int n = cnt - s * kFishCols - 64 * half;       // of this warp's 64 columns
             unsigned b2 = 0xffffffffu, s2 = 0xffffffffu;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const int col0 = 64 * half + 32 * q;
-                if (col0 >= n) continue;                    // the same in the whole warp
+                if (32 * q >= n) continue;                  // the same in the whole warp
                 unsigned v[32];
-                tmem_load(v, tmem + lanes + (unsigned)(s & 1) * kFishCols + (unsigned)col0);
-                if (col0 + 32 <= n) scan_columns<true>(v, col0, n, b2, s2);
-                else scan_columns<false>(v, col0, n, b2, s2);
+                tmem_load(v, tmem + lanes + (unsigned)((i & 1) * kFishCols + 64 * half + 32 * q));
+                if (32 * q + 32 <= n) scan_columns<true>(v, 32 * q, n, b2, s2);
+                else scan_columns<false>(v, 32 * q, n, b2, s2);
             }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const unsigned k = ((q & 1) ? s2 : b2) >> (q & 2 ? 16 : 0) & 0xffffu;
-                if (k == 0xffffu) continue;
-                const unsigned j = (unsigned)(j0 + S.list[s * kFishCols + (int)(k & 127u)]);
-                top2_push((k >> 7) << 20 | j, best, second);
+            // the step's two smallest; right indices ascend, so one whose
+            // distance is not below the row's second cannot enter any more
+            const unsigned bl = b2 & 0xffffu, bh = b2 >> 16, sl = s2 & 0xffffu, sh = s2 >> 16;
+            const unsigned k1 = min(bl, bh), k2 = min(max(bl, bh), min(sl, sh));
+            if (k1 != 0xffffu && k1 >> 7 < second >> 20) {
+                const uint16_t *at = S.list + s * kFishCols + 64 * half;
+                top2_push((k1 >> 7) << 20 | (unsigned)(j0 + at[k1 & 127u]), best, second);
+                if (k2 != 0xffffu && k2 >> 7 < second >> 20)
+                    top2_push((k2 >> 7) << 20 | (unsigned)(j0 + at[k2 & 127u]), best, second);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         }
-        __syncthreads();                            // the list is read before the next window's
+        ok = __syncthreads_and(ok);                 // the list is read before the next window's
     }
-    if (!ok && tid == 0) atomicOr(hdr->status, kStatusTimeout);
-    // the two halves of a row's columns, then the match
+    if (!ok) {
+        if (tid == 0) atomicOr(hdr->status, kStatusTimeout);
+        best = second = kNoKey;
+    }
+    // the parts of a row's columns (two halves of every block's steps) meet in
+    // the cluster's first block, which then writes the match
     const int r = 32 * (warp & 3) + lane;
-    if (half == 1) {
-        S.best[r] = best;
-        S.second[r] = second;
+    if (splits == 1) {
+        S.best[half][r] = best;
+        S.second[half][r] = second;
+        __syncthreads();
+    } else {
+        store_first(&S.best[2 * split + half][r], best);
+        store_first(&S.second[2 * split + half][r], second);
+        __syncthreads();
+        asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     }
-    __syncthreads();
     __syncwarp();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
-    if (half == 0 && r < rows) {
-        const unsigned ob = S.best[r], os = S.second[r];
-        second = min(min(second, os), max(best, ob));
-        best = min(best, ob);
-        if (!ok) best = second = kNoKey;
+    if (split == 0 && half == 0 && r < rows) {
+        for (int p = 1; p < 2 * splits; ++p) {
+            const unsigned ob = S.best[p][r], os = S.second[p][r];
+            second = min(min(second, os), max(best, ob));
+            best = min(best, ob);
+        }
         const int i = S.row[r];
         int match = -1, d1 = -1, d2 = -1;
         if (best != kNoKey) {
@@ -477,7 +526,7 @@ __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const Batch
         F.r_idx[i] = match;
         F.fd1[i] = d1;
         F.fd2[i] = d2;
-        if (F.fdepth) triangulate_match(P, F, i, match);
+        if (F.fdepth) triangulate_match(P, F, S.rig, i, match);
     }
 }
 
@@ -493,8 +542,23 @@ int fisheye_blocks(int nl) { return (nl + kFishRows - 1) / kFishRows; }
 cudaError_t launch_fisheye(const BatchHeader *dev_hdr, int nframes, int blocks, cudaStream_t stream)
 {
     if (nframes <= 0 || blocks <= 0) return cudaSuccess;
-    ft_fisheye_kernel<<<dim3((unsigned)blocks, (unsigned)nframes), kFishThreads, kFishSmem, stream>>>(dev_hdr);
-    return cudaGetLastError();
+    // columns are shared out while that still leaves the chip's 152 SMs a
+    // block each (about 60 % of a frame's blocks have rows: the overlap)
+    int splits = 1;
+    while (splits < kFishSplit && 2 * splits * blocks * nframes <= 256) splits *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, (unsigned)nframes, (unsigned)splits);
+    cfg.blockDim = dim3(kFishThreads);
+    cfg.dynamicSmemBytes = kFishSmem;
+    cfg.stream = stream;
+    cudaLaunchAttribute cluster;
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = 1;
+    cluster.val.clusterDim.y = 1;
+    cluster.val.clusterDim.z = (unsigned)splits;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, ft_fisheye_kernel, dev_hdr);
 }
 
 }  // namespace ft
