@@ -1208,13 +1208,16 @@ ft_status ft_extract_orb(ft_ctx *ctx, void *stream, const ft_params *params, int
             // suppressed corners are never 8-neighbours: at most one per 2 x 2 block
             L.cand_cap = ((L.w + 1) / 2) * ((L.h + 1) / 2);
             L.cand = reinterpret_cast<unsigned *>(carve(sizeof(unsigned) * (size_t)L.cand_cap));
-            L.tiles_x = (L.w + kOrbTile - 1) / kOrbTile;
+            L.tiles_x = (L.w + kOrbTileW - 1) / kOrbTileW;
             L.tile0 = tiles;
-            tiles += L.tiles_x * ((L.h + kOrbTile - 1) / kOrbTile);
+            I.tile0[l] = tiles;
+            L.tiles_x_inv = L.tiles_x > 1 ? (unsigned)((0x100000000ull + (unsigned)L.tiles_x - 1) / (unsigned)L.tiles_x) : 0;
+            tiles += L.tiles_x * ((L.h + kOrbTileH - 1) / kOrbTileH);
             L.slot0 = slot0;
             L.max_kp = orb->max_kp[l];
             slot0 += L.max_kp;
         }
+        for (int l = p.nlevels; l < FT_MAX_LEVELS; ++l) I.tile0[l] = 0x7fffffff;
         I.tiles = tiles;
         I.nslots = nslots;
         I.x = o.x;

@@ -173,7 +173,8 @@ struct BatchHeader {
 };
 
 // ---------------------------------------------------------------- f3: keypoint extraction
-constexpr int kOrbTile = 32;            // detection tile: 32 x 32 pixels, 4 per thread
+constexpr int kOrbTileW = 62;           // detection tile: with its suppression ring 64 x 32 pixels
+constexpr int kOrbTileH = 30;
 constexpr int kOrbHalo = 4;             // FAST circle (3) + suppression neighbours (1)
 constexpr int kOrbMaxDim = 4096;        // level sizes the 12-bit key coordinates allow
 constexpr int kOrbMaxSlots = 4096;      // slots per level (sorted in shared memory)
@@ -188,10 +189,12 @@ struct OrbLevel {
     unsigned *cand;                     // [cand_cap] suppressed corners as keys (scratch)
     int cand_cap;
     int tiles_x, tile0;                 // tiles per row, first tile of the level in the image
+    unsigned tiles_x_inv;               // ceil(2^32 / tiles_x) (tiles_x 1: 0, handled by the kernel)
     int slot0, max_kp;                  // first output slot of the level and its slots
 };
 
 struct OrbImage {
+    alignas(16) int tile0[FT_MAX_LEVELS];   // first tile of each level (levels that do not exist: past all tiles)
     OrbLevel lv[FT_MAX_LEVELS];
     int tiles, nslots;
     float *x, *y;                       // outputs, [nslots] each
