@@ -314,11 +314,11 @@ typedef struct {
 typedef struct ft_ctx ft_ctx;
 
 /* Launch shape of the fused kernel (chosen per batch-shape bucket by the
- * autotuner, or set by hand). */
+ * autotuner, or set by hand; otherwise from the rows and points a call brings). */
 typedef struct {
     int strip_rows;         /* image rows per pinhole stereo work item */
     int search_tile;        /* map points per search work item (multiple of 256) */
-    int fisheye_tile;       /* left keypoints per fisheye work item (64, or 128 for any larger value) */
+    int fisheye_tile;       /* kept for saved tables, any value: fisheye matching takes 128 left keypoints a block */
     int resolve_tile;       /* entries per conflict-resolution item */
     int ctas_per_sm;        /* persistent CTAs per SM (0: occupancy limit) */
     int search_stage;       /* kept for saved tables, any value: the search always stages a camera's
@@ -327,8 +327,8 @@ typedef struct {
                                scans its candidates (every test but the stereo consistency) before
                                it waits for the stereo step and applies the consistency after it,
                                -1 = it waits for the stereo step first (less work: best for large
-                               batches), 0 = automatic (1 for batches of at most 32 frames); results
-                               are the same */
+                               batches), 0 = automatic (1 while the search items do not exceed the
+                               resident CTAs and their records fit the arena); results are the same */
 } ft_tuning;
 
 /* Fill p with the default readings. */
@@ -512,14 +512,14 @@ ft_status ft_build_pyramids(ft_ctx *ctx, void *stream, const ft_params *params, 
 
 /* Stereo matching followed by the search, for a ragged batch of frames, in
  * one persistent fused launch (CUDA-graph replayed per batch-shape bucket if
- * the context was created with use_graphs).  Each frame's results equal
+ * the context was created with use_graphs; fisheye frames' stereo matching is a
+ * second kernel in the same graph).  Each frame's results equal
  * those of the per-frame calls. */
 ft_status ft_track_batch(ft_ctx *ctx, void *stream, const ft_params *params, const ft_batch *batch);
 
 /* Time candidate launch shapes on this batch (iters runs each) and keep the
  * fastest for the batch's bucket; *best receives it (may be NULL).  The
- * candidates: strip rows 16/32/64, search tile 256/512/1024, fisheye tile
- * 64/128, every count of CTAs per SM up to the resident maximum, and the
+ * candidates: strip rows 8/16/32/64, search tile 256/512/1024, every count of CTAs per SM up to the resident maximum, and the
  * search in one pass or two halves. */
 ft_status ft_autotune(ft_ctx *ctx, void *stream, const ft_params *params, const ft_batch *batch,
                       int iters, ft_tuning *best);

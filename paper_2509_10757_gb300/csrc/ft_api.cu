@@ -176,12 +176,65 @@ ft_tuning default_tuning()
     ft_tuning t{};
     t.strip_rows = 32;
     t.search_tile = 512;
-    t.fisheye_tile = 128;
+    t.fisheye_tile = 128;       // no effect
     t.resolve_tile = 2048;
     t.ctas_per_sm = 0;
     t.search_stage = 0;
     t.split_search = 0;
     return t;
+}
+
+// The launch shape of a batch that has none in the tuning table, from the work
+// its frames bring, for `slots` resident CTAs (456 on GB300).
+//   Strips: a frame's stereo step is a chain (row sort, strip, median, search),
+//   so few frames cut their rows finer until there are about 320 strips; a
+//   full chip takes 32 rows, and more than 600 strips of 48 rows waste less
+//   (752x480, 1250 keypoints, 3500 points, us per launch at 4 / 8 / 12 / 24 /
+//   32 / 48 rows: 1 frame 36 / 37 / 39 / - / 49 / -, 8 frames - / 49 / 43 / - /
+//   54 / -, 16 frames - / - / 55 / 53 / 56 / -, 32 frames - / - / - / 70 / 67 /
+//   74, 64 frames - / - / - / - / 107 / 105; 1280x720 stereo alone with 4000
+//   keypoints 39 / 40 / 47 / 53 / 62 / -).
+//   Search tiles: the smallest of 256, 512 and 1024 points that does not make
+//   more items than CTAs: below that a CTA's second tile only adds latency
+//   (20000 points, one frame: 34 us at 256, 38 at 512), above it staging the
+//   grid once per tile pays (32 fisheye frames of 6000 points: 103 / 98 / 91
+//   us; 32 1080p frames of 100000 points: 559 at 512, 520 at 1024).
+ft_tuning shape_for(const std::vector<Job> &jobs, int slots)
+{
+    ft_tuning t = default_tuning();
+    long long rows = 0, points = 0;
+    auto items = [&](int tile) {
+        long long n = 0;
+        for (const Job &j : jobs)
+            if (j.do_search) n += (long long)((j.map.n + tile - 1) / tile) * (j.camera == FT_CAMERA_FISHEYE ? 2 : 1);
+        return n;
+    };
+    for (const Job &j : jobs) {
+        if (j.do_stereo && j.camera == FT_CAMERA_PINHOLE) rows += j.pin.height;
+        if (j.do_search) points += j.map.n;
+    }
+    if (rows > 0) {
+        t.strip_rows = (int)std::min<long long>(std::max<long long>(rows / 320, 4), 32);
+        if (rows / 48 > 600) t.strip_rows = 48;
+    }
+    if (points > 0) {
+        t.search_tile = 256;
+        while (t.search_tile < 1024 && items(t.search_tile) > slots) t.search_tile *= 2;
+    }
+    return t;
+}
+
+// Search in two halves around the stereo step (ft_tuning.split_search 0): it
+// shortens the chain, and costs the records of the points between the halves,
+// so it pays while the search does not fill the chip more than once (64 frames
+// of 3500 points: 105 us split, 107 in one pass; 32 1080p frames of 100000:
+// 541 and 520).
+bool split_pays(const std::vector<Job> &jobs, int tile, int slots)
+{
+    long long n = 0;
+    for (const Job &j : jobs)
+        if (j.do_search && j.wait_stereo) n += (j.map.n + tile - 1) / tile;
+    return n <= slots;
 }
 
 }  // namespace
@@ -490,6 +543,7 @@ ft_status build_table(ft_ctx *ctx, const ft_params &params, const std::vector<Jo
         return p;
     };
     const int halo = B.p.halo;
+    const bool split = tune.split_search > 0;
     int counts[K_KINDS] = {};
     for (int f = 0; f < n; ++f) {
         const Job &j = jobs[f];
@@ -619,7 +673,7 @@ ft_status build_table(ft_ctx *ctx, const ft_params &params, const std::vector<Jo
                 C.owner = reinterpret_cast<unsigned long long *>(carve(sizeof(unsigned long long) * (size_t)C.nk));
                 // a pinhole frame whose stereo step runs in the same launch splits
                 // its search around it (search items need not wait for it)
-                F.split_search = j.wait_stereo && (tune.split_search > 0 || (tune.split_search == 0 && n <= 32));
+                F.split_search = j.wait_stereo && split;
                 if (F.split_search) C.scan = reinterpret_cast<uint4 *>(carve(sizeof(uint4) * 2 * (size_t)F.nm));
                 n_search[c] = (F.nm + F.search_tile - 1) / F.search_tile;
                 n_resolve[c] = (std::max(F.nm, C.nk) + F.resolve_tile - 1) / F.resolve_tile;
@@ -737,6 +791,13 @@ ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int sl
     return FT_OK;
 }
 
+// the launch shape of a batch: the table's, or the one its work suggests
+ft_tuning tuning_of(ft_ctx *ctx, const Bucket &bk, const std::vector<Job> &jobs)
+{
+    auto it = ctx->tuning.find(bk);
+    return it != ctx->tuning.end() ? it->second : shape_for(jobs, ctx->sm_count * ctx->occ);
+}
+
 ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, const std::vector<Job> &jobs,
                  const ft_tuning *force_tuning, bool allow_graph)
 {
@@ -752,20 +813,24 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
     }
     FT_CUDA(cudaSetDevice(ctx->device));
     const Bucket bk = bucket_of(jobs);
-    ft_tuning tune = default_tuning();
-    if (force_tuning) tune = *force_tuning;
-    else {
-        auto it = ctx->tuning.find(bk);
-        if (it != ctx->tuning.end()) tune = it->second;
-    }
+    const ft_tuning tune0 = force_tuning ? *force_tuning : tuning_of(ctx, bk, jobs);
+    ft_tuning tune = tune0;
+    // the search tile as the table uses it
+    const int tile = std::max(kThreads, tune.search_tile / kThreads * kThreads);
+    if (tune.split_search == 0) tune.split_search = split_pays(jobs, tile, ctx->sm_count * ctx->occ) ? 1 : -1;
     const int slot = ctx->slot;
     ctx->slot = (ctx->slot + 1) % kSlots;
     FT_CUDA(cudaEventSynchronize(ctx->slot_done[slot]));      // staging slot free again
     char *table_dev = ctx->arena + align_up(sizeof(unsigned) * 64);
     size_t bytes = 0;
     int items = 0;
-    if ((s = build_table(ctx, params, jobs, tune, ctx->staging[slot], table_dev, &bytes, &items)) != FT_OK)
-        return s;
+    s = build_table(ctx, params, jobs, tune, ctx->staging[slot], table_dev, &bytes, &items);
+    if (s == FT_ENOMEM && tune0.split_search == 0 && tune.split_search > 0) {
+        // the split search's records did not fit the arena: in one pass then
+        tune.split_search = -1;
+        s = build_table(ctx, params, jobs, tune, ctx->staging[slot], table_dev, &bytes, &items);
+    }
+    if (s != FT_OK) return s;
     if ((s = order_stream(ctx, stream)) != FT_OK) return s;
     const int cps = tune.ctas_per_sm > 0 ? std::min(tune.ctas_per_sm, ctx->occ) : ctx->occ;
     const int grid_max = ctx->sm_count * cps;
@@ -1435,36 +1500,31 @@ ft_status ft_get_tuning(ft_ctx *ctx, const ft_batch *batch, ft_tuning *t)
     std::vector<Job> jobs;
     ft_status s = jobs_of_batch(batch, jobs);
     if (s != FT_OK) return s;
-    auto it = ctx->tuning.find(bucket_of(jobs));
-    *t = it != ctx->tuning.end() ? it->second : default_tuning();
+    *t = tuning_of(ctx, bucket_of(jobs), jobs);
     return FT_OK;
 }
 
-// The launch shapes both autotuners try: strip rows 16/32/64, search tile
-// 256/512/1024, fisheye tile 64/128, every count of CTAs per SM from the
-// resident maximum down to one (fewer leave room for a concurrent launch)
+// The launch shapes both autotuners try: strip rows 8/16/32/64, search tile
+// 256/512/1024, every count of CTAs per SM from the resident maximum down to one (fewer leave room for a concurrent launch)
 // and the search in one pass or two halves.
 static std::vector<ft_tuning> tuning_candidates(int occ)
 {
-    const int strips[] = {16, 32, 64};
+    const int strips[] = {8, 16, 32, 64};
     const int tiles[] = {256, 512, 1024};
-    const int fish[] = {64, 128};
     std::vector<int> occs;
     for (int o = std::max(1, occ); o >= 1; --o) occs.push_back(o);
     std::vector<ft_tuning> cand;
     for (int a : strips)
         for (int b : tiles)
-            for (int c : fish)
-                for (int o : occs)
-                    for (int sp : {1, -1}) {
-                        ft_tuning t = default_tuning();
-                        t.strip_rows = a;
-                        t.search_tile = b;
-                        t.fisheye_tile = c;
-                        t.ctas_per_sm = o;
-                        t.split_search = sp;
-                        cand.push_back(t);
-                    }
+            for (int o : occs)
+                for (int sp : {1, -1}) {
+                    ft_tuning t = default_tuning();
+                    t.strip_rows = a;
+                    t.search_tile = b;
+                    t.ctas_per_sm = o;
+                    t.split_search = sp;
+                    cand.push_back(t);
+                }
     return cand;
 }
 
