@@ -45,6 +45,10 @@ ft_status fail(ft_status s, const char *fmt, ...)
     } while (0)
 
 constexpr int kSlots = 4;
+// words of the arena's first 256 bytes (the status word is the first): the
+// queue and the counters of one-frame calls, zero between launches
+constexpr int kOneQueue = 16, kOneCounters = 32;
+static_assert(kOneCounters + kCounters <= 64, "one-frame counters past the arena's head");
 constexpr size_t kAlign = 256;
 
 size_t align_up(size_t v, size_t a = kAlign) { return (v + a - 1) / a * a; }
@@ -149,6 +153,7 @@ struct ft_ctx {
     int max_frames = 0;
     size_t table_cap = 0;             // bytes of the table region
     size_t scratch_off = 0;           // scratch region offset in the arena
+    std::vector<char> one_table;      // host buffer a one-frame call's table is built in
     unsigned *status = nullptr;       // device status word
     char *staging[kSlots] = {};
     cudaEvent_t slot_done[kSlots] = {};
@@ -818,17 +823,23 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
     // the search tile as the table uses it
     const int tile = std::max(kThreads, tune.search_tile / kThreads * kThreads);
     if (tune.split_search == 0) tune.split_search = split_pays(jobs, tile, ctx->sm_count * ctx->occ) ? 1 : -1;
+    // one frame goes as kernel parameters (see FrameCall), unless its pyramids
+    // are built first or the launch is traced
+    const bool one = jobs.size() == 1 && !jobs[0].build_pyr && !ctx->trace;
     const int slot = ctx->slot;
-    ctx->slot = (ctx->slot + 1) % kSlots;
-    FT_CUDA(cudaEventSynchronize(ctx->slot_done[slot]));      // staging slot free again
+    if (!one) {
+        ctx->slot = (ctx->slot + 1) % kSlots;
+        FT_CUDA(cudaEventSynchronize(ctx->slot_done[slot]));      // staging slot free again
+    }
+    char *table = one ? ctx->one_table.data() : ctx->staging[slot];
     char *table_dev = ctx->arena + align_up(sizeof(unsigned) * 64);
     size_t bytes = 0;
     int items = 0;
-    s = build_table(ctx, params, jobs, tune, ctx->staging[slot], table_dev, &bytes, &items);
+    s = build_table(ctx, params, jobs, tune, table, table_dev, &bytes, &items);
     if (s == FT_ENOMEM && tune0.split_search == 0 && tune.split_search > 0) {
         // the split search's records did not fit the arena: in one pass then
         tune.split_search = -1;
-        s = build_table(ctx, params, jobs, tune, ctx->staging[slot], table_dev, &bytes, &items);
+        s = build_table(ctx, params, jobs, tune, table, table_dev, &bytes, &items);
     }
     if (s != FT_OK) return s;
     if ((s = order_stream(ctx, stream)) != FT_OK) return s;
@@ -864,6 +875,21 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
     int pose_frames = 0;
     for (size_t f = 0; f < jobs.size(); ++f)
         if (jobs[f].do_pose) pose_frames = (int)f + 1;
+    if (one) {
+        FrameCall call;
+        const TableLayout L = table_layout(1);
+        call.h = *reinterpret_cast<const BatchHeader *>(table + L.hdr);
+        call.f = *reinterpret_cast<const FrameDev *>(table + L.frames);
+        call.h.prefix = nullptr;
+        call.h.frames = nullptr;
+        call.h.queue = ctx->status + kOneQueue;
+        call.f.ctr = ctx->status + kOneCounters;
+        FT_CUDA(launch_fisheye(call, fish_blocks, stream));
+        if (items > 0) FT_CUDA(launch_fused(call, std::min(items, grid_max), stream));
+        if (pose_frames > 0) FT_CUDA(launch_pose(call, stream));
+        ctx->launches += (items > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) + (fish_frames > 0 ? 1 : 0);
+        return finish_call(ctx, stream);
+    }
     if (items > 0 || pyr_frames > 0 || pose_frames > 0 || fish_frames > 0) {
         if (allow_graph && ctx->use_graphs && items > 0) {
             const int fp2 = bk.frames_p2;
@@ -997,6 +1023,7 @@ ft_status ft_create(ft_ctx **out, const ft_ctx_desc *desc)
     // the table region holds a batch table of max_frames frames or an
     // extraction table of 4 x max_frames images
     c->table_cap = std::max(table_layout(d.max_frames).total, orb_table_bytes(4 * d.max_frames));
+    c->one_table.resize(table_layout(1).total);
     const size_t head = align_up(sizeof(unsigned) * 64);
     c->scratch_off = align_up(head + c->table_cap);
     c->arena_bytes = std::max(d.arena_bytes, c->scratch_off + ((size_t)1 << 20));

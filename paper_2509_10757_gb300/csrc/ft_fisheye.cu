@@ -361,12 +361,10 @@ __device__ __forceinline__ void scan_columns(const unsigned (&v)[32], const int 
     }
 }
 
-__global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const BatchHeader *__restrict__ hdr)
+__device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameDev &F)
 {
     extern __shared__ unsigned char fish_raw[];
     SmemFish &S = *reinterpret_cast<SmemFish *>(fish_raw + ((1024u - (smem_addr(fish_raw) & 1023u)) & 1023u));
-    if ((int)blockIdx.y >= hdr->nframes) return;
-    const FrameDev &F = hdr->frames[blockIdx.y];
     const int tile = (int)blockIdx.x;
     if (F.camera != FT_CAMERA_FISHEYE || !F.do_stereo || tile * kFishRows >= F.nl) return;
     const DevParams &P = hdr->p;
@@ -530,11 +528,45 @@ __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const Batch
     }
 }
 
+__global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const BatchHeader *__restrict__ hdr)
+{
+    if ((int)blockIdx.y >= hdr->nframes) return;
+    fisheye_run(hdr, hdr->frames[blockIdx.y]);
+}
+
+// one frame, its header and descriptor as kernel parameters
+__global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_one_kernel(const __grid_constant__ FrameCall call)
+{
+    fisheye_run(&call.h, call.f);
+}
+
+// Columns are shared out while that still leaves the chip's 152 SMs a block
+// each (about 60 % of a frame's blocks have rows: the overlap).
+void fisheye_launch_config(int nframes, int blocks, cudaStream_t stream, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &cluster)
+{
+    int splits = 1;
+    while (splits < kFishSplit && 2 * splits * blocks * nframes <= 256) splits *= 2;
+    cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, (unsigned)nframes, (unsigned)splits);
+    cfg.blockDim = dim3(kFishThreads);
+    cfg.dynamicSmemBytes = kFishSmem;
+    cfg.stream = stream;
+    cluster.id = cudaLaunchAttributeClusterDimension;
+    cluster.val.clusterDim.x = 1;
+    cluster.val.clusterDim.y = 1;
+    cluster.val.clusterDim.z = (unsigned)splits;
+    cfg.attrs = &cluster;
+    cfg.numAttrs = 1;
+}
+
 }  // namespace
 
 cudaError_t fisheye_setup()
 {
-    return cudaFuncSetAttribute(ft_fisheye_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFishSmem);
+    cudaError_t e = cudaFuncSetAttribute(ft_fisheye_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFishSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ft_fisheye_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFishSmem);
+    return e;
 }
 
 int fisheye_blocks(int nl) { return (nl + kFishRows - 1) / kFishRows; }
@@ -542,23 +574,19 @@ int fisheye_blocks(int nl) { return (nl + kFishRows - 1) / kFishRows; }
 cudaError_t launch_fisheye(const BatchHeader *dev_hdr, int nframes, int blocks, cudaStream_t stream)
 {
     if (nframes <= 0 || blocks <= 0) return cudaSuccess;
-    // columns are shared out while that still leaves the chip's 152 SMs a
-    // block each (about 60 % of a frame's blocks have rows: the overlap)
-    int splits = 1;
-    while (splits < kFishSplit && 2 * splits * blocks * nframes <= 256) splits *= 2;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks, (unsigned)nframes, (unsigned)splits);
-    cfg.blockDim = dim3(kFishThreads);
-    cfg.dynamicSmemBytes = kFishSmem;
-    cfg.stream = stream;
+    cudaLaunchConfig_t cfg;
     cudaLaunchAttribute cluster;
-    cluster.id = cudaLaunchAttributeClusterDimension;
-    cluster.val.clusterDim.x = 1;
-    cluster.val.clusterDim.y = 1;
-    cluster.val.clusterDim.z = (unsigned)splits;
-    cfg.attrs = &cluster;
-    cfg.numAttrs = 1;
+    fisheye_launch_config(nframes, blocks, stream, cfg, cluster);
     return cudaLaunchKernelEx(&cfg, ft_fisheye_kernel, dev_hdr);
+}
+
+cudaError_t launch_fisheye(const FrameCall &call, int blocks, cudaStream_t stream)
+{
+    if (blocks <= 0) return cudaSuccess;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute cluster;
+    fisheye_launch_config(1, blocks, stream, cfg, cluster);
+    return cudaLaunchKernelEx(&cfg, ft_fisheye_one_kernel, call);
 }
 
 }  // namespace ft

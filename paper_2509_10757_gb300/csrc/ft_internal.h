@@ -172,6 +172,16 @@ struct BatchHeader {
     int pad_;
 };
 
+// A call of one frame: its header and descriptor travel as kernel parameters
+// (no table copy ahead of the kernel, and no descriptor loads in it).  Its
+// queue and counters are a few words of the arena that are zero between
+// launches: the fused kernel's last block zeroes them again.
+struct FrameCall {
+    BatchHeader h;                 // prefix and frames are not used; queue[2] counts finished blocks
+    FrameDev f;
+};
+static_assert(sizeof(FrameCall) <= 4096, "a frame's call exceeds the kernel parameters");
+
 // ---------------------------------------------------------------- f3: keypoint extraction
 constexpr int kOrbTileW = 62;           // detection tile: with its suppression ring 64 x 32 pixels
 constexpr int kOrbTileH = 30;
@@ -219,6 +229,9 @@ struct OrbHeader {
 // Launch helpers implemented in ft_kernels.cu (host-callable).
 namespace ft {
 cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stream);
+cudaError_t launch_fused(const FrameCall &call, int grid, cudaStream_t stream);
+cudaError_t launch_pose(const FrameCall &call, cudaStream_t stream);
+cudaError_t launch_fisheye(const FrameCall &call, int blocks, cudaStream_t stream);
 // pose optimization of the frames with do_pose (one cluster per frame of the
 // first nframes; after the fused kernel on the same stream)
 cudaError_t launch_pose(const BatchHeader *dev_hdr, int nframes, cudaStream_t stream);

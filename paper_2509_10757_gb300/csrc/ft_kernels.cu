@@ -1576,7 +1576,18 @@ __device__ __forceinline__ void copy_words(void *dst, const void *src, size_t by
     for (size_t i = threadIdx.x; i < bytes / 4; i += kThreads) b[i] = __ldg(a + i);
 }
 
-__global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(const BatchHeader *__restrict__ hdr)
+// Words of a kernel parameter (not global memory).
+__device__ __forceinline__ void copy_param(void *dst, const void *src, size_t bytes)
+{
+    const unsigned *a = reinterpret_cast<const unsigned *>(src);
+    unsigned *b = reinterpret_cast<unsigned *>(dst);
+    for (size_t i = threadIdx.x; i < bytes / 4; i += blockDim.x) b[i] = a[i];
+}
+
+// The persistent loop over the batch table at hdr, or (kOne) over the single
+// frame of a call whose header hdr and descriptor one are kernel parameters.
+template <bool kOne>
+__device__ __forceinline__ void fused_run(const BatchHeader *hdr, const FrameDev *one)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_item;
@@ -1586,7 +1597,12 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(
     // then shared-memory loads instead of dependent global loads
     __shared__ __align__(16) BatchHeader sB;
     __shared__ __align__(16) FrameDev sF;
-    copy_words(&sB, hdr, sizeof(BatchHeader));
+    if (kOne) {
+        copy_param(&sB, hdr, sizeof(BatchHeader));
+        copy_param(&sF, one, sizeof(FrameDev));
+    } else {
+        copy_words(&sB, hdr, sizeof(BatchHeader));
+    }
     __syncthreads();
     for (;;) {
         if (threadIdx.x == 0) s_item = (int)atomicAdd(sB.queue, 1u);
@@ -1603,17 +1619,21 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(
         int kind = 0;
         while (kind < K_KINDS - 1 && item >= B.kind_begin[kind + 1]) ++kind;
         const int local = item - B.kind_begin[kind];
-        const int *pre = B.prefix + kind * (B.nframes + 1);
-        int lo = 0, hi = B.nframes - 1;          // last frame f with pre[f] <= local
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (pre[mid] <= local) lo = mid;
-            else hi = mid - 1;
+        int lo = 0, first = 0;                   // the item's frame, and its first item of the kind
+        if (!kOne) {
+            const int *pre = B.prefix + kind * (B.nframes + 1);
+            int hi = B.nframes - 1;              // last frame f with pre[f] <= local
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (pre[mid] <= local) lo = mid;
+                else hi = mid - 1;
+            }
+            first = pre[lo];
+            copy_words(&sF, B.frames + lo, sizeof(FrameDev));
+            __syncthreads();
         }
-        copy_words(&sF, B.frames + lo, sizeof(FrameDev));
-        __syncthreads();
         const FrameDev &F = *reinterpret_cast<const FrameDev *>(reinterpret_cast<const char *>(&sF) + 16 * zero);
-        const int tile = local - pre[lo];
+        const int tile = local - first;
         unsigned long long t_start = 0;
         if (B.trace != nullptr && threadIdx.x == 0) {
             t_start = global_ns();
@@ -1652,6 +1672,24 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(
             }
         }
     }
+    if (kOne && threadIdx.x == 0) {
+        // the last block of the launch leaves the queue and the counters zero
+        __threadfence();
+        if (atomicAdd(sB.queue + 2, 1u) == gridDim.x - 1) {
+            sB.queue[0] = sB.queue[2] = 0u;
+            for (int c = 0; c < kCounters; ++c) sF.ctr[c] = 0u;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_kernel(const BatchHeader *__restrict__ hdr)
+{
+    fused_run<false>(hdr, nullptr);
+}
+
+__global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_one_kernel(const __grid_constant__ FrameCall call)
+{
+    fused_run<true>(&call.h, &call.f);
 }
 
 }  // namespace
@@ -1909,20 +1947,24 @@ __device__ int pose_sum(int v, PoseShared &S, unsigned rank, int slot)
     return sum;
 }
 
-__global__ void __cluster_dims__(kPoseCtas, 1, 1) __launch_bounds__(kPoseThreads)
-    ft_pose_kernel(const BatchHeader *__restrict__ hdr)
+// kOne: the header and the frame are kernel parameters.
+template <bool kOne>
+__device__ __forceinline__ void pose_run(const BatchHeader *hdr, const FrameDev *one)
 {
     extern __shared__ __align__(16) float4 pose_stage[];      // [2][kPoseSlots]: the observations' two parts
     __shared__ PoseShared S;
     __shared__ __align__(16) DevParams sP;
     __shared__ __align__(16) FrameDev sF;
     const int f = (int)blockIdx.x / kPoseCtas;
-    if (f >= hdr->nframes || !hdr->frames[f].do_pose) return;       // the whole cluster
+    if (!kOne && (f >= hdr->nframes || !hdr->frames[f].do_pose)) return;       // the whole cluster
     const unsigned rank = cluster_rank();
     const int tid = threadIdx.x, lane = tid & 31;
     const int vt = (int)rank * kPoseThreads + tid;            // thread of the frame
     const int vw = vt >> 5;                                   // warp of the frame
-    {
+    if (kOne) {
+        copy_param(&sF, one, sizeof(FrameDev));
+        copy_param(&sP, &hdr->p, sizeof(DevParams));
+    } else {
         const unsigned *a = reinterpret_cast<const unsigned *>(hdr->frames + f);
         unsigned *b = reinterpret_cast<unsigned *>(&sF);
         for (int i = tid; i < (int)(sizeof(FrameDev) / 4); i += kPoseThreads) b[i] = __ldg(a + i);
@@ -2098,6 +2140,18 @@ __global__ void __cluster_dims__(kPoseCtas, 1, 1) __launch_bounds__(kPoseThreads
     }
 }
 
+__global__ void __cluster_dims__(kPoseCtas, 1, 1) __launch_bounds__(kPoseThreads)
+    ft_pose_kernel(const BatchHeader *__restrict__ hdr)
+{
+    pose_run<false>(hdr, nullptr);
+}
+
+__global__ void __cluster_dims__(kPoseCtas, 1, 1) __launch_bounds__(kPoseThreads)
+    ft_pose_one_kernel(const __grid_constant__ FrameCall call)
+{
+    pose_run<true>(&call.h, &call.f);
+}
+
 }  // namespace
 
 int fused_smem_bytes() { return (int)sizeof(Smem); }
@@ -2109,7 +2163,11 @@ cudaError_t fused_occupancy(int *ctas_per_sm)
     cudaError_t e = cudaFuncSetAttribute(ft_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(Smem));
     if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ft_fused_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+    if (e == cudaSuccess)
         e = cudaFuncSetAttribute(ft_pose_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPoseSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ft_pose_one_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPoseSmem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas_per_sm, ft_fused_kernel, kThreads,
                                                          sizeof(Smem));
@@ -2118,6 +2176,18 @@ cudaError_t fused_occupancy(int *ctas_per_sm)
 cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stream)
 {
     ft_fused_kernel<<<grid, kThreads, sizeof(Smem), stream>>>(dev_hdr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fused(const FrameCall &call, int grid, cudaStream_t stream)
+{
+    ft_fused_one_kernel<<<grid, kThreads, sizeof(Smem), stream>>>(call);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pose(const FrameCall &call, cudaStream_t stream)
+{
+    ft_pose_one_kernel<<<kPoseCtas, kPoseThreads, kPoseSmem, stream>>>(call);
     return cudaGetLastError();
 }
 
