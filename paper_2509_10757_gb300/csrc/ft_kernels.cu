@@ -169,7 +169,8 @@ struct RefineJob {
 
 constexpr int kGroup = 4;                       // lanes per left keypoint in the Hamming phase
 constexpr int kGroups = kThreads / kGroup;      // left keypoints in flight per CTA
-constexpr int kSadChunk = 64;                   // matches refined per round
+constexpr int kSadChunk = 23;                   // matches refined per round: 253 of their patch rows, one a thread
+constexpr int kSadBufs = 3;                     // rounds of patches on chip: one in use, two on their way
 constexpr int kChunksL = 2;                     // 16-byte chunks holding a left patch row (11 bytes)
 constexpr int kChunksR = 3;                     // chunks holding a right strip row (21 bytes)
 
@@ -191,16 +192,16 @@ struct StageBuf {
     float4 rkp[kStageCap];             // staged right keypoints sorted by (octave, row)
     uint4 sdesc[2 * kStageCap];        // their descriptors in row order
     LeftBuf left;
+    int bptr[kOctBuckets * kWinRows + 1];   // start of each (octave, window row) bucket
 };
 
 struct SmemStereo {
     union {                            // the window and the left keypoints are dead once
         StageBuf st;                   // the Hamming phase is over; the patches reuse them
-        PatchBuf patch;                // (a strip with a second pass stages its window again)
+        PatchBuf patch[kSadBufs];      // (a strip with a second pass stages its window again)
     } u;
     RefineJob ref[kThreads];
-    int sad[kSadChunk][12];
-    int bptr[kOctBuckets * kWinRows + 1];   // start of each (octave, window row) bucket
+    int sad[2][kSadChunk][12];         // this round's and the last one's
     int warp_sums[kWarps];
     int nref;
 };
@@ -600,8 +601,8 @@ __device__ void hamming_phase(const DevParams &P, const FrameDev &F, SmemStereo 
                         const int h = P.halo_c[o];
                         const int ra = max(row - h, w_a) - w_a;
                         const int rb = min(row + h, w_a + nrows - 1) - w_a;
-                        const int e1 = S.bptr[o * nrows + rb + 1];
-                        for (int e = S.bptr[o * nrows + ra] + sub; e < e1; e += kGroup) {
+                        const int e1 = S.u.st.bptr[o * nrows + rb + 1];
+                        for (int e = S.u.st.bptr[o * nrows + ra] + sub; e < e1; e += kGroup) {
                             const float4 g = S.u.st.rkp[e];
                             const int oj = rec_octave(g.w);
                             if (oj < oi - 1 || oj > oi + 1) continue;
@@ -691,54 +692,57 @@ __device__ void hamming_phase(const DevParams &P, const FrameDev &F, SmemStereo 
     }
 }
 
-// Phases 2-3 for refine jobs [r0, r0 + nc), nc <= kSadChunk:
-// (2) one warp per match copies its 11 left patch rows and 11 right strip
-//     rows into shared memory, lanes on consecutive bytes (coalesced);
-// (3) one thread per (match, patch row) reads its rows as words and adds the
-//     row's part of the 11 SADs of centre-subtracted patches; then per match
-//     the first strict minimum over the shifts, the parabola, disparity and
-//     depth.
-__device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &S, int r0, int nc)
+// Asks for the patches of refine round r (jobs r * kSadChunk ...) by
+// asynchronous copies of the 16-byte chunks holding every patch row, and
+// closes the group; a match has five chunk slots (two of a left row, three of
+// a right row) and two threads per slot walk the 11 rows.  Level pointers and
+// pitches are 16-byte aligned (checked on the host): a row's chunks start at
+// its column rounded down to a multiple of 16 and end within the row's pitch.
+__device__ __forceinline__ void refine_copy(const FrameDev &F, SmemStereo &S, int r, int nref)
 {
-    const int tid = threadIdx.x;
-    constexpr int kRows = 2 * kW + 1;
-    for (int q = tid; q < nc * kShifts; q += kThreads) S.sad[q / kShifts][q % kShifts] = 0;
-    // asynchronous copies of the 16-byte chunks holding every patch row; a
-    // match has five chunk slots (two of a left row, three of a right row)
-    // and one thread per slot walks the 11 rows.  Level pointers and pitches
-    // are 16-byte aligned (checked on the host): a row's chunks start at its
-    // column rounded down to a multiple of 16 and end within the row's pitch.
-    constexpr int kSlots = kChunksL + kChunksR;
-    for (int q = tid; q < nc * kSlots; q += kThreads) {
-        const int mm = q / kSlots, w = q - mm * kSlots;
+    constexpr int kSlots = kChunksL + kChunksR, kRows = 2 * kW + 1, kHalf = (kRows + 1) / 2;
+    const int nc = min(kSadChunk, nref - r * kSadChunk);
+    const int q = threadIdx.x, mm = q / (2 * kSlots), w = (q - mm * 2 * kSlots) >> 1, row0 = (q & 1) * kHalf;
+    PatchBuf &B = S.u.patch[r % kSadBufs];
+    if (mm < nc) {
         const bool right = w >= kChunksL;
         const int k = right ? w - kChunksL : w;
-        const RefineJob &J = S.ref[r0 + mm];
+        const RefineJob &J = S.ref[r * kSadChunk + mm];
         const int col = right ? J.ur0 - kL - kW : J.ul - kW;
         const int len = right ? kStripW : 2 * kW + 1;
-        if (k > (((col & 15) + len - 1) >> 4)) continue;    // the chunk holds none of the row's bytes
-        const int pitch = right ? F.rp[J.l] : F.lp[J.l];
-        const uint8_t *src = (right ? F.pyrR[J.l] : F.pyrL[J.l]) + (size_t)(J.vl - kW) * pitch + (col & ~15) + 16 * k;
-        const unsigned dst = (unsigned)__cvta_generic_to_shared(right ? &S.u.patch.r[mm][0][k]
-                                                                       : &S.u.patch.l[mm][0][k]);
-        const unsigned dstep = 16u * (right ? kChunksR : kChunksL);
+        if (k <= (((col & 15) + len - 1) >> 4)) {           // else the chunk holds none of the row's bytes
+            const int pitch = right ? F.rp[J.l] : F.lp[J.l];
+            const uint8_t *src =
+                (right ? F.pyrR[J.l] : F.pyrL[J.l]) + (size_t)(J.vl - kW + row0) * pitch + (col & ~15) + 16 * k;
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(right ? &B.r[mm][row0][k] : &B.l[mm][row0][k]);
+            const unsigned dstep = 16u * (right ? kChunksR : kChunksL);
 #pragma unroll
-        for (int row = 0; row < kRows; ++row)
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + row * dstep),
-                         "l"(src + (size_t)row * pitch)
-                         : "memory");
+            for (int row = 0; row < kHalf; ++row)
+                if (row0 + row < kRows)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + row * dstep),
+                                 "l"(src + (size_t)row * pitch)
+                                 : "memory");
+        }
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    __syncthreads();
-    for (int q = tid; q < nc * kRows; q += kThreads) {
-        const int dy = q / nc, m = q - dy * nc;
-        const RefineJob &J = S.ref[r0 + m];
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Adds this thread's patch row of round r to the 11 SADs of its match.
+__device__ __forceinline__ void refine_row(SmemStereo &S, int r, int nref)
+{
+    constexpr int kRows = 2 * kW + 1;
+    static_assert(kSadChunk * kRows <= kThreads, "one patch row a thread");
+    const int nc = min(kSadChunk, nref - r * kSadChunk);
+    const PatchBuf &B = S.u.patch[r % kSadBufs];
+    const int dy = threadIdx.x / kSadChunk, m = threadIdx.x - dy * kSadChunk;
+    if (dy < kRows && m < nc) {
+        const RefineJob &J = S.ref[r * kSadChunk + m];
         const int ol = (J.ul - kW) & 15, orr = (J.ur0 - kL - kW) & 15;
         // the rows as 32-bit words; byte b of a row is byte (o + b) of its chunks
-        const unsigned *ql = reinterpret_cast<const unsigned *>(S.u.patch.l[m][dy]) + (ol >> 2);
-        const unsigned *qr = reinterpret_cast<const unsigned *>(S.u.patch.r[m][dy]) + (orr >> 2);
-        const unsigned *qc = reinterpret_cast<const unsigned *>(S.u.patch.r[m][kW]) + (orr >> 2);
-        const unsigned *qlc = reinterpret_cast<const unsigned *>(S.u.patch.l[m][kW]) + (ol >> 2);
+        const unsigned *ql = reinterpret_cast<const unsigned *>(B.l[m][dy]) + (ol >> 2);
+        const unsigned *qr = reinterpret_cast<const unsigned *>(B.r[m][dy]) + (orr >> 2);
+        const unsigned *qc = reinterpret_cast<const unsigned *>(B.r[m][kW]) + (orr >> 2);
+        const unsigned *qlc = reinterpret_cast<const unsigned *>(B.l[m][kW]) + (ol >> 2);
         const int sl = 8 * (ol & 3), sr = 8 * (orr & 3);
         // realigned words: byte b of the row is byte b & 3 of word b >> 2
         unsigned wl[3], wr[6], wc[4];
@@ -763,21 +767,38 @@ __device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &
             int s = 0;
 #pragma unroll
             for (int dx = 0; dx < 2 * kW + 1; ++dx) s = __sad(lc[dx] + cr[k], rv[k + dx], s);
-            atomicAdd(&S.sad[m][k], s);
+            atomicAdd(&S.sad[r & 1][m][k], s);
         }
     }
-    __syncthreads();
-    for (int m = tid; m < nc; m += kThreads) {
-        const RefineJob &J = S.ref[r0 + m];
-        const int *sad = S.sad[m];
-        int kb = 0;
+}
+
+// Match m of round r: the first strict minimum over the shifts, the parabola,
+// disparity and depth; its SADs are left zero for round r + 2.
+__device__ __forceinline__ void refine_finish(const DevParams &P, const FrameDev &F, SmemStereo &S, int r, int nref, int m)
+{
+    if (m < min(kSadChunk, nref - r * kSadChunk)) {
+        const RefineJob &J = S.ref[r * kSadChunk + m];
+        int sad[kShifts];
+#pragma unroll
+        for (int k = 0; k < kShifts; ++k) {
+            sad[k] = S.sad[r & 1][m][k];
+            S.sad[r & 1][m][k] = 0;
+        }
+        // (the neighbours of the minimum are carried along: no dynamic index)
+        int kb = 0, lo = 0, best = sad[0], hi = sad[1];
+#pragma unroll
         for (int k = 1; k < kShifts; ++k)
-            if (sad[k] < sad[kb]) kb = k;
+            if (sad[k] < best) {
+                kb = k;
+                lo = sad[k - 1];
+                best = sad[k];
+                hi = k + 1 < kShifts ? sad[k + 1 < kShifts ? k + 1 : k] : 0;
+            }
         const int shift = kb - kL;
         int sadb = -1;
         float ur = -1.0f, dep = -1.0f;
         if (kb != 0 && kb != 2 * kL) {
-            const float d1 = (float)sad[kb - 1], d2 = (float)sad[kb], d3 = (float)sad[kb + 1];
+            const float d1 = (float)lo, d2 = (float)best, d3 = (float)hi;
             const float delta = fdiv(fsub(d1, d3), fmul(2.0f, fsub(fadd(d1, d3), fmul(2.0f, d2))));
             if (!(delta < -1.0f || delta > 1.0f)) {
                 float ur_sub = fmul(P.sc[J.l], fadd(fadd((float)J.ur0, (float)shift), delta));
@@ -790,13 +811,38 @@ __device__ void refine_round(const DevParams &P, const FrameDev &F, SmemStereo &
                     }
                     dep = fdiv(F.bf, disparity);
                     ur = ur_sub;
-                    sadb = sad[kb];
+                    sadb = best;
                 }
             }
         }
         write_stereo(F, J.i, J.j, J.d, shift, sadb, ur, dep);
     }
+}
+
+// Refinement of the pass's nref matches: rounds of kSadChunk, the copies of
+// the next two rounds on their way while a round is summed and the last
+// warp finishes the round before it; one block-wide synchronization a round.
+// What bounds a round is the latency of its scattered rows: rounds of 64
+// matches that waited for their own copies took 15 us a strip of 112
+// matches (64 frames, 3 blocks an SM), these 10 us.
+__device__ void refine_matches(const DevParams &P, const FrameDev &F, SmemStereo &S, int nref)
+{
+    const int tid = threadIdx.x, last = tid - (kThreads - 32);
+    static_assert(kSadChunk <= 32 && kSadBufs == 3, "a warp finishes a round; two rounds of copies in flight");
+    for (int q = tid; q < 2 * kSadChunk * 12; q += kThreads) (&S.sad[0][0][0])[q] = 0;
+    refine_copy(F, S, 0, nref);
+    refine_copy(F, S, 1, nref);
+    const int rounds = (nref + kSadChunk - 1) / kSadChunk;
+    for (int r = 0; r < rounds; ++r) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncthreads();
+        refine_copy(F, S, r + 2, nref);             // into the buffer of round r - 1
+        if (r > 0 && last >= 0) refine_finish(P, F, S, r - 1, nref, last);
+        refine_row(S, r, nref);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
+    if (rounds > 0 && last >= 0) refine_finish(P, F, S, rounds - 1, nref, last);
 }
 
 // warp 0: bin of the k-th smallest value (0-based) of a 256-bin histogram
@@ -910,7 +956,7 @@ __device__ __forceinline__ void stage_window(const FrameDev &F, SmemStereo &S, i
     for (int e = tid; e < 2 * n_st; e += kThreads) cp_async16(&S.u.st.sdesc[e], F.rs_desc + 2 * e_base + e);
     constexpr int Q = kStageCap / kThreads;
     const int nb = kOctBuckets * nrows;
-    for (int b = tid; b <= nb; b += kThreads) S.bptr[b] = 0;
+    for (int b = tid; b <= nb; b += kThreads) S.u.st.bptr[b] = 0;
     __syncthreads();
     float4 g[Q];
     int bucket[Q], rank[Q];
@@ -920,17 +966,17 @@ __device__ __forceinline__ void stage_window(const FrameDev &F, SmemStereo &S, i
         if (e < n_st) {
             g[q] = __ldcg(F.rs_kp + e_base + e);
             bucket[q] = clampi(rec_octave(g[q].w), 0, kOctBuckets - 1) * nrows + (__float_as_int(g[q].z) - w_a);
-            rank[q] = atomicAdd(&S.bptr[bucket[q]], 1);
+            rank[q] = atomicAdd(&S.u.st.bptr[bucket[q]], 1);
         }
     }
     __syncthreads();
-    block_scan(S.bptr, S.bptr, nb + 1, S.warp_sums);
+    block_scan(S.u.st.bptr, S.u.st.bptr, nb + 1, S.warp_sums);
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int e = q * kThreads + tid;
         if (e < n_st) {
             g[q].z = __int_as_float(e);          // row-order position: its descriptor
-            S.u.st.rkp[S.bptr[bucket[q]] + rank[q]] = g[q];
+            S.u.st.rkp[S.u.st.bptr[bucket[q]] + rank[q]] = g[q];
         }
     }
 }
@@ -973,10 +1019,9 @@ __device__ void stereo_pinhole_item(const BatchHeader &B, const FrameDev &F, int
             __syncthreads();
             mark(B, 1);
             const int nref = S.nref;
-            for (int r0 = 0; r0 < nref; r0 += kSadChunk)
-                refine_round(P, F, S, r0, min(kSadChunk, nref - r0));
-            if (tid == 0) S.nref = 0;
+            refine_matches(P, F, S, nref);
             __syncthreads();
+            if (tid == 0) S.nref = 0;
             mark(B, 2);
         }
     }
