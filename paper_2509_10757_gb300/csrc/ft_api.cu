@@ -2,10 +2,14 @@
 //
 // Context = one device arena allocated once at creation (the paper
 // preallocates all GPU memory at start-up and reuses it, section IV-A),
-// a ring of pinned staging slots for the per-call batch table, events, a
-// CUDA-graph cache and the tuning table.  Every entry point turns its
-// arguments into a batch table (see ft_internal.h), copies it into the
-// arena with one cudaMemcpyAsync and launches the fused persistent kernel.
+// a ring of staging slots for the per-call batch table (pinned host memory and
+// a device copy each), events, a CUDA-graph cache and the tuning table.  Every
+// entry point turns its arguments into a batch table (see ft_internal.h),
+// copies it to the slot's device memory and launches the fused persistent
+// kernel.  The copy runs on a stream of the context's own and the call's
+// stream waits for it, so that a call issued while earlier work runs finds its
+// table there: 64 frames' 115 KB table cost 8 us between two launches when it
+// was copied on the call's stream.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -151,13 +155,17 @@ struct ft_ctx {
     char *arena = nullptr;
     size_t arena_bytes = 0;
     int max_frames = 0;
-    size_t table_cap = 0;             // bytes of the table region
+    size_t table_cap = 0;             // bytes of a slot's table
     size_t scratch_off = 0;           // scratch region offset in the arena
     std::vector<char> one_table;      // host buffer a one-frame call's table is built in
     unsigned *status = nullptr;       // device status word
     char *staging[kSlots] = {};
-    cudaEvent_t slot_done[kSlots] = {};
+    char *tables = nullptr;           // device copies of the slots' tables, table_cap bytes each
+    cudaStream_t copy_stream = nullptr;
+    cudaEvent_t copied[kSlots] = {};  // the slot's table has reached the device
+    cudaEvent_t slot_done[kSlots] = {};     // the slot's kernels have ended
     int slot = 0;
+    const char *last_table = nullptr; // device table of the last call (tracing)
     cudaEvent_t done = nullptr;
     cudaStream_t last_stream = nullptr;
     bool have_last = false;
@@ -759,9 +767,30 @@ ft_status finish_call(ft_ctx *ctx, cudaStream_t s)
     return FT_OK;
 }
 
-ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int slot, int grid,
-                    size_t copy_bytes, int pyr_frames, int pyr_blocks, int pyr_levels, int pose_frames,
-                    int fish_blocks, cudaGraphExec_t *out)
+// Copies the first `bytes` of the slot's staged table to its device memory
+// ahead of what `stream` runs next.  A stream that is being captured takes the
+// copy itself.
+ft_status send_table(ft_ctx *ctx, int slot, size_t bytes, cudaStream_t stream)
+{
+    char *dev = ctx->tables + (size_t)slot * ctx->table_cap;
+    ctx->last_table = dev;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &capturing) != cudaSuccess) {
+        (void)cudaGetLastError();
+        capturing = cudaStreamCaptureStatusNone;
+    }
+    if (capturing != cudaStreamCaptureStatusNone) {
+        FT_CUDA(cudaMemcpyAsync(dev, ctx->staging[slot], bytes, cudaMemcpyHostToDevice, stream));
+        return FT_OK;
+    }
+    FT_CUDA(cudaMemcpyAsync(dev, ctx->staging[slot], bytes, cudaMemcpyHostToDevice, ctx->copy_stream));
+    FT_CUDA(cudaEventRecord(ctx->copied[slot], ctx->copy_stream));
+    FT_CUDA(cudaStreamWaitEvent(stream, ctx->copied[slot], 0));
+    return FT_OK;
+}
+
+ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int slot, int grid, int pyr_frames, int pyr_blocks,
+                    int pyr_levels, int pose_frames, int fish_blocks, cudaGraphExec_t *out)
 {
     // the pyramid launch's shared memory depends on the level count
     const auto key = std::make_tuple(frames_p2, cps, slot, pyr_frames, pyr_blocks, pyr_levels, pose_frames, fish_blocks);
@@ -774,10 +803,9 @@ ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int sl
     cudaStream_t cs = ctx->capture_stream;
     cudaGraph_t g = nullptr;
     FT_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-    const cudaError_t e1 = cudaMemcpyAsync(table_dev, ctx->staging[slot], copy_bytes, cudaMemcpyHostToDevice, cs);
-    const cudaError_t e0 =
+    const cudaError_t e1 =
         launch_pyramids(reinterpret_cast<const BatchHeader *>(table_dev), pyr_frames, pyr_levels, pyr_blocks, cs);
-    cudaError_t e2 = e0 != cudaSuccess ? e0 : launch_fisheye(reinterpret_cast<const BatchHeader *>(table_dev),
+    cudaError_t e2 = e1 != cudaSuccess ? e1 : launch_fisheye(reinterpret_cast<const BatchHeader *>(table_dev),
                                                              frames_p2, fish_blocks, cs);
     if (e2 == cudaSuccess) e2 = launch_fused(reinterpret_cast<const BatchHeader *>(table_dev), grid, cs);
     if (e2 == cudaSuccess) e2 = launch_pose(reinterpret_cast<const BatchHeader *>(table_dev), pose_frames, cs);
@@ -832,7 +860,7 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         FT_CUDA(cudaEventSynchronize(ctx->slot_done[slot]));      // staging slot free again
     }
     char *table = one ? ctx->one_table.data() : ctx->staging[slot];
-    char *table_dev = ctx->arena + align_up(sizeof(unsigned) * 64);
+    char *table_dev = ctx->tables + (size_t)slot * ctx->table_cap;
     size_t bytes = 0;
     int items = 0;
     s = build_table(ctx, params, jobs, tune, table, table_dev, &bytes, &items);
@@ -893,15 +921,14 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
     if (items > 0 || pyr_frames > 0 || pose_frames > 0 || fish_frames > 0) {
         if (allow_graph && ctx->use_graphs && items > 0) {
             const int fp2 = bk.frames_p2;
-            const size_t copy = std::max(bytes, table_layout(fp2).total);
             cudaGraphExec_t exec = nullptr;
-            if ((s = get_graph(ctx, table_dev, fp2, cps, slot, grid_max, std::min(copy, ctx->table_cap),
-                               pyr_frames > 0 ? fp2 : 0, pyr_blocks, params.nlevels, pose_frames > 0 ? fp2 : 0,
+            if ((s = send_table(ctx, slot, bytes, stream)) != FT_OK) return s;
+            if ((s = get_graph(ctx, table_dev, fp2, cps, slot, grid_max, pyr_frames > 0 ? fp2 : 0, pyr_blocks, params.nlevels, pose_frames > 0 ? fp2 : 0,
                                next_pow2_or_zero(fish_blocks), &exec)) != FT_OK)
                 return s;
             FT_CUDA(cudaGraphLaunch(exec, stream));
         } else {
-            FT_CUDA(cudaMemcpyAsync(table_dev, ctx->staging[slot], bytes, cudaMemcpyHostToDevice, stream));
+            if ((s = send_table(ctx, slot, bytes, stream)) != FT_OK) return s;
             if (pyr_frames > 0)
                 FT_CUDA(launch_pyramids(reinterpret_cast<const BatchHeader *>(table_dev), pyr_frames, params.nlevels,
                                         pyr_blocks,
@@ -1020,12 +1047,12 @@ ft_status ft_create(ft_ctx **out, const ft_ctx_desc *desc)
     if (e == cudaSuccess) e = fisheye_setup();
     c->sm_count = prop.multiProcessorCount;
     if (c->occ < 1) c->occ = 1;
-    // the table region holds a batch table of max_frames frames or an
-    // extraction table of 4 x max_frames images
-    c->table_cap = std::max(table_layout(d.max_frames).total, orb_table_bytes(4 * d.max_frames));
+    // a slot's table holds a batch table of max_frames frames or an extraction
+    // table of 4 x max_frames images
+    c->table_cap = align_up(std::max(table_layout(d.max_frames).total, orb_table_bytes(4 * d.max_frames)));
     c->one_table.resize(table_layout(1).total);
     const size_t head = align_up(sizeof(unsigned) * 64);
-    c->scratch_off = align_up(head + c->table_cap);
+    c->scratch_off = head;
     c->arena_bytes = std::max(d.arena_bytes, c->scratch_off + ((size_t)1 << 20));
     if (e == cudaSuccess) e = cudaMalloc(&c->arena, c->arena_bytes);
     if (e == cudaSuccess) {
@@ -1035,9 +1062,12 @@ ft_status ft_create(ft_ctx **out, const ft_ctx_desc *desc)
     for (int i = 0; i < kSlots && e == cudaSuccess; ++i) {
         e = cudaMallocHost(&c->staging[i], c->table_cap);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->slot_done[i], cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->copied[i], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->capture_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->copy_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMalloc(&c->tables, (size_t)kSlots * c->table_cap);
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         ft_destroy(c);
@@ -1056,9 +1086,12 @@ void ft_destroy(ft_ctx *c)
     for (int i = 0; i < kSlots; ++i) {
         if (c->staging[i]) cudaFreeHost(c->staging[i]);
         if (c->slot_done[i]) cudaEventDestroy(c->slot_done[i]);
+        if (c->copied[i]) cudaEventDestroy(c->copied[i]);
     }
     if (c->done) cudaEventDestroy(c->done);
     if (c->capture_stream) cudaStreamDestroy(c->capture_stream);
+    if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
+    if (c->tables) cudaFree(c->tables);
     if (c->arena) cudaFree(c->arena);
     if (c->trace) cudaFree(c->trace);
     delete c;
@@ -1101,8 +1134,9 @@ ft_status ft_read_trace(ft_ctx *c, ft_trace_record *out, int max, int *n)
     FT_CUDA(cudaSetDevice(c->device));
     if (c->have_last) FT_CUDA(cudaStreamSynchronize(c->last_stream));
     unsigned cnt = 0;
-    const char *queue = c->arena + align_up(sizeof(unsigned) * 64) + table_layout(1).queue;
-    FT_CUDA(cudaMemcpy(&cnt, queue + sizeof(unsigned), sizeof(unsigned), cudaMemcpyDeviceToHost));
+    if (c->last_table)
+        FT_CUDA(cudaMemcpy(&cnt, c->last_table + table_layout(1).queue + sizeof(unsigned), sizeof(unsigned),
+                           cudaMemcpyDeviceToHost));
     *n = (int)cnt;
     const int k = std::min<int>(std::min<unsigned>(cnt, (unsigned)c->trace_cap), max);
     if (k > 0 && c->trace)
@@ -1267,7 +1301,7 @@ ft_status ft_extract_orb(ft_ctx *ctx, void *stream, const ft_params *params, int
     ctx->slot = (ctx->slot + 1) % kSlots;
     FT_CUDA(cudaEventSynchronize(ctx->slot_done[slot]));
     char *h = ctx->staging[slot];
-    char *dev = ctx->arena + align_up(sizeof(unsigned) * 64);
+    char *dev = ctx->tables + (size_t)slot * ctx->table_cap;
     std::memset(h, 0, bytes);
     OrbHeader &Hd = *reinterpret_cast<OrbHeader *>(h);
     Hd.nimages = n;
@@ -1331,7 +1365,7 @@ ft_status ft_extract_orb(ft_ctx *ctx, void *stream, const ft_params *params, int
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = order_stream(ctx, st)) != FT_OK) return s;
     if (n > 0) {
-        FT_CUDA(cudaMemcpyAsync(dev, h, bytes, cudaMemcpyHostToDevice, st));
+        if ((s = send_table(ctx, slot, bytes, st)) != FT_OK) return s;
         FT_CUDA(launch_orb(reinterpret_cast<const OrbHeader *>(dev), n, p.nlevels, max_tiles, nslots, st));
         ctx->launches += 3;
     }
@@ -1531,12 +1565,12 @@ ft_status ft_get_tuning(ft_ctx *ctx, const ft_batch *batch, ft_tuning *t)
     return FT_OK;
 }
 
-// The launch shapes both autotuners try: strip rows 8/16/32/64, search tile
+// The launch shapes both autotuners try: strip rows 16/32/64, search tile
 // 256/512/1024, every count of CTAs per SM from the resident maximum down to one (fewer leave room for a concurrent launch)
 // and the search in one pass or two halves.
 static std::vector<ft_tuning> tuning_candidates(int occ)
 {
-    const int strips[] = {8, 16, 32, 64};
+    const int strips[] = {16, 32, 64};
     const int tiles[] = {256, 512, 1024};
     std::vector<int> occs;
     for (int o = std::max(1, occ); o >= 1; --o) occs.push_back(o);
