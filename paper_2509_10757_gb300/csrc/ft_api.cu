@@ -805,10 +805,10 @@ ft_status get_graph(ft_ctx *ctx, char *table_dev, int frames_p2, int cps, int sl
     FT_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     const cudaError_t e1 =
         launch_pyramids(reinterpret_cast<const BatchHeader *>(table_dev), pyr_frames, pyr_levels, pyr_blocks, cs);
-    cudaError_t e2 = e1 != cudaSuccess ? e1 : launch_fisheye(reinterpret_cast<const BatchHeader *>(table_dev),
-                                                             frames_p2, fish_blocks, cs);
-    if (e2 == cudaSuccess) e2 = launch_fused(reinterpret_cast<const BatchHeader *>(table_dev), grid, cs);
-    if (e2 == cudaSuccess) e2 = launch_pose(reinterpret_cast<const BatchHeader *>(table_dev), pose_frames, cs);
+    const BatchHeader *hdr = reinterpret_cast<const BatchHeader *>(table_dev);
+    cudaError_t e2 = e1 != cudaSuccess ? e1 : launch_fisheye(hdr, frames_p2, fish_blocks, cs, pyr_frames > 0);
+    if (e2 == cudaSuccess) e2 = launch_fused(hdr, grid, cs, pyr_frames > 0 || fish_blocks > 0);
+    if (e2 == cudaSuccess) e2 = launch_pose(hdr, pose_frames, cs);
     const cudaError_t e3 = cudaStreamEndCapture(cs, &g);
     if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
         if (g) cudaGraphDestroy(g);
@@ -912,8 +912,10 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         call.h.frames = nullptr;
         call.h.queue = ctx->status + kOneQueue;
         call.f.ctr = ctx->status + kOneCounters;
+        // a call's first kernel follows the stream's earlier work as any launch
+        // does; only a kernel behind another of the same call may start early
         FT_CUDA(launch_fisheye(call, fish_blocks, stream));
-        if (items > 0) FT_CUDA(launch_fused(call, std::min(items, grid_max), stream));
+        if (items > 0) FT_CUDA(launch_fused(call, std::min(items, grid_max), stream, fish_blocks > 0));
         if (pose_frames > 0) FT_CUDA(launch_pose(call, stream));
         ctx->launches += (items > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) + (fish_frames > 0 ? 1 : 0);
         return finish_call(ctx, stream);
@@ -933,12 +935,11 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
                 FT_CUDA(launch_pyramids(reinterpret_cast<const BatchHeader *>(table_dev), pyr_frames, params.nlevels,
                                         pyr_blocks,
                                         stream));
-            FT_CUDA(launch_fisheye(reinterpret_cast<const BatchHeader *>(table_dev), fish_frames, fish_blocks, stream));
-            if (items > 0)
-                FT_CUDA(launch_fused(reinterpret_cast<const BatchHeader *>(table_dev), std::min(items, grid_max),
-                                     stream));
-            if (pose_frames > 0)
-                FT_CUDA(launch_pose(reinterpret_cast<const BatchHeader *>(table_dev), pose_frames, stream));
+            const BatchHeader *hdr = reinterpret_cast<const BatchHeader *>(table_dev);
+            FT_CUDA(launch_fisheye(hdr, fish_frames, fish_blocks, stream, pyr_frames > 0));
+            if (items > 0) FT_CUDA(launch_fused(hdr, std::min(items, grid_max), stream,
+                                                pyr_frames > 0 || (fish_frames > 0 && fish_blocks > 0)));
+            if (pose_frames > 0) FT_CUDA(launch_pose(hdr, pose_frames, stream));
         }
         ctx->launches += (items > 0 ? 1 : 0) + (pyr_frames > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) +
                          (fish_frames > 0 ? 1 : 0);

@@ -530,6 +530,8 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
 
 __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const BatchHeader *__restrict__ hdr)
 {
+    let_next_start();
+    wait_for_previous();
     if ((int)blockIdx.y >= hdr->nframes) return;
     fisheye_run(hdr, hdr->frames[blockIdx.y]);
 }
@@ -537,26 +539,17 @@ __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_kernel(const Batch
 // one frame, its header and descriptor as kernel parameters
 __global__ void __launch_bounds__(kFishThreads, 2) ft_fisheye_one_kernel(const __grid_constant__ FrameCall call)
 {
+    let_next_start();
     fisheye_run(&call.h, call.f);
 }
 
 // Columns are shared out while that still leaves the chip's 152 SMs a block
 // each (about 60 % of a frame's blocks have rows: the overlap).
-void fisheye_launch_config(int nframes, int blocks, cudaStream_t stream, cudaLaunchConfig_t &cfg, cudaLaunchAttribute &cluster)
+int fisheye_splits(int nframes, int blocks)
 {
     int splits = 1;
     while (splits < kFishSplit && 2 * splits * blocks * nframes <= 256) splits *= 2;
-    cfg = {};
-    cfg.gridDim = dim3((unsigned)blocks, (unsigned)nframes, (unsigned)splits);
-    cfg.blockDim = dim3(kFishThreads);
-    cfg.dynamicSmemBytes = kFishSmem;
-    cfg.stream = stream;
-    cluster.id = cudaLaunchAttributeClusterDimension;
-    cluster.val.clusterDim.x = 1;
-    cluster.val.clusterDim.y = 1;
-    cluster.val.clusterDim.z = (unsigned)splits;
-    cfg.attrs = &cluster;
-    cfg.numAttrs = 1;
+    return splits;
 }
 
 }  // namespace
@@ -571,22 +564,22 @@ cudaError_t fisheye_setup()
 
 int fisheye_blocks(int nl) { return (nl + kFishRows - 1) / kFishRows; }
 
-cudaError_t launch_fisheye(const BatchHeader *dev_hdr, int nframes, int blocks, cudaStream_t stream)
+cudaError_t launch_fisheye(const BatchHeader *dev_hdr, int nframes, int blocks, cudaStream_t stream, bool overlap)
 {
     if (nframes <= 0 || blocks <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute cluster;
-    fisheye_launch_config(nframes, blocks, stream, cfg, cluster);
-    return cudaLaunchKernelEx(&cfg, ft_fisheye_kernel, dev_hdr);
+    const unsigned splits = (unsigned)fisheye_splits(nframes, blocks);
+    OverlapLaunch l(dim3((unsigned)blocks, (unsigned)nframes, splits), kFishThreads, kFishSmem, stream, overlap);
+    l.cluster(1, 1, splits);
+    return cudaLaunchKernelEx(&l.cfg, ft_fisheye_kernel, dev_hdr);
 }
 
 cudaError_t launch_fisheye(const FrameCall &call, int blocks, cudaStream_t stream)
 {
     if (blocks <= 0) return cudaSuccess;
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute cluster;
-    fisheye_launch_config(1, blocks, stream, cfg, cluster);
-    return cudaLaunchKernelEx(&cfg, ft_fisheye_one_kernel, call);
+    const unsigned splits = (unsigned)fisheye_splits(1, blocks);
+    OverlapLaunch l(dim3((unsigned)blocks, 1, splits), kFishThreads, kFishSmem, stream, false);
+    l.cluster(1, 1, splits);
+    return cudaLaunchKernelEx(&l.cfg, ft_fisheye_one_kernel, call);
 }
 
 }  // namespace ft

@@ -1018,6 +1018,7 @@ __device__ void stereo_pinhole_item(const BatchHeader &B, const FrameDev &F, int
             hamming_phase(P, F, S, npass, staged, w_a, nrows);
             __syncthreads();
             mark(B, 1);
+            wait_for_previous();                // the levels the refinement reads
             const int nref = S.nref;
             refine_matches(P, F, S, nref);
             __syncthreads();
@@ -1642,6 +1643,7 @@ __device__ __forceinline__ void fused_run(const BatchHeader *hdr, const FrameDev
     // then shared-memory loads instead of dependent global loads
     __shared__ __align__(16) BatchHeader sB;
     __shared__ __align__(16) FrameDev sF;
+    let_next_start();
     if (kOne) {
         copy_param(&sB, hdr, sizeof(BatchHeader));
         copy_param(&sF, one, sizeof(FrameDev));
@@ -1717,6 +1719,7 @@ __device__ __forceinline__ void fused_run(const BatchHeader *hdr, const FrameDev
             }
         }
     }
+    wait_for_previous();
     if (kOne && threadIdx.x == 0) {
         // the last block of the launch leaves the queue and the counters zero
         __threadfence();
@@ -2218,16 +2221,16 @@ cudaError_t fused_occupancy(int *ctas_per_sm)
                                                          sizeof(Smem));
 }
 
-cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stream)
+cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stream, bool overlap)
 {
-    ft_fused_kernel<<<grid, kThreads, sizeof(Smem), stream>>>(dev_hdr);
-    return cudaGetLastError();
+    OverlapLaunch l(dim3((unsigned)grid), kThreads, sizeof(Smem), stream, overlap);
+    return cudaLaunchKernelEx(&l.cfg, ft_fused_kernel, dev_hdr);
 }
 
-cudaError_t launch_fused(const FrameCall &call, int grid, cudaStream_t stream)
+cudaError_t launch_fused(const FrameCall &call, int grid, cudaStream_t stream, bool overlap)
 {
-    ft_fused_one_kernel<<<grid, kThreads, sizeof(Smem), stream>>>(call);
-    return cudaGetLastError();
+    OverlapLaunch l(dim3((unsigned)grid), kThreads, sizeof(Smem), stream, overlap);
+    return cudaLaunchKernelEx(&l.cfg, ft_fused_one_kernel, call);
 }
 
 cudaError_t launch_pose(const FrameCall &call, cudaStream_t stream)

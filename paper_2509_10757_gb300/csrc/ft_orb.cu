@@ -160,6 +160,7 @@ __global__ void __launch_bounds__(kDetThreads, 6) orb_detect_kernel(const OrbHea
     __shared__ uint16_t listed[2][kListCap];                // pairs that passed the compass test: bright, dark
     __shared__ uint16_t corner[2 * kListCap];               // corners of the tile: ring row << 6 | ring column
     __shared__ unsigned n_listed[2];                        // bright | dark << 16, corners
+    let_next_start();
     const OrbHeader &H = *hdr;
     const OrbImage &I = H.images[blockIdx.y];
     const int tile = blockIdx.x;
@@ -425,6 +426,8 @@ __global__ void __launch_bounds__(kOrbSelectThreads) orb_select_kernel(const Orb
     __shared__ int s_n[2];
     const OrbHeader &H = *hdr;
     const int l = blockIdx.x;
+    let_next_start();
+    wait_for_previous();                // the detection's corners
     if (l >= H.nlevels) return;
     const OrbImage &I = H.images[blockIdx.y];
     const OrbLevel &L = I.lv[l];
@@ -569,6 +572,7 @@ __global__ void __launch_bounds__(32 * kDescribeWarps, 7) orb_describe_kernel(co
     const OrbImage &I = H.images[blockIdx.y];
     const int lane = threadIdx.x & 31, wv = threadIdx.x >> 5;
     const int slot = blockIdx.x * kDescribeWarps + wv;
+    wait_for_previous();                // the selection's keypoints
     if (slot >= I.nslots) return;
     int l = 0;
     for (int k = 0; k < H.nlevels; ++k)
@@ -700,12 +704,12 @@ cudaError_t launch_orb(const OrbHeader *dev_hdr, int nimages, int nlevels, int m
         dev_hdr);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    orb_select_kernel<<<dim3((unsigned)nlevels, (unsigned)nimages), kOrbSelectThreads, 0, stream>>>(dev_hdr);
-    e = cudaGetLastError();
+    OverlapLaunch select(dim3((unsigned)nlevels, (unsigned)nimages), kOrbSelectThreads, 0, stream, true);
+    e = cudaLaunchKernelEx(&select.cfg, orb_select_kernel, dev_hdr);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((max(max_slots, 1) + kDescribeWarps - 1) / kDescribeWarps);
-    orb_describe_kernel<<<dim3(blocks, (unsigned)nimages), 32 * kDescribeWarps, 0, stream>>>(dev_hdr);
-    return cudaGetLastError();
+    OverlapLaunch describe(dim3(blocks, (unsigned)nimages), 32 * kDescribeWarps, 0, stream, true);
+    return cudaLaunchKernelEx(&describe.cfg, orb_describe_kernel, dev_hdr);
 }
 
 }  // namespace ft

@@ -125,6 +125,7 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
     PyrRow *tab = reinterpret_cast<PyrRow *>(tile + (kPyrTileRows + 1) * kPyrStride);   // [levels][kPyrRowsPerLevel]
     __shared__ PyrLevelInfo info[FT_MAX_LEVELS + 1];
 
+    let_next_start();
     const int f = (int)(blockIdx.y >> 1), side = (int)(blockIdx.y & 1);
     if (f >= hdr->nframes) return;
     const FrameDev &F = hdr->frames[f];
