@@ -32,7 +32,6 @@ constexpr int kRowSortItems = 4;                    // row-sort work items per p
 constexpr int kPyrThreads = 256;                    // threads per pyramid block
 constexpr int kPyrTileRows = 16;                    // source rows a pyramid block owns
 constexpr int kPyrTileCols = 752;                   // source columns a pyramid block owns (a multiple of 16)
-constexpr int kPyrStride = kPyrTileCols + 16;       // floats per staged row (owned columns + 16)
 constexpr int kPyrRowsPerLevel = 2 * kPyrTileRows;  // output rows of one level in a tile, at most
 
 // Tiles of a pyramid's level 0 (one pyramid block each).

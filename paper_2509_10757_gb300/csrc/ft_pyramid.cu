@@ -10,8 +10,11 @@
 //
 // One block per tile of level 0: kPyrTileRows source rows (plus the next
 // row) by kPyrTileCols source columns (plus the next 16).  The block
-//   1. reads the tile with 16-byte loads and stores it in shared memory as
-//      floats (each source byte is converted once, for every level);
+//   1. reads the tile and stores in shared memory one 32-bit word per source
+//      pixel: its own byte, the next column's, and the same two of the next
+//      row, the four values of the formula, so that an output pixel is one
+//      shared load (a float per pixel took two per source row, and the
+//      shared-memory pipe and the issue slots were both two thirds busy);
 //   2. finds, for every level, the output rows whose upper source row y0
 //      and the output columns whose left source column c0 lie in the tile
 //      (searches over the same FP32 operations as the formula, one lane of
@@ -20,19 +23,21 @@
 //      source-row offsets and vertical weights;
 //   3. gives each thread kPyrCols output columns (x, x + 32, ...) of one
 //      level at a time (all levels' columns in one list, so few threads
-//      idle) and walks those columns' rows in the tile, keeping the
-//      horizontal interpolations of the last bottom source row for the next
-//      output row when it is the next row's top.  The lanes of a warp take
-//      32 neighbouring columns, so the byte stores of a row coalesce.
-// The image's last column and row are repeated past the tile's staged ones
-// where the tile reaches the image's edge, so the formula's clamped c1 and y1
-// are always the staged c0 + 1 and y0 + 1.
+//      idle) and walks those columns' rows in the tile, two columns to a
+//      packed operation.  The lanes of a warp take 32 neighbouring columns,
+//      so the byte stores of a row coalesce.
+// Past the image's last column and row the words hold other bytes (or zero):
+// the formula clamps the source coordinate there, its weight is zero, and zero
+// times any byte is the same zero.
 // Every tile is independent: no block waits for another.
 //
-// A byte b becomes the float b exactly by placing it in the mantissa of 2^23
-// and subtracting 2^23.  Products and sums are single FP32 operations with
-// explicit rounding (a multiply feeding an add is never contracted into a
-// fused multiply-add).  The value v lies in [0, 255] up to rounding (a
+// A byte b placed in the mantissa of 2^23 is the float 2^23 + b, and
+// fma(2^23 + b, w, -2^23 w) rounds the exact b w once: the product b w as one
+// FP32 multiplication gives it, without the conversion.  The vertical
+// products are fused multiply-adds of -0.0 (a x b - 0 rounds as a x b) that
+// the compiler does not know to be zero: a packed multiply that feeds a packed
+// add it contracts even when both carry a rounding mode.  Sums are single
+// packed FP32 additions.  The value v lies in [0, 255] up to rounding (a
 // convex combination of bytes), so adding 1.5 * 2^23 rounds it to the
 // nearest integer, ties to even, and the low mantissa byte is the result.
 // Levels therefore equal the per-pixel formula bit for bit.
@@ -45,7 +50,8 @@
 namespace ft {
 namespace {
 
-constexpr int kPyrCols = FT_PYR_COLS;        // output columns per thread (32 apart)
+constexpr int kPyrCols = FT_PYR_COLS;        // output columns per thread (32 apart), an even count
+constexpr int kPyrFillRows = 4;              // tile rows a thread fills at a time
 
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b); }
@@ -64,6 +70,13 @@ __device__ __forceinline__ f32x2 f2_pack(unsigned lo, unsigned hi)
 __device__ __forceinline__ void f2_unpack(f32x2 a, unsigned &lo, unsigned &hi)
 {
     asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(a));
+}
+__device__ __forceinline__ f32x2 f2_dup(float a) { return f2_pack(__float_as_uint(a), __float_as_uint(a)); }
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
 }
 __device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b)
 {
@@ -120,9 +133,9 @@ struct alignas(16) PyrRow {
 
 __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchHeader *__restrict__ hdr)
 {
-    extern __shared__ float4 pyr_smem[];
-    float *tile = reinterpret_cast<float *>(pyr_smem);                       // [kPyrTileRows + 1][kPyrStride]
-    PyrRow *tab = reinterpret_cast<PyrRow *>(tile + (kPyrTileRows + 1) * kPyrStride);   // [levels][kPyrRowsPerLevel]
+    extern __shared__ uint4 pyr_smem[];
+    unsigned *tile = reinterpret_cast<unsigned *>(pyr_smem);                 // [kPyrTileRows][kPyrTileCols]
+    PyrRow *tab = reinterpret_cast<PyrRow *>(tile + kPyrTileRows * kPyrTileCols);       // [levels][kPyrRowsPerLevel]
     __shared__ PyrLevelInfo info[FT_MAX_LEVELS + 1];
 
     let_next_start();
@@ -139,25 +152,33 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
     const int Y0 = ((int)blockIdx.x / ntx) * kPyrTileRows, X0 = ((int)blockIdx.x % ntx) * kPyrTileCols;
     const int tid = (int)threadIdx.x;
 
-    // 1. the tile as floats: source rows Y0 .. Y0 + nr - 1, bytes X0 .. X0 +
-    // nb - 1 (16-byte chunks; W rounded up to 16 is within the pitch)
-    const int nr = min(kPyrTileRows + 1, H - Y0);
-    const int nch = min(kPyrStride, ((W + 15) & ~15) - X0) >> 4;
-    for (int k = tid; k < nr * nch; k += kPyrThreads) {
-        const int r = k / nch, c = k - r * nch;
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(src + (size_t)(Y0 + r) * sp + X0 + 16 * c));
-        float4 *d = reinterpret_cast<float4 *>(tile + r * kPyrStride + 16 * c);
-        const unsigned wd[4] = {v.x, v.y, v.z, v.w};
-        const f32x2 neg = f2_pack(__float_as_uint(-kTwo23), __float_as_uint(-kTwo23));
+    // 1. the tile's words: four columns (one 4-byte word) of kPyrFillRows rows
+    // per thread at a time, each row's bytes joined with the next row's (W
+    // rounded up to 16 is within the pitch)
+    const int nr = min(kPyrTileRows, H - Y0);
+    const int left = ((W + 15) & ~15) - X0;          // bytes of a row from the tile on
+    const int nw = min(kPyrTileCols, left) >> 2;
+    const unsigned inv = (1u << 20) / (unsigned)nw + 1u;      // k / nw = k inv >> 20 for k nw < 2^20
+    for (int k = tid; k < nw * (kPyrTileRows / kPyrFillRows); k += kPyrThreads) {
+        const int g = (int)(((unsigned)k * inv) >> 20), c = k - g * nw;
+        const int r0 = g * kPyrFillRows;
+        if (r0 >= nr) break;
+        const uint8_t *p = src + X0 + 4 * c;
+        const bool more = 4 * c + 4 < left;
+        unsigned a[kPyrFillRows + 1], t[kPyrFillRows + 1];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            unsigned a, b, c2, e;
-            f2_unpack(f2_add(f2_pack(__byte_perm(wd[j], kExp23, 0x7440), __byte_perm(wd[j], kExp23, 0x7441)), neg),
-                      a, b);
-            f2_unpack(f2_add(f2_pack(__byte_perm(wd[j], kExp23, 0x7442), __byte_perm(wd[j], kExp23, 0x7443)), neg),
-                      c2, e);
-            d[j] = make_float4(__uint_as_float(a), __uint_as_float(b), __uint_as_float(c2), __uint_as_float(e));
+        for (int i = 0; i <= kPyrFillRows; ++i) {
+            const uint8_t *q = p + (size_t)min(Y0 + r0 + i, H - 1) * sp;
+            a[i] = __ldg(reinterpret_cast<const unsigned *>(q));
+            t[i] = more ? __ldg(reinterpret_cast<const unsigned *>(q) + 1) : 0u;
         }
+#pragma unroll
+        for (int i = 0; i <= kPyrFillRows; ++i) t[i] = __byte_perm(a[i], t[i], 0x0043);     // columns 3, 4
+#pragma unroll
+        for (int i = 0; i < kPyrFillRows; ++i)
+            *reinterpret_cast<uint4 *>(tile + (r0 + i) * kPyrTileCols + 4 * c) =
+                make_uint4(__byte_perm(a[i], a[i + 1], 0x5410), __byte_perm(a[i], a[i + 1], 0x6521),
+                           __byte_perm(a[i], a[i + 1], 0x7632), __byte_perm(t[i], t[i + 1], 0x5410));
     }
     // 2. the rows and columns of every level whose source lies in the tile:
     // lane l - 1 of the last warp takes level l (nlevels <= 16 <= 32), while
@@ -197,16 +218,6 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
         if (l == nl - 1 || (nl <= 1 && lane == 0)) info[nl].unit0 = nl <= 1 ? 0 : end;   // end of the unit list
     }
     __syncthreads();
-    // the image's last column and row repeated past the tile's last staged
-    // ones where the tile reaches the image's edge, so that the source
-    // column c0 + 1 and row y0 + 1 always hold the formula's c1 and y1
-    // (both clamped to the image)
-    const int cl = W - 1 - X0;                       // last column, tile-local (< kPyrTileCols if owned)
-    if (cl < kPyrTileCols)
-        for (int r = tid; r < nr; r += kPyrThreads) tile[r * kPyrStride + cl + 1] = tile[r * kPyrStride + cl];
-    if (nr <= kPyrTileRows)                          // the tile holds the image's last row, nr - 1
-        for (int c = tid; c < kPyrStride; c += kPyrThreads)
-            tile[nr * kPyrStride + c] = tile[(nr - 1) * kPyrStride + (cl < kPyrTileCols ? min(c, cl) : c)];
     for (int k = tid; k < (nl - 1) * kPyrRowsPerLevel; k += kPyrThreads) {
         const int l = 1 + k / kPyrRowsPerLevel, i = k - (l - 1) * kPyrRowsPerLevel;
         if (i >= info[l].nrows) continue;
@@ -214,7 +225,7 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
         const float ys = pyr_src(y, fdiv((float)H, (float)lh[l]), H);
         const int y0 = f2i(floorf(ys));
         PyrRow e;
-        e.r0 = (unsigned)((y0 - Y0) * kPyrStride);
+        e.r0 = (unsigned)((y0 - Y0) * kPyrTileCols);
         e.fy = fsub(ys, (float)y0);
         e.gy = fsub(1.0f, e.fy);
         e.doff = (unsigned)(y * info[l].dp);
@@ -224,6 +235,7 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
     // 3. one unit (kPyrCols output columns 32 apart) of one level per thread
     // at a time, down the level's rows in this tile
     const int units = info[nl].unit0;
+    const f32x2 minus0 = f2_dup(__uint_as_float(0x80000000u | ((unsigned)nl >> 8)));     // nl <= 16: -0.0
     int l = 1;
     for (int u = tid; u < units; u += kPyrThreads) {
         while (u >= info[l + 1].unit0) ++l;          // units are in level order; u only grows
@@ -247,8 +259,8 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
         if (x0 >= xs_end) continue;
         const float sx = info[l].sx;
         bool st[kPyrCols];
-        const float *P[kPyrCols];
-        float fx[kPyrCols], gx[kPyrCols], hb[kPyrCols], ht[kPyrCols];
+        const unsigned *P[kPyrCols];
+        float fx[kPyrCols], gx[kPyrCols];
 #pragma unroll
         for (int j = 0; j < kPyrCols; ++j) {
             st[j] = x0 + 32 * j < xs_end;
@@ -256,33 +268,40 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
             const int c0 = f2i(floorf(xs));
             fx[j] = fsub(xs, (float)c0);
             gx[j] = fsub(1.0f, fx[j]);
-            // source columns c0 and c0 + 1; the next row lies kPyrStride floats further
             P[j] = tile + (c0 - X0);
-            hb[j] = 0.0f;
+        }
+        // the weights of a pair of columns, and -2^23 times them
+        f32x2 fx2[kPyrCols / 2], gx2[kPyrCols / 2], nf2[kPyrCols / 2], ng2[kPyrCols / 2];
+#pragma unroll
+        for (int q = 0; q < kPyrCols / 2; ++q) {
+            const float f0 = fx[2 * q], f1 = fx[2 * q + 1], g0 = gx[2 * q], g1 = gx[2 * q + 1];
+            fx2[q] = f2_pack(__float_as_uint(f0), __float_as_uint(f1));
+            gx2[q] = f2_pack(__float_as_uint(g0), __float_as_uint(g1));
+            nf2[q] = f2_pack(__float_as_uint(fmul(f0, -kTwo23)), __float_as_uint(fmul(f1, -kTwo23)));
+            ng2[q] = f2_pack(__float_as_uint(fmul(g0, -kTwo23)), __float_as_uint(fmul(g1, -kTwo23)));
         }
         uint8_t *o0 = out + x0;
-        unsigned cr1 = 0xffffffffu;
         for (int i = 0; i < n; ++i) {
             const PyrRow e = T[i];
-            if (e.r0 != cr1) {                        // else the previous bottom row is this top row
-#pragma unroll
-                for (int j = 0; j < kPyrCols; ++j) {
-                    const float *a = P[j] + e.r0;
-                    hb[j] = fadd(fmul(a[0], gx[j]), fmul(a[1], fx[j]));
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < kPyrCols; ++j) {
-                const float *a = P[j] + e.r0 + kPyrStride;
-                ht[j] = hb[j];
-                hb[j] = fadd(fmul(a[0], gx[j]), fmul(a[1], fx[j]));
-            }
-            cr1 = e.r0 + kPyrStride;
+            const f32x2 fy2 = f2_dup(e.fy), gy2 = f2_dup(e.gy);
             uint8_t *o = o0 + e.doff;
+            unsigned w4[kPyrCols];
 #pragma unroll
-            for (int j = 0; j < kPyrCols; ++j) {
-                const float v = fadd(fmul(ht[j], e.gy), fmul(hb[j], e.fy));
-                if (st[j]) o[32 * j] = (uint8_t)__float_as_uint(fadd(v, kRound23));
+            for (int j = 0; j < kPyrCols; ++j) w4[j] = P[j][e.r0];
+#pragma unroll
+            for (int q = 0; q < kPyrCols / 2; ++q) {
+                const unsigned wa = w4[2 * q], wb = w4[2 * q + 1];
+                const f32x2 t0 = f2_pack(__byte_perm(wa, kExp23, 0x7440), __byte_perm(wb, kExp23, 0x7440));
+                const f32x2 t1 = f2_pack(__byte_perm(wa, kExp23, 0x7441), __byte_perm(wb, kExp23, 0x7441));
+                const f32x2 b0 = f2_pack(__byte_perm(wa, kExp23, 0x7442), __byte_perm(wb, kExp23, 0x7442));
+                const f32x2 b1 = f2_pack(__byte_perm(wa, kExp23, 0x7443), __byte_perm(wb, kExp23, 0x7443));
+                const f32x2 top = f2_add(f2_fma(t0, gx2[q], ng2[q]), f2_fma(t1, fx2[q], nf2[q]));
+                const f32x2 bot = f2_add(f2_fma(b0, gx2[q], ng2[q]), f2_fma(b1, fx2[q], nf2[q]));
+                const f32x2 v = f2_add(f2_fma(top, gy2, minus0), f2_fma(bot, fy2, minus0));
+                unsigned va, vb;
+                f2_unpack(f2_add(v, f2_dup(kRound23)), va, vb);
+                if (st[2 * q]) o[64 * q] = (uint8_t)va;
+                if (st[2 * q + 1]) o[64 * q + 32] = (uint8_t)vb;
             }
         }
     }
@@ -291,7 +310,7 @@ __global__ void __launch_bounds__(kPyrThreads, 4) ft_pyramid_kernel(const BatchH
 // Dynamic shared memory of the pyramid kernel for nlevels levels.
 size_t pyr_smem_bytes(int nlevels)
 {
-    return sizeof(float) * (kPyrTileRows + 1) * kPyrStride +
+    return sizeof(unsigned) * kPyrTileRows * kPyrTileCols +
            sizeof(PyrRow) * (size_t)(nlevels > 1 ? nlevels - 1 : 1) * kPyrRowsPerLevel;
 }
 
