@@ -111,17 +111,6 @@ __device__ __forceinline__ void load_circle(const unsigned (*pe)[kHalfW], const 
     }
 }
 
-// Appends the lanes' flagged values to a list in shared memory.
-__device__ __forceinline__ void list_append(uint16_t *list, unsigned *count, bool flag, int value, int lane)
-{
-    const unsigned m = __ballot_sync(kFull, flag);
-    if (m == 0u) return;
-    unsigned at = 0;
-    if (lane == 0) at = atomicAdd(count, (unsigned)__popc(m));
-    at = __shfl_sync(kFull, at, 0) + (unsigned)__popc(m & ((1u << lane) - 1u));
-    if (flag) list[at] = (uint16_t)value;
-}
-
 // One block per tile of 62 x 30 pixels of a level, so that the tile with its
 // one-pixel suppression ring is 64 x 32 pixels: a warp takes whole rows, a
 // lane two adjacent pixels, every shared-memory row read is conflict-free and
@@ -150,7 +139,12 @@ __device__ __forceinline__ void list_append(uint16_t *list, unsigned *count, boo
 // What bounds the kernel is instruction issue, and a pixel of footage is
 // rarely a corner: 128 images of 752x480 footage-like content (2.4 % corners;
 // 14 % of the pixels pass the test), 143 M pixels, took 1176 us with every
-// pair's arcs in both polarities, 975 us with the test on 32 x 32 tiles.
+// pair's arcs in both polarities, 975 us with the test on 32 x 32 tiles,
+// 743 us on these.  A warp then takes its rows of a phase together, their loads
+// in flight at once and one reservation for all its listed pairs: 648 us (79 %
+// of the shared-memory wavefronts, 77 % of the issue slots).  62 x 62 tiles of
+// 512 threads load fewer halo rows but cover more outside the small levels:
+// extraction 853 us against 808.
 __global__ void __launch_bounds__(kDetThreads, 6) orb_detect_kernel(const OrbHeader *__restrict__ hdr)
 {
     __shared__ __align__(16) unsigned pe[kHaloRows][kHalfW];
@@ -195,12 +189,19 @@ __global__ void __launch_bounds__(kDetThreads, 6) orb_detect_kernel(const OrbHea
         const bool wide = x0 < kOrbHalo || x0 + kOrbTileW + kOrbHalo > W;    // some columns lie outside
         const int pc = min(max(p, 0), (W - 1) & ~3);         // the word that is read
         const unsigned have = (unsigned)(W - pc);            // pixels of the level from there
+        constexpr int kRows = (kHaloRows + kDetWarps - 1) / kDetWarps;      // of a warp, all in flight at once
+        unsigned word[kRows];
 #pragma unroll
-        for (int s = 0; s < (kHaloRows + kDetWarps - 1) / kDetWarps; ++s) {
+        for (int s = 0; s < kRows; ++s) {
+            const int r = min(warp + s * kDetWarps, kHaloRows - 1);
+            const uint8_t *row = img + (size_t)clampi(y0 - kOrbHalo + r, 0, Hl - 1) * pitch;
+            word[s] = lane < 18 ? __ldg(reinterpret_cast<const unsigned *>(row + pc)) : 0u;
+        }
+#pragma unroll
+        for (int s = 0; s < kRows; ++s) {
             const int r = warp + s * kDetWarps;
             if (r >= kHaloRows) break;                       // the whole warp
-            const uint8_t *row = img + (size_t)clampi(y0 - kOrbHalo + r, 0, Hl - 1) * pitch;
-            unsigned w = lane < 18 ? __ldg(reinterpret_cast<const unsigned *>(row + pc)) : 0u;
+            unsigned w = word[s];
             if (wide) {
                 // bytes past the level's last pixel repeat it; words before
                 // the first or past the last pixel repeat that one
@@ -229,37 +230,50 @@ __global__ void __launch_bounds__(kDetThreads, 6) orb_detect_kernel(const OrbHea
     const unsigned th2 = (unsigned)(256 + th) * 0x00010001u;
     const int px = x0 - 1 + 2 * lane;
     const bool in0 = px >= E && px < W - E, in1 = px + 1 >= E && px + 1 < W - E;
+    constexpr int kRows = kRingRows / kDetWarps;            // of a warp
+    unsigned mb[kRows], md[kRows], n2 = 0u;
 #pragma unroll
-    for (int s = 0; s < kRingRows / kDetWarps; ++s) {
+    for (int s = 0; s < kRows; ++s) {
         const int ry = warp + s * kDetWarps, py = y0 - 1 + ry;
         key[ry][lane] = 0u;
-        if (py < E || py >= Hl - E) continue;               // the whole warp
         const unsigned c = po[ry + 3][lane + 1], up = po[ry][lane + 1], dn = po[ry + 6][lane + 1];
         const unsigned lf = pe[ry + 3][lane], rt = pe[ry + 3][lane + 3];
         // the best a corner could score, + 256 in each lane (the lanes stay
         // in [1, 511]); above t + 256 in one of them?
         const unsigned br = vmin2(vmax2(up, dn), vmax2(lf, rt)) + 0x01000100u - c;
         const unsigned dk = c + 0x01000100u - vmax2(vmin2(up, dn), vmin2(lf, rt));
-        const bool in = in0 || in1;
-        const bool pb = in && vmax2(br, th2) != th2, pd = in && vmax2(dk, th2) != th2;
-        const unsigned mb = __ballot_sync(kFull, pb), md = __ballot_sync(kFull, pd);
-        if ((mb | md) == 0u) continue;
-        // both lists' counters in one word (each stays below 2^16)
+        const bool in = (in0 || in1) && py >= E && py < Hl - E;
+        mb[s] = __ballot_sync(kFull, in && vmax2(br, th2) != th2);
+        md[s] = __ballot_sync(kFull, in && vmax2(dk, th2) != th2);
+        n2 += (unsigned)__popc(mb[s]) | (unsigned)__popc(md[s]) << 16;
+    }
+    if (n2 != 0u) {
+        // both lists' counters in one word (each stays below 2^16), one
+        // reservation for all the warp's rows
         unsigned at = 0;
-        if (lane == 0) at = atomicAdd(&n_listed[0], (unsigned)__popc(mb) | (unsigned)__popc(md) << 16);
+        if (lane == 0) at = atomicAdd(&n_listed[0], n2);
         at = __shfl_sync(kFull, at, 0);
         const unsigned below = (1u << lane) - 1u;
-        const uint16_t q = (uint16_t)(ry * kRingPairs + lane);
-        if (pb) listed[0][(at & 0xffffu) + __popc(mb & below)] = q;
-        if (pd) listed[1][(at >> 16) + __popc(md & below)] = q;
+        uint16_t *lb = listed[0] + (at & 0xffffu), *ld = listed[1] + (at >> 16);
+#pragma unroll
+        for (int s = 0; s < kRows; ++s) {
+            const uint16_t q = (uint16_t)((warp + s * kDetWarps) * kRingPairs + lane);
+            if (mb[s] >> lane & 1u) lb[__popc(mb[s] & below)] = q;
+            if (md[s] >> lane & 1u) ld[__popc(md[s] & below)] = q;
+            lb += __popc(mb[s]);
+            ld += __popc(md[s]);
+        }
     }
     // horizontal binomial sums (1 4 6 4 1) of halo rows 2 .. 35, output
     // columns 2k and 2k + 1 (taps at halo columns 2k + 2 .. 2k + 7)
-    for (int r = warp; r < kOrbTileH + 4; r += kDetWarps)
-        if (lane < kOrbTileW / 2) {
+#pragma unroll
+    for (int s = 0; s < (kOrbTileH + 4 + kDetWarps - 1) / kDetWarps; ++s) {
+        const int r = warp + s * kDetWarps;
+        if (r < kOrbTileH + 4 && lane < kOrbTileW / 2) {
             const unsigned *e = pe[r + 2], *o = po[r + 2];
             hs[r][lane] = e[lane + 1] + 4u * o[lane + 1] + 6u * e[lane + 2] + 4u * o[lane + 2] + e[lane + 3];
         }
+    }
     __syncthreads();
     // the listed pairs' arcs; a pixel is a corner of one polarity at most (9 of
     // 16 circle pixels each), so no key is written and no corner listed twice
@@ -290,8 +304,16 @@ __global__ void __launch_bounds__(kDetThreads, 6) orb_detect_kernel(const OrbHea
         __syncwarp();
         // the tile's own corners (not its ring's)
         const bool own = ry >= 1 && ry <= kOrbTileH;
-        list_append(corner, &n_listed[1], k0 && own && h > 0, ry << 6 | 2 * h, lane);
-        list_append(corner, &n_listed[1], k1 && own && h < kRingPairs - 1, ry << 6 | (2 * h + 1), lane);
+        k0 = k0 && own && h > 0;
+        k1 = k1 && own && h < kRingPairs - 1;
+        const unsigned m0 = __ballot_sync(kFull, k0), m1 = __ballot_sync(kFull, k1);
+        if ((m0 | m1) == 0u) continue;
+        unsigned at = 0;
+        if (lane == 0) at = atomicAdd(&n_listed[1], (unsigned)(__popc(m0) + __popc(m1)));
+        at = __shfl_sync(kFull, at, 0);
+        const unsigned below = (1u << lane) - 1u;
+        if (k0) corner[at + __popc(m0 & below)] = (uint16_t)(ry << 6 | 2 * h);
+        if (k1) corner[at + __popc(m0) + __popc(m1 & below)] = (uint16_t)(ry << 6 | (2 * h + 1));
     }
     // vertical sums: a warp's four rows (two of the last warp's) from eight
     // rows of horizontal sums
