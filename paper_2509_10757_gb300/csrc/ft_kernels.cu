@@ -201,7 +201,7 @@ struct SmemStereo {
         PatchBuf patch[kSadBufs];      // (a strip with a second pass stages its window again)
     } u;
     RefineJob ref[kThreads];
-    int sad[2][kSadChunk][12];         // this round's and the last one's
+    int sad[2][kShifts][kSadChunk];    // this round's and the last one's
     int warp_sums[kWarps];
     int nref;
 };
@@ -727,22 +727,28 @@ __device__ __forceinline__ void refine_copy(const FrameDev &F, SmemStereo &S, in
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// Adds this thread's patch row of round r to the 11 SADs of its match.
+// Adds this thread's patch row of round r to the 11 SADs of its match.  The
+// pixels go in pairs: |p - q| = 2 max(p, q) - p - q, so a pair costs one
+// instruction (an add of the centres' difference and the larger of the lanes;
+// the larger is never below the right pixel, so sums of lanes do not borrow)
+// and the two other sums come from dot products, the right one sliding from
+// shift to shift.  (A difference and an absolute sum per pixel before: 64
+// frames 98.0 us, now 96.2; 32 frames of 1920x1080 507 and 501.)
 __device__ __forceinline__ void refine_row(SmemStereo &S, int r, int nref)
 {
     constexpr int kRows = 2 * kW + 1;
     static_assert(kSadChunk * kRows <= kThreads, "one patch row a thread");
     const int nc = min(kSadChunk, nref - r * kSadChunk);
     const PatchBuf &B = S.u.patch[r % kSadBufs];
-    const int dy = threadIdx.x / kSadChunk, m = threadIdx.x - dy * kSadChunk;
-    if (dy < kRows && m < nc) {
-        const RefineJob &J = S.ref[r * kSadChunk + m];
+    const int dy = threadIdx.x / kSadChunk, mm = threadIdx.x - dy * kSadChunk;
+    if (dy < kRows && mm < nc) {
+        const RefineJob &J = S.ref[r * kSadChunk + mm];
         const int ol = (J.ul - kW) & 15, orr = (J.ur0 - kL - kW) & 15;
         // the rows as 32-bit words; byte b of a row is byte (o + b) of its chunks
-        const unsigned *ql = reinterpret_cast<const unsigned *>(B.l[m][dy]) + (ol >> 2);
-        const unsigned *qr = reinterpret_cast<const unsigned *>(B.r[m][dy]) + (orr >> 2);
-        const unsigned *qc = reinterpret_cast<const unsigned *>(B.r[m][kW]) + (orr >> 2);
-        const unsigned *qlc = reinterpret_cast<const unsigned *>(B.l[m][kW]) + (ol >> 2);
+        const unsigned *ql = reinterpret_cast<const unsigned *>(B.l[mm][dy]) + (ol >> 2);
+        const unsigned *qr = reinterpret_cast<const unsigned *>(B.r[mm][dy]) + (orr >> 2);
+        const unsigned *qc = reinterpret_cast<const unsigned *>(B.r[mm][kW]) + (orr >> 2);
+        const unsigned *qlc = reinterpret_cast<const unsigned *>(B.l[mm][kW]) + (ol >> 2);
         const int sl = 8 * (ol & 3), sr = 8 * (orr & 3);
         // realigned words: byte b of the row is byte b & 3 of word b >> 2
         unsigned wl[3], wr[6], wc[4];
@@ -752,22 +758,44 @@ __device__ __forceinline__ void refine_row(SmemStereo &S, int r, int nref)
         for (int k = 0; k < 6; ++k) wr[k] = __funnelshift_r(qr[k], qr[k + 1], sr);
 #pragma unroll
         for (int k = 1; k < 4; ++k) wc[k] = __funnelshift_r(qc[k], qc[k + 1], sr);
-        // left row minus the left centre, right row, and the centres of the
-        // 11 right patches (bytes 5..15 of the right centre row)
+        // pairs of left pixels, and of right pixels that start at an even or
+        // an odd byte, in 16-bit lanes; the left row's sixth pair is its last
+        // pixel and a value below all others
+        unsigned a[6], e[11], o[10];
+#pragma unroll
+        for (int i = 0; i < 6; ++i) a[i] = __byte_perm(wl[i >> 1], 0u, i & 1 ? 0x4342 : 0x4140);
+        a[5] = (a[5] & 0xffffu) | 0x8ad00000u;              // -30000 in the upper lane
+#pragma unroll
+        for (int i = 0; i < 11; ++i) e[i] = __byte_perm(wr[i >> 1], 0u, i & 1 ? 0x4342 : 0x4140);
+#pragma unroll
+        for (int i = 0; i < 10; ++i)
+            o[i] = i & 1 ? __byte_perm(__funnelshift_r(wr[i >> 1], wr[(i >> 1) + 1], 24), 0u, 0x4140)
+                         : __byte_perm(wr[i >> 1], 0u, 0x4241);
         const int cl = (int)((__funnelshift_r(qlc[1], qlc[2], sl) >> 8) & 0xff);
-        int lc[2 * kW + 1], rv[kStripW], cr[kShifts];
+        // minus the sums of the left row (centred) and of the shift's right
+        // pixels, which slide by one
+        int minus = 11 * cl;
 #pragma unroll
-        for (int b = 0; b < 2 * kW + 1; ++b) lc[b] = (int)((wl[b >> 2] >> (8 * (b & 3))) & 0xff) - cl;
-#pragma unroll
-        for (int b = 0; b < kStripW; ++b) rv[b] = (wr[b >> 2] >> (8 * (b & 3))) & 0xff;
-#pragma unroll
-        for (int k = 0; k < kShifts; ++k) cr[k] = (wc[(k + kW) >> 2] >> (8 * ((k + kW) & 3))) & 0xff;
+        for (int k = 0; k < 3; ++k) {
+            const int w = k < 2 ? (int)0xffffffff : 0x00ffffff;              // -1 per byte
+            asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(minus) : "r"(wl[k]), "r"(w));
+            asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(minus) : "r"(wr[k]), "r"(w));
+        }
 #pragma unroll
         for (int k = 0; k < kShifts; ++k) {
-            int s = 0;
+            const int c = (int)__byte_perm(wc[(k + kW) >> 2], 0u, 0x4440 + ((k + kW) & 3));
+            const unsigned c2 = __byte_perm((unsigned)(c - cl), 0u, 0x1010);
+            const unsigned *b = k & 1 ? o + (k >> 1) : e + (k >> 1);
+            unsigned m[6];
 #pragma unroll
-            for (int dx = 0; dx < 2 * kW + 1; ++dx) s = __sad(lc[dx] + cr[k], rv[k + dx], s);
-            atomicAdd(&S.sad[r & 1][m][k], s);
+            for (int i = 0; i < 5; ++i) m[i] = __viaddmax_s16x2(a[i], c2, b[i]);
+            m[5] = __viaddmax_s16x2(a[5], c2, b[5] & 0xffffu);
+            const unsigned sum = (m[0] + m[1] + m[2]) + (m[3] + m[4] + m[5]);
+            atomicAdd(&S.sad[r & 1][k][mm], (int)__dp2a_lo(sum, 0x0202u, (unsigned)(minus - 11 * c)));
+            if (k + 1 < kShifts) {
+                const unsigned t = __byte_perm(wr[k >> 2], wr[(k + 11) >> 2], 0x0000 + (k & 3) + ((4 + ((k + 11) & 3)) << 4));
+                asm("dp4a.u32.s32 %0, %1, %2, %0;" : "+r"(minus) : "r"(t), "r"(0xff01));     // + the first, - the next
+            }
         }
     }
 }
@@ -781,8 +809,8 @@ __device__ __forceinline__ void refine_finish(const DevParams &P, const FrameDev
         int sad[kShifts];
 #pragma unroll
         for (int k = 0; k < kShifts; ++k) {
-            sad[k] = S.sad[r & 1][m][k];
-            S.sad[r & 1][m][k] = 0;
+            sad[k] = S.sad[r & 1][k][m];
+            S.sad[r & 1][k][m] = 0;
         }
         // (the neighbours of the minimum are carried along: no dynamic index)
         int kb = 0, lo = 0, best = sad[0], hi = sad[1];
@@ -829,7 +857,7 @@ __device__ void refine_matches(const DevParams &P, const FrameDev &F, SmemStereo
 {
     const int tid = threadIdx.x, last = tid - (kThreads - 32);
     static_assert(kSadChunk <= 32 && kSadBufs == 3, "a warp finishes a round; two rounds of copies in flight");
-    for (int q = tid; q < 2 * kSadChunk * 12; q += kThreads) (&S.sad[0][0][0])[q] = 0;
+    for (int q = tid; q < 2 * kShifts * kSadChunk; q += kThreads) (&S.sad[0][0][0])[q] = 0;
     refine_copy(F, S, 0, nref);
     refine_copy(F, S, 1, nref);
     const int rounds = (nref + kSadChunk - 1) / kSadChunk;
