@@ -519,8 +519,9 @@ ft_status ft_track_batch(ft_ctx *ctx, void *stream, const ft_params *params, con
 
 /* Time candidate launch shapes on this batch (iters runs each) and keep the
  * fastest for the batch's bucket; *best receives it (may be NULL).  The
- * candidates: strip rows 16/32/64, search tile 256/512/1024, every count of CTAs per SM up to the resident maximum, and the
- * search in one pass or two halves. */
+ * candidates: strip rows 16/32/64, search tile 256/512/1024, every count of
+ * CTAs per SM up to the resident maximum, and the search in one pass or two
+ * halves. */
 ft_status ft_autotune(ft_ctx *ctx, void *stream, const ft_params *params, const ft_batch *batch,
                       int iters, ft_tuning *best);
 

@@ -1,13 +1,16 @@
 // ft_internal.h -- structures shared by the library's host and device code.
 //
-// One persistent kernel runs every entry point.  The host writes a "batch
-// table" (header, per-frame descriptors, per-kind work prefixes, zeroed
-// counters) into pinned memory and copies it into the context's arena with
-// one cudaMemcpyAsync; the kernel's CTAs then pull work items from a queue
-// (an atomic head counter) in a fixed order: grid builds, stereo items,
-// search items, resolve items.  An item waits only on items that sit before
-// it in the queue, so the queue drains without deadlock whatever the number
-// of resident CTAs.
+// One persistent kernel runs the index, pinhole stereo, search and resolve
+// work of every entry point; pyramids, fisheye matching and pose optimization
+// are kernels before and after it, and extraction has three of its own.  The
+// host writes a "batch table" (header, per-frame descriptors, per-kind work
+// prefixes, zeroed counters) into pinned memory and copies it to the slot's
+// device table; a call of one frame passes its header and descriptor as kernel
+// parameters instead.  The fused kernel's CTAs pull work items from a queue (an
+// atomic head counter) in a fixed order: row sorts and grid builds, stereo
+// items, search items, resolve items.  An item waits only on items that sit
+// before it in the queue, so the queue drains without deadlock whatever the
+// number of resident CTAs.
 #pragma once
 
 #include <cstddef>

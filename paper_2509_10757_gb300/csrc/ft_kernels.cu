@@ -7,20 +7,21 @@
 //              section IV-E; grid reading 64x48), also a counting sort.
 //   K_STEREO   pinhole: one horizontal strip of image rows.  The CTA stages
 //              the row-sorted right keypoints that can reach the strip in
-//              shared memory, then runs three CTA-wide phases so that every
-//              memory latency is paid once per phase, not once per keypoint:
-//              (1) one thread per left keypoint: band Hamming search over the
-//              staged candidates (kernel 1 of section IV-C); (2) the 11x11
-//              left patches and 11x21 right strips of all matches gathered
-//              into shared memory; (3) one thread per (match, shift): SAD of
-//              centre-subtracted patches, then per match the best shift,
-//              parabola, disparity and depth (kernel 2 of section IV-C).  The
-//              frame's last strip runs the median rejection.
+//              shared memory, then (1) a few lanes per left keypoint search
+//              the staged candidates of its band (kernel 1 of section IV-C);
+//              (2) rounds of matches: the 11x11 left patches and 11x21 right
+//              strips of the next two rounds on their way into shared memory
+//              while one thread per (match, patch row) adds its row to the SADs
+//              of centre-subtracted patches and a warp finishes the round
+//              before (best shift, parabola, disparity and depth: kernel 2 of
+//              section IV-C).  The frame's last strip runs the median rejection.
 //              (Fisheye frames' brute force is a kernel of its own:
 //              ft_fisheye.cu.)
 //   K_SEARCH   one tile of map points, one thread each: frustum test, FP32
-//              projection, predicted level, grid-window gather, top-2 Hamming,
-//              ratio test; accepted claims go to an atomicMin per keypoint.
+//              projection, predicted level, scan of the grid window's packed
+//              places on chip; a warp pools its points' candidates for the
+//              exact tests and the Hamming distances; top-2 and ratio test;
+//              accepted claims go to an atomicMin per keypoint.
 //              A frame whose search is split around its stereo step scans its
 //              candidates before waiting for the stereo step and applies the
 //              stereo consistency after it, in the same item.
@@ -865,8 +866,8 @@ __device__ __forceinline__ void refine_finish(const DevParams &P, const FrameDev
 // the next two rounds on their way while a round is summed and the last
 // warp finishes the round before it; one block-wide synchronization a round.
 // What bounds a round is the latency of its scattered rows: rounds of 64
-// matches that waited for their own copies took 15 us a strip of 112
-// matches (64 frames, 3 blocks an SM), these 10 us.
+// matches that waited for their own copies took 15.2 us a strip of 112
+// matches (64 frames, 3 blocks an SM), these 12.5 us, 12 with paired pixels.
 __device__ void refine_matches(const DevParams &P, const FrameDev &F, SmemStereo &S, int nref)
 {
     const int tid = threadIdx.x, last = tid - (kThreads - 32);
@@ -1797,8 +1798,9 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_one_ker
 // What bounds it is the serial chain of a frame's Gauss-Newton steps (up to
 // 40), so one frame gets a cluster of kPoseCtas blocks with one warp per
 // scheduler instead of one block with four: 512 threads on one SM spent half
-// of a 3.2 us step issuing the observations' 27 sums.  Every block keeps its threads' observations on chip; each warp reduce-scatters
-// its 27 sums (lane q ends with sum q) and writes them to all blocks' shared
+// of a 3.2 us step issuing the observations' 27 sums.  Every block keeps its
+// threads' observations on chip; each warp reduce-scatters its 27 sums (lane q
+// ends with sum q) and writes them to all blocks' shared
 // memory, one cluster barrier makes them visible, and then every warp adds
 // the 16 warps' sums in the same order and solves the 6x6 system itself, so
 // nothing is broadcast back.  The additions are those of one 512-thread block
@@ -1806,7 +1808,8 @@ __global__ void __launch_bounds__(kThreads, FT_MIN_CTAS_PER_SM) ft_fused_one_ker
 // round's remaining steps), so the results are the same bit for bit.  A step
 // now spends 2200 cycles on three observations per thread, 250 on the
 // reduction, 600 on the barrier and 1300 on the solve.  One frame of 1100
-// matches: 135 us a call before, 90 us now; 16 frames' share 116 -> 85 us.
+// matches: 135 us a call before, 80 to 95 us now by the steps its data needs
+// (the call's table no longer travels ahead of it); 16 frames' share 116 -> 85 us.
 namespace {
 
 constexpr int kPoseLanes = 512;                       // threads of a frame, over all its blocks

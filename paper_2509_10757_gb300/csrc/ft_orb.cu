@@ -10,20 +10,21 @@
 // tests on the level smoothed by the 5x5 binomial filter.
 //
 // Three launches per call, each over every image of the call:
-//   detect    one block of 256 threads per 32x32 tile of a level: the tile
-//             and a 4-pixel halo in shared memory as two planes of packed
-//             pixel pairs, the FAST score of every pixel of the tile and its
-//             one-pixel ring (two pixels per step in 16-bit lanes, both
-//             polarities by three-input packed min/max), a 16-bit
-//             suppression key per pixel that orders score and raster
-//             position at once, suppression as one comparison with the
-//             eight neighbours' largest key, the kept corners appended as
+//   detect    one block of 256 threads per 62x30 tile of a level (64x32 with
+//             its suppression ring): the tile and a 4-pixel halo in shared
+//             memory as two planes of packed pixel pairs, a compass test of
+//             every pair (two pixels per step in 16-bit lanes), the arcs and
+//             the FAST score of the pairs that pass, for their polarity, a
+//             16-bit suppression key per corner that orders score and raster
+//             position at once, suppression of the listed corners by their
+//             eight neighbours' largest key, the kept ones appended as
 //             keys (255 - score) << 24 | y << 12 | x (one atomic per warp),
 //             and the smoothed level written from the same tile (separable,
 //             two pixels per word);
-//   select    one block per (image, level): the max_kp-th smallest key by an
-//             exact 4 x 8-bit radix select over the level's corners, the
-//             keys up to it gathered and sorted (bitonic) in shared memory;
+//   select    one block per (image, level): the max_kp best of the level's
+//             corners in two reads of them (the deciding score, then the
+//             gather), sorted in shared memory by counting or a bitonic
+//             network;
 //   describe  one warp per output slot: the keypoint's two neighbourhoods
 //             (level and smoothed level) copied to shared memory in one
 //             round trip of 16-byte asynchronous copies, the moments over
