@@ -269,6 +269,11 @@ struct OverlapLaunch {
 };
 }  // namespace ft
 
+// Copies a batch table from pinned host memory (bytes rounded up to whole 16).
+namespace ft {
+cudaError_t launch_table_copy(void *dst, const void *pinned, size_t bytes, cudaStream_t stream);
+}  // namespace ft
+
 // Launch helpers implemented in ft_kernels.cu (host-callable).  overlap: the
 // call's previous kernel lets this one start before it ends.
 namespace ft {

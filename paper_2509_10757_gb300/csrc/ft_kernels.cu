@@ -2246,6 +2246,22 @@ __global__ void __cluster_dims__(kPoseCtas, 1, 1) __launch_bounds__(kPoseThreads
 
 }  // namespace
 
+// A batch table's 16-byte words from mapped pinned host memory: small blocks
+// without shared memory, which find room beside a running fused kernel.
+__global__ void __launch_bounds__(128) ft_table_kernel(uint4 *__restrict__ dst, const uint4 *src, unsigned n)
+{
+    const unsigned i = blockIdx.x * 128u + threadIdx.x;
+    if (i < n) dst[i] = __ldcv(src + i);
+}
+
+cudaError_t launch_table_copy(void *dst, const void *pinned, size_t bytes, cudaStream_t stream)
+{
+    const unsigned n = (unsigned)((bytes + 15) / 16);
+    if (n == 0) return cudaSuccess;
+    ft_table_kernel<<<(n + 127) / 128, 128, 0, stream>>>(static_cast<uint4 *>(dst), static_cast<const uint4 *>(pinned), n);
+    return cudaGetLastError();
+}
+
 int fused_smem_bytes() { return (int)sizeof(Smem); }
 
 const void *fused_kernel_ptr() { return (const void *)ft_fused_kernel; }
