@@ -67,7 +67,10 @@ int next_pow2(int v)
     return p;
 }
 
-int next_pow2_or_zero(int v) { return v > 0 ? next_pow2(v) : 0; }
+// blocks per frame of a graph's fisheye kernel: few sizes, so that calls of
+// uneven frames meet few graphs (16 blocks are 2048 left keypoints; a frame's
+// blocks past its keypoints exit)
+int fisheye_graph_blocks(int v) { return v > 0 ? std::max(16, next_pow2(v)) : 0; }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -924,12 +927,16 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         return finish_call(ctx, stream);
     }
     if (items > 0 || pyr_frames > 0 || pose_frames > 0 || fish_frames > 0) {
-        if (allow_graph && ctx->use_graphs && items > 0) {
+        // a call of one kernel is launched as it is: a graph of one node saves
+        // nothing over it and costs its instantiation at the first call of its
+        // kind, which a served mix of uneven batches pays again and again
+        const bool several = pyr_frames > 0 || fish_frames > 0 || pose_frames > 0;
+        if (allow_graph && ctx->use_graphs && items > 0 && several) {
             const int fp2 = bk.frames_p2;
             cudaGraphExec_t exec = nullptr;
             if ((s = send_table(ctx, slot, bytes, stream)) != FT_OK) return s;
             if ((s = get_graph(ctx, table_dev, fp2, cps, slot, grid_max, pyr_frames > 0 ? fp2 : 0, pyr_blocks, params.nlevels, pose_frames > 0 ? fp2 : 0,
-                               next_pow2_or_zero(fish_blocks), &exec)) != FT_OK)
+                               fisheye_graph_blocks(fish_blocks), &exec)) != FT_OK)
                 return s;
             FT_CUDA(cudaGraphLaunch(exec, stream));
         } else {

@@ -197,13 +197,13 @@ def test_smallest_arena_gives_the_same_results(lib):
     # the launch rule takes the two-pass search for a small batch; its extra
     # scratch is given up where the arena has no room for it
     from paper_2509_10757_gb300.batch import Context, PackedBatch, stream_handle
-    frames = scenes.pinhole_batch(seed=38, n_frames=3)
+    frames = scenes.pinhole_batch(seed=38, n_frames=16)
     pb = PackedBatch(frames)
     pb.upload()
     b = pb.batch()
 
     def status(arena):
-        c = Context(arena_bytes=arena, max_frames=4)
+        c = Context(arena_bytes=arena, max_frames=16)
         try:
             r = c.lib.ft_track_batch(c.ptr, stream_handle(), None, C.byref(b))
             torch.cuda.synchronize()
@@ -219,6 +219,7 @@ def test_smallest_arena_gives_the_same_results(lib):
         r = status(mid)
         assert r in (lib.FT_OK, lib.FT_ENOMEM)
         lo, hi = (lo, mid) if r == 0 else (mid, hi)
+    assert status(lo) == lib.FT_ENOMEM
     pb.clear_outputs()
     assert status(hi) == 0
     pb.download()
