@@ -3,8 +3,8 @@
 Default workload (N=1): the batched pinhole workload: 64 frames per fused
 launch, 752x480 stereo pairs, 1000-1500 left keypoints and 2000-5000 local
 map points per frame, seeded synthetic scenes; a step is one ft_track_batch
-call (stereo matching then local-map search for all 64 frames), replayed
-through a CUDA graph with tile shapes from the autotuner.
+call (stereo matching then local-map search for all 64 frames) with tile
+shapes from the autotuner.
 
 metric: matched keypoints/s + map-point searches/s, i.e. (left keypoints
 stereo-matched + map points searched) per second, whole job over all ranks.
@@ -679,7 +679,7 @@ def fisheye_pairs(frames) -> int:
 
 def time_batch(frames, steps: int, warmup: int, dev, local_rank: int, arena_bytes: int, lasts=None,
                pose: bool = False) -> dict:
-    """One fused launch per step over `frames` (graph replay, autotuned tiles,
+    """One fused launch per step over `frames` (autotuned tiles,
     L2 flushed between steps): launch time, throughput and the HBM roofline."""
     import ctypes as C
 
@@ -876,7 +876,7 @@ def small_batch_result(steps: int, warmup: int, dev, local_rank: int) -> dict:
             ctx.close()
         out[str(n)] = row
     return {"frames": out, "steps": steps,
-            "form": "one context, one stream, CUDA graphs, L2 flushed before each launch, median of launches "
+            "form": "one context, one stream, L2 flushed before each launch, median of launches "
                     "timed alone; default launch shape with the search in two halves or in one pass"}
 
 
@@ -1032,7 +1032,7 @@ def run_gpu(args, rank, world, local_rank):
     # clocks are sampled from here (before the warm-up) to after the last timed form
     clocks = ClockSampler(local_rank)
     clocks.start()
-    # warm-up on every lane (graph capture happens on the first calls)
+    # warm-up on every lane
     for i in range(max(args.warmup, LANES)):
         step(i)
     torch.cuda.synchronize(dev)
@@ -1259,7 +1259,7 @@ def run_gpu(args, rank, world, local_rank):
                          f"the {LANES} buffer sets take turns, so a launch's inputs return after "
                          f"~{135 * (LANES - 1)} MB of other traffic); the serial form flushes (256 MB write) "
                          "before every launch",
-                   "cuda_graph": True, "tuning": ctx_tuning,
+                   "cuda_graph": False, "tuning": ctx_tuning,
                    "tuning_from": "ft_autotune_stream (the serial form: ft_autotune)"},
         "serial": {"value": serial_units / serial_s, "ms_per_launch": statistics.mean(step_ms),
                    "steps": n_serial, "tuning": tuning_of(best),
@@ -1291,7 +1291,7 @@ def run_gpu(args, rank, world, local_rank):
                             "value": (kp_units + mp_units) * world / (statistics.mean(pyr_ms) / 1e3),
                             "levels_built_bytes": pyr_built_bytes,
                             "form": "inputs resident, levels 1-7 of both pyramids built on the device "
-                                    "before the fused launch (two kernels, one graph)"},
+                                    "before the fused launch (two kernels)"},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                      "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
                      "algorithmic_bytes_per_launch": alg_bytes,
