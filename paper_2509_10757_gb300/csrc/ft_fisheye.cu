@@ -570,7 +570,7 @@ cudaError_t launch_fisheye(const BatchHeader *dev_hdr, int nframes, int blocks, 
     const unsigned splits = (unsigned)fisheye_splits(nframes, blocks);
     OverlapLaunch l(dim3((unsigned)blocks, (unsigned)nframes, splits), kFishThreads, kFishSmem, stream, overlap);
     l.cluster(1, 1, splits);
-    return cudaLaunchKernelEx(&l.cfg, ft_fisheye_kernel, dev_hdr);
+    return l.run(ft_fisheye_kernel, dev_hdr);
 }
 
 cudaError_t launch_fisheye(const FrameCall &call, int blocks, cudaStream_t stream)
@@ -579,7 +579,7 @@ cudaError_t launch_fisheye(const FrameCall &call, int blocks, cudaStream_t strea
     const unsigned splits = (unsigned)fisheye_splits(1, blocks);
     OverlapLaunch l(dim3((unsigned)blocks, 1, splits), kFishThreads, kFishSmem, stream, false);
     l.cluster(1, 1, splits);
-    return cudaLaunchKernelEx(&l.cfg, ft_fisheye_one_kernel, call);
+    return l.run(ft_fisheye_one_kernel, call);
 }
 
 }  // namespace ft

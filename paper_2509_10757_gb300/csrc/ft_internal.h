@@ -266,6 +266,11 @@ struct OverlapLaunch {
         attr[cfg.numAttrs].val.clusterDim.z = z;
         ++cfg.numAttrs;
     }
+    template <class... P, class... A>
+    cudaError_t run(void (*kernel)(P...), const A &...args)
+    {
+        return cudaLaunchKernelEx(&cfg, kernel, args...) == cudaSuccess ? cudaSuccess : cudaGetLastError();
+    }
 };
 }  // namespace ft
 

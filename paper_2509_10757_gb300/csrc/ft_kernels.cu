@@ -2284,13 +2284,13 @@ cudaError_t fused_occupancy(int *ctas_per_sm)
 cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stream, bool overlap)
 {
     OverlapLaunch l(dim3((unsigned)grid), kThreads, sizeof(Smem), stream, overlap);
-    return cudaLaunchKernelEx(&l.cfg, ft_fused_kernel, dev_hdr);
+    return l.run(ft_fused_kernel, dev_hdr);
 }
 
 cudaError_t launch_fused(const FrameCall &call, int grid, cudaStream_t stream, bool overlap)
 {
     OverlapLaunch l(dim3((unsigned)grid), kThreads, sizeof(Smem), stream, overlap);
-    return cudaLaunchKernelEx(&l.cfg, ft_fused_one_kernel, call);
+    return l.run(ft_fused_one_kernel, call);
 }
 
 cudaError_t launch_pose(const FrameCall &call, cudaStream_t stream)

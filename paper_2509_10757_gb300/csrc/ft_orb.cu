@@ -728,11 +728,11 @@ cudaError_t launch_orb(const OrbHeader *dev_hdr, int nimages, int nlevels, int m
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     OverlapLaunch select(dim3((unsigned)nlevels, (unsigned)nimages), kOrbSelectThreads, 0, stream, true);
-    e = cudaLaunchKernelEx(&select.cfg, orb_select_kernel, dev_hdr);
+    e = select.run(orb_select_kernel, dev_hdr);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((max(max_slots, 1) + kDescribeWarps - 1) / kDescribeWarps);
     OverlapLaunch describe(dim3(blocks, (unsigned)nimages), 32 * kDescribeWarps, 0, stream, true);
-    return cudaLaunchKernelEx(&describe.cfg, orb_describe_kernel, dev_hdr);
+    return describe.run(orb_describe_kernel, dev_hdr);
 }
 
 }  // namespace ft
