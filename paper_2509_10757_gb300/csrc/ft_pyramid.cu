@@ -30,6 +30,12 @@
 // the formula clamps the source coordinate there, its weight is zero, and zero
 // times any byte is the same zero.
 // Every tile is independent: no block waits for another.
+// What bounds it is instruction issue and the shared-memory pipe together: 128
+// images of 752x480, 97 M output pixels, take 103 us (131 with a float per
+// pixel and scalar products; 25 against 31 warp instructions a pixel, 10 against
+// 25 M shared-memory wavefronts of loads).  Two, four and six columns a thread:
+// 300 / 297 / 306 us for the call of 64 frames with pose; 384 and 512 threads
+// 309 and 323.
 //
 // A byte b placed in the mantissa of 2^23 is the float 2^23 + b, and
 // fma(2^23 + b, w, -2^23 w) rounds the exact b w once: the product b w as one
