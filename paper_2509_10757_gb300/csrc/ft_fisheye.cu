@@ -400,6 +400,10 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
     }
     const int rows = min(seen - tile * kFishRows, kFishRows);
     if (rows <= 0) return;                          // the whole cluster
+    // says that this block has started; the first block's shared memory may be
+    // written by the others once all have said so (waited for below, long over
+    // by then: the matching lies between)
+    if (splits > 1) asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
 
     __syncwarp();
     if (warp == 0) {
@@ -500,6 +504,7 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
         S.second[half][r] = second;
         __syncthreads();
     } else {
+        asm volatile("barrier.cluster.wait;" ::: "memory");             // every block has started
         store_first(&S.best[2 * split + half][r], best);
         store_first(&S.second[2 * split + half][r], second);
         __syncthreads();
