@@ -43,6 +43,7 @@ constexpr int kFishRowBytes = 256;      // an expanded descriptor
 constexpr int kFishTile = kFishRows * kFishRowBytes;
 constexpr int kFishSplit = 4;           // blocks that share a row's columns, at most (a cluster)
 constexpr unsigned kTmemCols = 2 * kFishCols;
+constexpr unsigned long long kDrainNs = 2000000000ull;       // bound of the wait for products after a wait ran out
 static_assert(kFishRows == kFishCols, "both operands share the tile layout");
 static_assert(kFishThreads == 2 * kFishRows, "two threads expand a row, two warps read a row");
 
@@ -428,7 +429,7 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
     unsigned best = kNoKey, second = kNoKey;        // of row 32 (warp & 3) + lane, half the columns
     const int half = warp >> 2;
     const unsigned lanes = (unsigned)(32 * (warp & 3)) << 16;
-    unsigned phase[2] = {0, 0};
+    unsigned phase = 0, flying = 0;                 // bit k: parity of mbar[k]; a product that arrives on it is on its way
     bool ok = true;
     for (int j0 = 0; j0 < nr && ok; j0 += kFishWindow) {
         const int cnt = compact(rx, j0, min(kFishWindow, nr - j0), lap_r0, lap_r1, S.count,
@@ -449,6 +450,7 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             ok = __syncthreads_and(ok);
             if (!ok) return;
+            flying |= 1u << (i & 1);
             if (tid == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 mma_step(tmem + (unsigned)(i & 1) * kFishCols, smem_addr(S.a), smem_addr(S.b[i & 1]),
@@ -465,8 +467,10 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
             if (i + 1 < mine) stage(i + 1);
             if (!ok) break;                         // a wait ran out: known to the whole block
             const int s = split + i * splits;
-            ok = __all_sync(kFull, mbar_wait(smem_addr(&S.mbar[i & 1]), phase[i & 1], timeout_ns));
-            phase[i & 1] ^= 1u;
+            ok = __all_sync(kFull, mbar_wait(smem_addr(&S.mbar[i & 1]), (phase >> (i & 1)) & 1u, timeout_ns));
+            if (!ok) continue;                      // the others learn of it at the next block-wide synchronization
+            phase ^= 1u << (i & 1);
+            flying &= ~(1u << (i & 1));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const int n = cnt - s * kFishCols - 64 * half;       // of this warp's 64 columns
             unsigned b2 = 0xffffffffu, s2 = 0xffffffffu;
@@ -495,6 +499,11 @@ __device__ __forceinline__ void fisheye_run(const BatchHeader *hdr, const FrameD
     if (!ok) {
         if (tid == 0) atomicOr(hdr->status, kStatusTimeout);
         best = second = kNoKey;
+        // products still on their way write tensor memory and read the tiles:
+        // they end before either is given back
+        for (int k = 0; k < 2; ++k)
+            if (flying >> k & 1u) (void)mbar_wait(smem_addr(&S.mbar[k]), (phase >> k) & 1u, kDrainNs);
+        __syncthreads();
     }
     // the parts of a row's columns (two halves of every block's steps) meet in
     // the cluster's first block, which then writes the match

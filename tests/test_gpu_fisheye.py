@@ -55,3 +55,36 @@ def test_blocks_without_columns(ctx, inside, nl):
         many = run_fused(ctx, [fr] * n)
         for f in range(n):
             assert_fisheye_equal(many.outputs(f), ref, f"{nl} left, {inside} in the overlap, frame {f} of {n}: ")
+
+
+@pytest.mark.parametrize("n", [1, 3])
+def test_waits_that_run_out_leave_a_usable_context(ctx, n):
+    # a bound of 1 ns on the waits for products: whether or not one runs out,
+    # the call ends, its outputs are defined (a right keypoint or none) and the
+    # next call's results are the oracle's
+    from paper_2509_10757_gb300 import _lib as L
+    from paper_2509_10757_gb300.batch import PackedBatch, run_batch
+    fr = scenes.fisheye_frame(82, n_left=2500, n_map=0)
+    ref = orc.stereo_frame(P, fr)
+    pb = PackedBatch([fr] * n)
+    pb.upload()
+    try:
+        for _ in range(20):
+            L.check(L.ft_set_debug(ctx.ptr, 0, 1), "debug")
+            pb.clear_outputs()
+            run_batch(ctx, pb)
+            status = ctx.sync_status()
+            assert status in (L.FT_OK, L.FT_ETIMEOUT)
+            pb.download()
+            for f in range(n):
+                out = pb.outputs(f)
+                assert out["r_idx"].min() >= -1 and out["r_idx"].max() < fr.right.n
+                assert out["d1"].min() >= -1 and out["d2"].max() <= 256
+    finally:
+        L.check(L.ft_set_debug(ctx.ptr, 0, 0), "debug")
+    pb.clear_outputs()
+    run_batch(ctx, pb)
+    pb.download()
+    assert ctx.sync_status() == L.FT_OK
+    for f in range(n):
+        assert_fisheye_equal(pb.outputs(f), ref, f"after the short waits, frame {f} of {n}: ")
