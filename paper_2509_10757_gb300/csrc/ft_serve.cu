@@ -16,9 +16,18 @@
 // the batch's completion.  Requests that arrive while a batch runs are taken
 // by the next free slot, so batches overlap on the device.
 //
+// No thread holds the server's lock across a CUDA call, and the host function
+// takes no lock: a page-locked allocation, a free or a synchronous copy may
+// wait for the device, whose streams wait for the host function to return (with
+// the lock on both sides, a submit whose images needed their staging and a
+// batch's completion waited for each other for ever).  What a call allocates or
+// copies it reserves under the lock, does without it, and then publishes.
+//
 // A dry-run server (no GPU) replaces the device work by a fake completion
 // after a fixed delay; it exercises the same admission and scheduling code.
 #include <cuda_runtime.h>
+#include <semaphore.h>
+#include <time.h>
 
 #include <algorithm>
 #include <atomic>
@@ -180,6 +189,8 @@ struct StreamState {
                                    // allocated at the first request that carries images)
     int next_out = 0;
     bool in_flight = false;
+    bool uploading = false;        // a map or pyramids on their way to the block (the lock is not held meanwhile)
+    bool reserved = false;         // the entry is taken by a stream that is being opened
     int queued = 0;
 };
 
@@ -211,6 +222,25 @@ struct Slot {
 
 void CUDART_CB host_done(void *p);
 
+// What the scheduler sleeps on: a semaphore, which a host function may post
+// (it waits for nothing).
+struct Wake {
+    sem_t s;
+    Wake() { sem_init(&s, 0, 0); }
+    ~Wake() { sem_destroy(&s); }
+    void post() { sem_post(&s); }
+    void wait_us(long us)
+    {
+        timespec t;
+        clock_gettime(CLOCK_MONOTONIC, &t);
+        t.tv_nsec += us * 1000;
+        t.tv_sec += t.tv_nsec / 1000000000;
+        t.tv_nsec %= 1000000000;
+        (void)sem_clockwait(&s, CLOCK_MONOTONIC, &t);
+        while (sem_trywait(&s) == 0) {}         // one look answers all posts so far
+    }
+};
+
 }  // namespace
 
 struct ft_server {
@@ -223,8 +253,9 @@ struct ft_server {
     std::deque<StreamState> streams;   // a deque: references stay valid while streams open
     std::vector<Slot *> slots;
     std::mutex mu;
-    std::condition_variable cv;        // scheduler wake-up
+    Wake wake;                         // the scheduler's
     std::condition_variable done_cv;   // completions available
+    std::condition_variable upload_cv; // an upload has ended
     std::deque<Request> pending;
     std::deque<ft_completion> completed;
     std::thread thread;
@@ -253,11 +284,8 @@ void CUDART_CB host_done(void *p)
 {
     DoneArg *a = static_cast<DoneArg *>(p);
     a->slot->t_done = now_us();
-    {
-        std::lock_guard<std::mutex> lk(a->server->mu);
-        a->slot->done.store(1);
-    }
-    a->server->cv.notify_one();
+    a->slot->done.store(1);                     // (t_done is read after it)
+    a->server->wake.post();
 }
 
 // resident pyramid rows are padded to 16 bytes (the kernel reads 4-byte words)
@@ -442,7 +470,8 @@ void scheduler(ft_server *s)
             std::vector<int> taken_streams;
             for (auto it = s->pending.begin(); it != s->pending.end() && (int)sl->reqs.size() < s->desc.max_batch;) {
                 StreamState &S = s->streams[it->sid];
-                if (S.in_flight || std::find(taken_streams.begin(), taken_streams.end(), it->sid) != taken_streams.end()) {
+                if (S.in_flight || S.uploading ||
+                    std::find(taken_streams.begin(), taken_streams.end(), it->sid) != taken_streams.end()) {
                     // keep this stream's order: none of its later requests may pass
                     taken_streams.push_back(it->sid);
                     ++it;
@@ -468,9 +497,45 @@ void scheduler(ft_server *s)
             if (st != FT_OK) s->last_launch_status = st;
             progress = true;
         }
-        if (!progress) s->cv.wait_for(lk, std::chrono::microseconds(s->dry ? 20 : 200));
+        if (!progress) {
+            lk.unlock();
+            s->wake.wait_us(s->dry ? 20 : 200);
+            lk.lock();
+        }
     }
 }
+
+// The open stream sid once no other call's upload to it is running (nullptr: not
+// open); lk is held before and after.
+StreamState *open_idle(ft_server *s, int sid, std::unique_lock<std::mutex> &lk)
+{
+    auto open = [&] { return sid >= 0 && sid < (int)s->streams.size() && s->streams[sid].open; };
+    s->upload_cv.wait(lk, [&] { return !open() || !s->streams[sid].uploading; });
+    return open() ? &s->streams[sid] : nullptr;
+}
+
+// Holds a stream for an upload that runs without the lock: the scheduler passes
+// the stream's requests over meanwhile.  lk is held before and after.
+class Upload {
+  public:
+    Upload(ft_server *s, StreamState &S, std::unique_lock<std::mutex> &lk) : s_(s), S_(S), lk_(lk)
+    {
+        S_.uploading = true;
+        lk_.unlock();
+    }
+    ~Upload()
+    {
+        lk_.lock();
+        S_.uploading = false;
+        s_->upload_cv.notify_all();
+        s_->wake.post();
+    }
+
+  private:
+    ft_server *s_;
+    StreamState &S_;
+    std::unique_lock<std::mutex> &lk_;
+};
 
 }  // namespace
 
@@ -545,7 +610,7 @@ void ft_server_destroy(ft_server *s)
         std::lock_guard<std::mutex> lk(s->mu);
         s->stop = true;
     }
-    s->cv.notify_all();
+    s->wake.post();
     if (s->thread.joinable()) s->thread.join();
     for (Slot *sl : s->slots) {
         if (sl->stream) {
@@ -577,11 +642,26 @@ ft_status ft_server_open_stream(ft_server *s, const ft_stream_desc *d, int *stre
     StreamState S;
     S.desc = *d;
     const size_t bytes = stream_block_bytes(*d, s->params, &S);
-    std::lock_guard<std::mutex> lk(s->mu);
+    // the block and an entry are taken under the lock, the staging is allocated
+    // without it
     size_t off = 0;
-    if (!s->pool->alloc(bytes, &off))
-        return fail(FT_EBUSY, "HBM budget: stream needs %zu bytes, %zu of %zu in use", bytes, s->pool->used(),
-                    s->pool->capacity());
+    int id = -1;
+    {
+        std::lock_guard<std::mutex> lk(s->mu);
+        if (!s->pool->alloc(bytes, &off))
+            return fail(FT_EBUSY, "HBM budget: stream needs %zu bytes, %zu of %zu in use", bytes, s->pool->used(),
+                        s->pool->capacity());
+        for (size_t i = 0; i < s->streams.size(); ++i)
+            if (!s->streams[i].open && !s->streams[i].reserved) {
+                id = (int)i;
+                break;
+            }
+        if (id < 0) {
+            id = (int)s->streams.size();
+            s->streams.emplace_back();
+        }
+        s->streams[id].reserved = true;
+    }
     S.off = off;
     S.bytes = bytes;
     S.dev = s->dry ? nullptr : s->pool_mem + off;
@@ -595,23 +675,15 @@ ft_status ft_server_open_stream(ft_server *s, const ft_stream_desc *d, int *stre
             ok = cudaMallocHost(&S.h_out[b], std::max<size_t>(outb, 16)) == cudaSuccess;
         if (!ok) {
             free_staging(S);
+            std::lock_guard<std::mutex> lk(s->mu);
             s->pool->release(off, bytes);
+            s->streams[id] = StreamState();
             return fail(FT_ENOMEM, "pinned staging for the stream could not be allocated");
         }
     }
     S.open = true;
-    int id = -1;
-    for (size_t i = 0; i < s->streams.size(); ++i)
-        if (!s->streams[i].open) {
-            id = (int)i;
-            break;
-        }
-    if (id < 0) {
-        id = (int)s->streams.size();
-        s->streams.push_back(S);
-    } else {
-        s->streams[id] = S;
-    }
+    std::lock_guard<std::mutex> lk(s->mu);
+    s->streams[id] = S;
     s->stats.streams_open += 1;
     *stream_id = id;
     return FT_OK;
@@ -620,26 +692,35 @@ ft_status ft_server_open_stream(ft_server *s, const ft_stream_desc *d, int *stre
 ft_status ft_server_close_stream(ft_server *s, int sid)
 {
     if (!s) return fail(FT_EINVAL, "ft_server_close_stream: NULL server");
-    std::lock_guard<std::mutex> lk(s->mu);
-    if (sid < 0 || sid >= (int)s->streams.size() || !s->streams[sid].open) return fail(FT_EINVAL, "stream %d not open", sid);
-    StreamState &S = s->streams[sid];
-    if (S.in_flight || S.queued > 0) return fail(FT_EBUSY, "stream %d has requests in flight", sid);
-    s->pool->release(S.off, S.bytes);
-    free_staging(S);
-    S = StreamState();
-    s->stats.streams_open -= 1;
+    StreamState closed;
+    {
+        std::unique_lock<std::mutex> lk(s->mu);
+        StreamState *p = open_idle(s, sid, lk);
+        if (!p) return fail(FT_EINVAL, "stream %d not open", sid);
+        StreamState &S = *p;
+        if (S.in_flight || S.queued > 0) return fail(FT_EBUSY, "stream %d has requests in flight", sid);
+        for (int b = 0; b < kMaxQueue; ++b)
+            if (S.dyn_used[b]) return fail(FT_EBUSY, "stream %d has requests in flight", sid);    // being staged
+        s->pool->release(S.off, S.bytes);
+        closed = S;
+        S = StreamState();
+        s->stats.streams_open -= 1;
+    }
+    free_staging(closed);
     return FT_OK;
 }
 
 ft_status ft_server_set_pyramids(ft_server *s, int sid, const ft_pyramid *left, const ft_pyramid *right)
 {
     if (!s || !left || !right) return fail(FT_EINVAL, "ft_server_set_pyramids: NULL argument");
-    std::lock_guard<std::mutex> lk(s->mu);
-    if (sid < 0 || sid >= (int)s->streams.size() || !s->streams[sid].open) return fail(FT_EINVAL, "stream %d not open", sid);
-    StreamState &S = s->streams[sid];
+    std::unique_lock<std::mutex> lk(s->mu);
+    StreamState *p = open_idle(s, sid, lk);
+    if (!p) return fail(FT_EINVAL, "stream %d not open", sid);
+    StreamState &S = *p;
     if (S.desc.camera != FT_CAMERA_PINHOLE) return fail(FT_EINVAL, "stream %d has no pyramids", sid);
     if (S.in_flight) return fail(FT_EBUSY, "stream %d has a request in flight", sid);
     if (s->dry) return FT_OK;
+    Upload up(s, S, lk);
     for (int l = 0; l < S.desc.nlevels; ++l) {
         const int w = S.desc.level_width[l], h = S.desc.level_height[l];
         const ft_pyramid *src[2] = {left, right};
@@ -658,14 +739,16 @@ ft_status ft_server_set_pyramids(ft_server *s, int sid, const ft_pyramid *left, 
 ft_status ft_server_set_map(ft_server *s, int sid, const ft_map_view *map)
 {
     if (!s || !map) return fail(FT_EINVAL, "ft_server_set_map: NULL argument");
-    std::lock_guard<std::mutex> lk(s->mu);
-    if (sid < 0 || sid >= (int)s->streams.size() || !s->streams[sid].open) return fail(FT_EINVAL, "stream %d not open", sid);
-    StreamState &S = s->streams[sid];
+    std::unique_lock<std::mutex> lk(s->mu);
+    StreamState *p = open_idle(s, sid, lk);
+    if (!p) return fail(FT_EINVAL, "stream %d not open", sid);
+    StreamState &S = *p;
     if (map->n < 0 || map->n > S.desc.max_map) return fail(FT_EINVAL, "map of %d points exceeds capacity %d", map->n, S.desc.max_map);
     if (S.in_flight) return fail(FT_EBUSY, "stream %d has a request in flight", sid);
     if (!s->dry && map->n > 0) {
         if (!map->pos || !map->nrm || !map->desc) return fail(FT_EINVAL, "map: NULL array");
         const size_t n = (size_t)map->n;
+        Upload up(s, S, lk);
         bool ok = cudaMemcpy(S.dev + S.o_pos, map->pos, 16 * n, cudaMemcpyHostToDevice) == cudaSuccess &&
                   cudaMemcpy(S.dev + S.o_nrm, map->nrm, 16 * n, cudaMemcpyHostToDevice) == cudaSuccess &&
                   cudaMemcpy(S.dev + S.o_mdesc, map->desc, 32 * n, cudaMemcpyHostToDevice) == cudaSuccess;
@@ -691,6 +774,7 @@ ft_status ft_server_submit(ft_server *s, const ft_request *req)
     for (int i = 0; i < 3; ++i) r.O_right[i] = req->O_right[i];
     r.images = req->image_left != nullptr || req->image_right != nullptr;
     char *dst = nullptr, *img = nullptr;
+    StreamState *stream = nullptr;
     int W0 = 0, H0 = 0;
     size_t lp0 = 0;
     {
@@ -721,14 +805,19 @@ ft_status ft_server_submit(ft_server *s, const ft_request *req)
                 break;
             }
         if (r.buf < 0) return fail(FT_EBUSY, "stream %d already has %d requests waiting", r.sid, s->depth);
-        if (r.images && !s->dry && !S.h_img[r.buf] &&
-            cudaMallocHost(&S.h_img[r.buf], 2 * lp0 * (size_t)H0) != cudaSuccess) {
-            S.h_img[r.buf] = nullptr;
-            return fail(FT_ENOMEM, "pinned image staging for stream %d could not be allocated", r.sid);
-        }
-        S.dyn_used[r.buf] = 1;
+        S.dyn_used[r.buf] = 1;          // the buffer is this call's from here on, and the stream stays open
         dst = S.h_dyn[r.buf];
         img = S.h_img[r.buf];
+        stream = &S;
+    }
+    if (r.images && !s->dry && !img) {
+        const bool ok = cudaMallocHost(&img, 2 * lp0 * (size_t)H0) == cudaSuccess;
+        std::lock_guard<std::mutex> lk(s->mu);
+        stream->h_img[r.buf] = ok ? img : nullptr;
+        if (!ok) {
+            stream->dyn_used[r.buf] = 0;
+            return fail(FT_ENOMEM, "pinned image staging for stream %d could not be allocated", r.sid);
+        }
     }
     if (!s->dry) {
         const DynLayout D = dyn_layout(r.nl, r.nr);
@@ -758,11 +847,11 @@ ft_status ft_server_submit(ft_server *s, const ft_request *req)
     r.t_submit = now_us();
     {
         std::lock_guard<std::mutex> lk(s->mu);
-        s->streams[r.sid].queued += 1;
+        stream->queued += 1;
         s->pending.push_back(r);
         s->stats.submitted += 1;
     }
-    s->cv.notify_one();
+    s->wake.post();
     return FT_OK;
 }
 
