@@ -197,6 +197,7 @@ struct StreamState {
 struct Request {
     uint64_t tag = 0;
     int sid = -1, buf = 0, nl = 0, nr = 0;
+    StreamState *stream = nullptr; // of sid (it stays open while it has requests); launch() has no lock to look it up
     bool images = false;           // level-0 images staged in h_img[buf]
     ft_pose pose{};
     float O_right[3] = {0, 0, 0};
@@ -398,7 +399,7 @@ ft_status launch(ft_server *s, Slot &sl)
     std::vector<ft_frame_job> jobs;
     jobs.reserve(sl.reqs.size());
     for (Request &r : sl.reqs) {
-        StreamState &S = s->streams[r.sid];
+        StreamState &S = *r.stream;
         const DynLayout D = dyn_layout(r.nl, r.nr);
         if (cudaMemcpyAsync(S.dev + S.o_dyn, S.h_dyn[r.buf], D.bytes, cudaMemcpyHostToDevice, sl.stream) != cudaSuccess)
             return fail(FT_ECUDA, "server: upload failed");
@@ -420,7 +421,7 @@ ft_status launch(ft_server *s, Slot &sl)
     ft_status st = ft_track_batch(sl.ctx, sl.stream, &s->params, &b);
     if (st != FT_OK) return st;
     for (Request &r : sl.reqs) {
-        StreamState &S = s->streams[r.sid];
+        StreamState &S = *r.stream;
         const OutLayout O = out_layout(S.desc.camera, r.nl, r.nr, S.map_n);
         if (cudaMemcpyAsync(S.h_out[r.out_buf], S.dev + S.o_out, O.bytes, cudaMemcpyDeviceToHost, sl.stream) != cudaSuccess)
             return fail(FT_ECUDA, "server: download failed");
@@ -442,7 +443,7 @@ void scheduler(ft_server *s)
             if (s->dry && now_us() < sl->t_done) continue;
             if (!sl->done.load()) continue;
             for (Request &r : sl->reqs) {
-                StreamState &S = s->streams[r.sid];
+                StreamState &S = *r.stream;
                 ft_completion c{};
                 c.tag = r.tag;
                 c.stream_id = r.sid;
@@ -469,7 +470,7 @@ void scheduler(ft_server *s)
             if (sl->busy || s->pending.empty()) continue;
             std::vector<int> taken_streams;
             for (auto it = s->pending.begin(); it != s->pending.end() && (int)sl->reqs.size() < s->desc.max_batch;) {
-                StreamState &S = s->streams[it->sid];
+                StreamState &S = *it->stream;
                 if (S.in_flight || S.uploading ||
                     std::find(taken_streams.begin(), taken_streams.end(), it->sid) != taken_streams.end()) {
                     // keep this stream's order: none of its later requests may pass
@@ -774,7 +775,6 @@ ft_status ft_server_submit(ft_server *s, const ft_request *req)
     for (int i = 0; i < 3; ++i) r.O_right[i] = req->O_right[i];
     r.images = req->image_left != nullptr || req->image_right != nullptr;
     char *dst = nullptr, *img = nullptr;
-    StreamState *stream = nullptr;
     int W0 = 0, H0 = 0;
     size_t lp0 = 0;
     {
@@ -808,14 +808,14 @@ ft_status ft_server_submit(ft_server *s, const ft_request *req)
         S.dyn_used[r.buf] = 1;          // the buffer is this call's from here on, and the stream stays open
         dst = S.h_dyn[r.buf];
         img = S.h_img[r.buf];
-        stream = &S;
+        r.stream = &S;
     }
     if (r.images && !s->dry && !img) {
         const bool ok = cudaMallocHost(&img, 2 * lp0 * (size_t)H0) == cudaSuccess;
         std::lock_guard<std::mutex> lk(s->mu);
-        stream->h_img[r.buf] = ok ? img : nullptr;
+        r.stream->h_img[r.buf] = ok ? img : nullptr;
         if (!ok) {
-            stream->dyn_used[r.buf] = 0;
+            r.stream->dyn_used[r.buf] = 0;
             return fail(FT_ENOMEM, "pinned image staging for stream %d could not be allocated", r.sid);
         }
     }
@@ -847,7 +847,7 @@ ft_status ft_server_submit(ft_server *s, const ft_request *req)
     r.t_submit = now_us();
     {
         std::lock_guard<std::mutex> lk(s->mu);
-        stream->queued += 1;
+        r.stream->queued += 1;
         s->pending.push_back(r);
         s->stats.submitted += 1;
     }

@@ -59,3 +59,27 @@ done = drain(s, n)
 assert sorted(d[0] for d in done) == list(range(1, n + 1)), done
 L.ft_server_destroy(s)
 """, limit_s=30.0)
+
+
+def test_streams_open_while_batches_launch(fake):
+    # the table of streams grows (and moves) while the scheduler launches
+    run_against(fake, SERVER + """
+stop = []
+def opener():
+    d = stream_desc_of(scenes.pinhole_frame(3, W=64, H=48, n_left=4, n_map=4))
+    while not stop:
+        ids = []
+        for _ in range(400):
+            sid = C.c_int(-1)
+            if L.ft_server_open_stream(s, C.byref(d), C.byref(sid)) == L.FT_OK: ids.append(sid.value)
+        for i in ids: L.check(L.ft_server_close_stream(s, i))
+t = threading.Thread(target=opener); t.start()
+n = 0
+while n < 300:
+    for sid, h in ((a, hosts[0]), (b, hosts[1])):
+        if L.ft_server_submit(s, C.byref(h.request(sid, n))) == L.FT_OK: n += 1
+done = drain(s, n)
+stop.append(1); t.join()
+assert len(done) == n and all(d[2] == L.FT_OK for d in done)
+L.ft_server_destroy(s)
+""")
