@@ -657,7 +657,7 @@ typedef struct {
 typedef struct {
     uint64_t tag;
     int stream_id;
-    int32_t status;
+    int32_t status;             /* FT_OK, or why the request's launch failed (results are then empty) */
     double t_submit_us, t_start_us, t_done_us;
     ft_results results;
 } ft_completion;

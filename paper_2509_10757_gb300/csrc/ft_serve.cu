@@ -216,6 +216,7 @@ struct Slot {
     cudaStream_t stream = nullptr;
     std::vector<Request> reqs;
     bool busy = false;
+    ft_status status = FT_OK;      // of the batch's launch
     std::atomic<int> done{0};
     double t_start = 0, t_done = 0;
     DoneArg arg{};
@@ -447,11 +448,12 @@ void scheduler(ft_server *s)
                 ft_completion c{};
                 c.tag = r.tag;
                 c.stream_id = r.sid;
-                c.status = FT_OK;
+                c.status = sl->status;
                 c.t_submit_us = r.t_submit;
                 c.t_start_us = sl->t_start;
                 c.t_done_us = sl->t_done;
-                if (!s->dry) c.results = results_of(S, r, S.h_out[r.out_buf]);
+                if (sl->status != FT_OK) c.results = ft_results{};      // nothing was computed
+                else if (!s->dry) c.results = results_of(S, r, S.h_out[r.out_buf]);
                 else c.results.n_left = r.nl, c.results.n_right = r.nr, c.results.n_map = S.map_n;
                 S.in_flight = false;
                 S.dyn_used[r.buf] = 0;
@@ -493,9 +495,16 @@ void scheduler(ft_server *s)
             s->stats.batches += 1;
             s->stats.frames_launched += sl->reqs.size();
             lk.unlock();
-            const ft_status st = launch(s, *sl);
+            sl->status = launch(s, *sl);
+            if (sl->status != FT_OK) {
+                // its requests complete with the status once what did reach the
+                // stream has ended (their staging and blocks are free then)
+                (void)cudaStreamSynchronize(sl->stream);
+                sl->t_done = now_us();
+                sl->done.store(1);
+            }
             lk.lock();
-            if (st != FT_OK) s->last_launch_status = st;
+            if (sl->status != FT_OK) s->last_launch_status = sl->status;
             progress = true;
         }
         if (!progress) {

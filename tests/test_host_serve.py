@@ -83,3 +83,23 @@ stop.append(1); t.join()
 assert len(done) == n and all(d[2] == L.FT_OK for d in done)
 L.ft_server_destroy(s)
 """)
+
+
+# the first memory copy of a launch, the kernels, the copy of the results (a
+# launch of one request makes two copies), and the host function
+@pytest.mark.parametrize("what,after", [("memcpy_async", 0), ("fused", 0), ("memcpy_async", 1), ("host_func", 0)])
+def test_a_failed_launch_completes_its_requests(fake, what, after):
+    run_against(fake, SERVER + f"""
+lib.fake_fail({what!r}.encode(), {after})
+L.check(L.ft_server_submit(s, C.byref(hosts[0].request(a, 1))))
+assert drain(s, 1) == [(1, a, L.FT_ECUDA)]
+st = L.ft_server_stats()
+L.ft_server_get_stats(s, C.byref(st))
+assert st.last_error == L.FT_ECUDA and st.completed == 1
+for tag in range(2, 12):                    # the stream, its staging and both slots are free again
+    for sid, h in ((a, hosts[0]), (b, hosts[1])):
+        L.check(L.ft_server_submit(s, C.byref(h.request(sid, tag))))
+    assert sorted(drain(s, 2)) == [(tag, a, L.FT_OK), (tag, b, L.FT_OK)]
+L.check(L.ft_server_close_stream(s, a))
+L.ft_server_destroy(s)
+""")
