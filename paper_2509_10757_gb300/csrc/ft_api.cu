@@ -773,6 +773,37 @@ ft_status finish_call(ft_ctx *ctx, cudaStream_t s)
     return FT_OK;
 }
 
+// From the call's first enqueued operation to its end.  If the call fails in
+// between, what it did enqueue still uses the slot's tables and the arena: the
+// slot (>= 0) and the context count as in use until the stream has passed it.
+class CallGuard {
+  public:
+    CallGuard(ft_ctx *ctx, int slot, cudaStream_t s) : ctx_(ctx), slot_(slot), s_(s) {}
+    ~CallGuard()
+    {
+        if (!ctx_) return;
+        if (slot_ >= 0) (void)cudaEventRecord(ctx_->slot_done[slot_], s_);
+        if (cudaEventRecord(ctx_->done, s_) == cudaSuccess) {
+            ctx_->last_stream = s_;
+            ctx_->have_last = true;
+        }
+        (void)cudaGetLastError();
+    }
+    ft_status end()
+    {
+        ft_ctx *ctx = ctx_;
+        if (slot_ >= 0) FT_CUDA(cudaEventRecord(ctx->slot_done[slot_], s_));
+        const ft_status s = finish_call(ctx, s_);
+        if (s == FT_OK) ctx_ = nullptr;
+        return s;
+    }
+
+  private:
+    ft_ctx *ctx_;
+    int slot_;
+    cudaStream_t s_;
+};
+
 // Copies the first `bytes` of the slot's staged table to its device memory
 // ahead of what `stream` runs next.  A stream that is being captured takes the
 // copy itself.
@@ -790,8 +821,13 @@ ft_status send_table(ft_ctx *ctx, int slot, size_t bytes, cudaStream_t stream)
         return FT_OK;
     }
     FT_CUDA(launch_table_copy(dev, ctx->staging[slot], bytes, ctx->copy_stream));
-    FT_CUDA(cudaEventRecord(ctx->copied[slot], ctx->copy_stream));
-    FT_CUDA(cudaStreamWaitEvent(stream, ctx->copied[slot], 0));
+    cudaError_t e = cudaEventRecord(ctx->copied[slot], ctx->copy_stream);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(stream, ctx->copied[slot], 0);
+    if (e != cudaSuccess) {
+        // nothing on the call's stream stands for the copy: it ends here
+        (void)cudaStreamSynchronize(ctx->copy_stream);
+        FT_CUDA(e);
+    }
     return FT_OK;
 }
 
@@ -920,12 +956,14 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         call.f.ctr = ctx->status + kOneCounters;
         // a call's first kernel follows the stream's earlier work as any launch
         // does; only a kernel behind another of the same call may start early
+        CallGuard guard(ctx, -1, stream);
         FT_CUDA(launch_fisheye(call, fish_blocks, stream));
         if (items > 0) FT_CUDA(launch_fused(call, std::min(items, grid_max), stream, fish_blocks > 0));
         if (pose_frames > 0) FT_CUDA(launch_pose(call, stream));
         ctx->launches += (items > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) + (fish_frames > 0 ? 1 : 0);
-        return finish_call(ctx, stream);
+        return guard.end();
     }
+    CallGuard guard(ctx, slot, stream);
     if (items > 0 || pyr_frames > 0 || pose_frames > 0 || fish_frames > 0) {
         // a call of one or two kernels is launched as it is: a graph saves the
         // host nothing there, its launch shapes are the bucket's instead of the
@@ -956,8 +994,7 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         ctx->launches += (items > 0 ? 1 : 0) + (pyr_frames > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) +
                          (fish_frames > 0 ? 1 : 0);
     }
-    FT_CUDA(cudaEventRecord(ctx->slot_done[slot], stream));
-    return finish_call(ctx, stream);
+    return guard.end();
 }
 
 }  // namespace
@@ -1380,13 +1417,13 @@ ft_status ft_extract_orb(ft_ctx *ctx, void *stream, const ft_params *params, int
                     scratch);
     cudaStream_t st = (cudaStream_t)stream;
     if ((s = order_stream(ctx, st)) != FT_OK) return s;
+    CallGuard guard(ctx, slot, st);
     if (n > 0) {
         if ((s = send_table(ctx, slot, bytes, st)) != FT_OK) return s;
         FT_CUDA(launch_orb(reinterpret_cast<const OrbHeader *>(dev), n, p.nlevels, max_tiles, nslots, st));
         ctx->launches += 3;
     }
-    FT_CUDA(cudaEventRecord(ctx->slot_done[slot], st));
-    return finish_call(ctx, st);
+    return guard.end();
 }
 
 ft_status ft_pyramid_sizes(int width, int height, const ft_params *params, int *w, int *h)

@@ -1,0 +1,58 @@
+"""The context's host code against a CUDA runtime on host threads: what a call
+that fails half way has enqueued keeps its tables and its order."""
+import pytest
+
+from tests.host_common import fake_library, run_against
+
+SETUP = """
+def batch(n, seed, pyramids=False, fisheye=0, pose=False):
+    fr = [scenes.pinhole_frame(seed + i, W=160, H=120, n_left=40, n_map=60) for i in range(n)]
+    fr += [scenes.fisheye_frame(seed + i, n_left=150, n_map=60) for i in range(fisheye)]
+    return PackedBatch(fr, device='cpu', pin=False, device_pyramids=pyramids, pose=pose)
+
+ctx = Context(arena_bytes=64 << 20, max_frames=8)
+a, b = stream(), stream()
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    return fake_library(tmp_path_factory)
+
+
+def test_table_of_a_failed_call_stays_until_its_kernels_ran(fake):
+    # the pyramid kernel of a call of two frames waits on its stream; the
+    # fused kernel's launch fails; the fourth call after it takes the slot again
+    run_against(fake, SETUP + """
+two, three = batch(2, 1, pyramids=True), batch(3, 5)
+gate = lib.fake_gate(a)
+lib.fake_fail(b'fused', 0)
+assert track(ctx, two, a) == L.FT_ECUDA
+def more():
+    for _ in range(4): L.check(track(ctx, three, a))
+t = threading.Thread(target=more); t.start()
+time.sleep(0.5)
+lib.fake_open(gate)
+t.join()
+lib.cudaStreamSynchronize(a)
+assert log() == ['pyramids 2'] + ['fused 3'] * 4, log()
+ctx.close()
+""")
+
+
+@pytest.mark.parametrize("kind", ["several frames", "one frame"])
+def test_calls_on_another_stream_come_after_a_failed_one(fake, kind):
+    run_against(fake, SETUP + f"""
+one = {kind == "one frame"}
+first = batch(0, 1, fisheye=1) if one else batch(2, 1, pyramids=True)
+gate = lib.fake_gate(a)
+lib.fake_fail(b'fused', 0)
+assert track(ctx, first, a) == L.FT_ECUDA
+L.check(track(ctx, batch(3, 5), b))
+time.sleep(0.3)
+assert log() == [], log()
+lib.fake_open(gate)
+lib.cudaStreamSynchronize(a); lib.cudaStreamSynchronize(b)
+assert log() == ['fisheye one' if one else 'pyramids 2', 'fused 3'], log()
+ctx.close()
+""")
