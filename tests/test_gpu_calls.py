@@ -1,4 +1,6 @@
-"""Forms of a call that the other GPU tests do not reach: the largest batch."""
+"""Forms of a call that the other GPU tests do not reach: the largest batch, and
+graphs with a node of every kernel replayed for other batches of their bucket.
+Compared with the CPU oracle."""
 import ctypes as C
 
 import numpy as np
@@ -7,6 +9,8 @@ import pytest
 import oracle as orc
 from paper_2509_10757_gb300 import scenes
 from tests.gpu_common import assert_fisheye_equal, assert_search_equal
+from tests.test_gpu_parity import _shrink, _with_oracle_pyramids, check_frame
+from tests.test_gpu_pose import check_pose
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -51,3 +55,44 @@ def test_largest_batch_of_fisheye_frames(lib):
         assert_fisheye_equal(out, st, f"frame {f}: ")
         assert_search_equal(out, se, "l", "l", f"frame {f}: ")
         assert_search_equal(out, se, "r", "r", f"frame {f}: ")
+
+
+@pytest.mark.parametrize("pose", [False, True])
+def test_graphs_replay_other_batches_of_their_bucket(lib, pose):
+    # three kernels or four with a fisheye node among them (such calls run as
+    # graphs: test_host_calls): three frames, then four with other counts of
+    # keypoints and points, in turn through all table slots twice and again
+    from paper_2509_10757_gb300.batch import Context, PackedBatch, run_batch
+    q = scenes.fisheye_frame(61, n_left=1500, n_map=4000)
+    groups = [[scenes.single_pinhole(61), q, scenes.single_pinhole(62)],
+              [_shrink(q, nl=1100, nr=700, m=2100), _shrink(scenes.single_pinhole(63), nl=1100, m=2500),
+               scenes.single_pinhole(64), _shrink(scenes.fisheye_frame(62, n_left=1500, n_map=3000), nr=0)]]
+    pbs = [PackedBatch(g, device_pyramids=True, pose=pose) for g in groups]
+    c = Context(arena_bytes=256 << 20, max_frames=8, use_graphs=True)
+    runs = []
+    try:
+        for pb in pbs:
+            pb.upload()
+        for i in range(18):
+            pb = pbs[i % 2]
+            pb.clear_outputs()
+            run_batch(c, pb)
+            if i >= 14:
+                pb.download()
+                runs.append(pb.host_out.numpy().copy())
+        assert c.sync_status() == 0
+    finally:
+        c.close()
+    for k in (0, 1):
+        assert np.array_equal(runs[k], runs[k + 2])
+        for f, fr in enumerate(groups[k]):
+            out = pbs[k].outputs(f)
+            if fr.camera == "fisheye":
+                check_frame(pbs[k], f, what=f"graph of group {k}")
+                continue
+            fr = _with_oracle_pyramids(fr)
+            st, se = orc.track_frame(P, fr)
+            assert_search_equal(out, se, "l", None, f"graph of group {k}, frame {f}: ")
+            if pose:
+                ref = orc.optimize_pose(P, fr.cam, fr.pose, fr.left, st["u_right"], fr.map.pos, se["mp_kp"])
+                check_pose(out, ref, f"graph of group {k}, frame {f}: ")

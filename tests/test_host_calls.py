@@ -1,5 +1,6 @@
-"""The context's host code against a CUDA runtime on host threads: what a call
-that fails half way has enqueued keeps its tables and its order."""
+"""The context's host code against a CUDA runtime on host threads: which calls
+run as graphs, and that what a call that fails half way has enqueued keeps its
+tables and its order."""
 import pytest
 
 from tests.host_common import fake_library, run_against
@@ -55,4 +56,28 @@ lib.fake_open(gate)
 lib.cudaStreamSynchronize(a); lib.cudaStreamSynchronize(b)
 assert log() == ['fisheye one' if one else 'pyramids 2', 'fused 3'], log()
 ctx.close()
+""")
+
+
+@pytest.mark.parametrize("n,fisheye,pyramids,pose,kernels", [
+    (2, 1, True, False, ["pyramids", "fisheye", "fused"]), (2, 1, True, True, ["pyramids", "fisheye", "fused", "pose"]),
+    (3, 0, True, True, ["pyramids", "fused", "pose"]), (2, 1, False, True, ["fisheye", "fused", "pose"]),
+    (2, 1, False, False, ["fisheye", "fused"]), (3, 0, False, False, ["fused"])])
+def test_calls_of_three_kernels_run_as_graphs(fake, n, fisheye, pyramids, pose, kernels):
+    # a graph per table slot and bucket, made at the slot's first call of the
+    # kind and replayed for the other batches of the bucket
+    run_against(fake, SETUP + f"""
+g = Context(arena_bytes=64 << 20, max_frames=8, use_graphs=True)
+first = batch({n}, 1, {pyramids}, {fisheye}, {pose})
+other = batch({n} + 1, 7, {pyramids}, {fisheye}, {pose})
+for _ in range(4): L.check(track(g, first, a))
+for _ in range(4): L.check(track(g, other, a))
+lib.cudaStreamSynchronize(a)
+got = log()
+graphs = {len(kernels)} > 2
+assert got.count('graph made') == (4 if graphs else 0), got
+assert got.count('graph') == (8 if graphs else 0), got
+work = [x for x in got if not x.startswith('graph')]
+assert work == [k + {f"' {n + fisheye}'"} for k in {kernels}] * 4 + [k + {f"' {n + 1 + fisheye}'"} for k in {kernels}] * 4, got
+g.close()
 """)
