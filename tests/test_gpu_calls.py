@@ -1,6 +1,7 @@
 """Forms of a call that the other GPU tests do not reach: the largest batch, and
 graphs with a node of every kernel replayed for other batches of their bucket.
 Compared with the CPU oracle."""
+import copy
 import ctypes as C
 
 import numpy as np
@@ -96,3 +97,52 @@ def test_graphs_replay_other_batches_of_their_bucket(lib, pose):
             if pose:
                 ref = orc.optimize_pose(P, fr.cam, fr.pose, fr.left, st["u_right"], fr.map.pos, se["mp_kp"])
                 check_pose(out, ref, f"graph of group {k}, frame {f}: ")
+
+
+@pytest.mark.parametrize("kind,mode", [("pinhole", "global"), ("fisheye", "global"), ("two", "relaxed"),
+                                       ("pyramids and pose", "relaxed")])
+def test_calls_captured_into_a_callers_graph(lib, kind, mode):
+    # a captured call replays with the inputs its buffers hold then: a frame's
+    # own, another's, its own again, with other calls of the context between
+    from paper_2509_10757_gb300.batch import Context, PackedBatch, run_batch
+    # (the pose and the cameras are part of the call: the other frame has the same)
+    fr = scenes.fisheye_frame(65) if kind == "fisheye" else scenes.single_pinhole(65)
+    other = copy.deepcopy(fr)
+    other.right.desc[::3] ^= 0xff
+    other.map.desc[::3] ^= 0xff
+    more = [scenes.fisheye_frame(67)] if kind == "two" else [scenes.single_pinhole(67)] if "pose" in kind else []
+    kw = dict(device_pyramids=True, pose=True) if "pose" in kind else {}
+    a, b = PackedBatch([fr] + more, **kw), PackedBatch([other] + more, **kw)
+    assert a.lin.size == b.lin.size and a.lout.size == b.lout.size
+    c = Context(arena_bytes=256 << 20, max_frames=8)
+    try:
+        # (all the context's calls on one stream: a captured call cannot wait
+        # for one outside the capture)
+        s = torch.cuda.Stream()
+        want = []
+        for pb in (a, b):
+            pb.upload()
+            pb.clear_outputs()
+            torch.cuda.synchronize()
+            run_batch(c, pb, stream=s)
+            pb.download()
+            want.append(pb.host_out.numpy().copy())
+        if not kw:
+            check_frame(a, 0, what="before the capture")
+        assert not np.array_equal(*want)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s, capture_error_mode=mode):
+            run_batch(c, a, stream=s)
+        for k, src in ((0, a), (1, b), (0, a)):
+            a.dev_in.copy_(src.host_in)
+            a.clear_outputs()
+            torch.cuda.synchronize()
+            g.replay()
+            torch.cuda.synchronize()
+            a.download()
+            assert np.array_equal(a.host_out.numpy(), want[k])
+            run_batch(c, b, stream=s)
+        torch.cuda.synchronize()
+        assert c.sync_status() == 0
+    finally:
+        c.close()
