@@ -1,5 +1,5 @@
-"""The context's host code against a CUDA runtime on host threads: which calls
-run as graphs, and that what a call that fails half way has enqueued keeps its
+"""The context's host code against a CUDA runtime on host threads: how a call's
+table travels, which calls run as graphs, and that what a call that fails half way has enqueued keeps its
 tables and its order."""
 import pytest
 
@@ -80,4 +80,22 @@ assert got.count('graph') == (8 if graphs else 0), got
 work = [x for x in got if not x.startswith('graph')]
 assert work == [k + {f"' {n + fisheye}'"} for k in {kernels}] * 4 + [k + {f"' {n + 1 + fisheye}'"} for k in {kernels}] * 4, got
 g.close()
+""")
+
+
+def test_table_of_a_lone_call_is_one_copy_on_its_stream(fake):
+    # a stream with work takes the table from the context's own stream
+    run_against(fake, SETUP + """
+pb = batch(2, 1)
+for _ in range(5):
+    L.check(track(ctx, pb, a))
+    lib.cudaStreamSynchronize(a)
+assert lib.fake_table_kernels() == 0
+gate = lib.fake_gate(a)
+L.check(track(ctx, pb, a))
+assert lib.fake_table_kernels() == 1
+lib.fake_open(gate)
+lib.cudaStreamSynchronize(a)
+assert log() == ['fused 2'] * 6
+ctx.close()
 """)
