@@ -308,7 +308,8 @@ typedef struct {
     int device;             /* CUDA device ordinal */
     size_t arena_bytes;     /* preallocated scratch (0: 64 MiB) */
     int max_frames;         /* largest batch (0: 256) */
-    int use_graphs;         /* replay ft_track_batch calls of three kernels or more through CUDA graphs */
+    int use_graphs;         /* replay ft_track_batch calls of several frames and three kernels or more
+                               through CUDA graphs */
 } ft_ctx_desc;
 
 typedef struct ft_ctx ft_ctx;
@@ -513,8 +514,8 @@ ft_status ft_build_pyramids(ft_ctx *ctx, void *stream, const ft_params *params, 
 /* Stereo matching followed by the search, for a ragged batch of frames, in
  * one persistent fused launch; fisheye frames' stereo matching, device-built
  * pyramids and pose optimization are a kernel each around it, and a call of
- * three kernels or more is CUDA-graph replayed per batch-shape bucket if the
- * context was created with use_graphs.  Each frame's results equal
+ * several frames and three kernels or more is CUDA-graph replayed per
+ * batch-shape bucket if the context was created with use_graphs.  Each frame's results equal
  * those of the per-frame calls. */
 ft_status ft_track_batch(ft_ctx *ctx, void *stream, const ft_params *params, const ft_batch *batch);
 

@@ -902,9 +902,9 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
     // the search tile as the table uses it
     const int tile = std::max(kThreads, tune.search_tile / kThreads * kThreads);
     if (tune.split_search == 0) tune.split_search = split_pays(jobs, tile, ctx->sm_count * ctx->occ) ? 1 : -1;
-    // one frame goes as kernel parameters (see FrameCall), unless its pyramids
-    // are built first or the launch is traced
-    const bool one = jobs.size() == 1 && !jobs[0].build_pyr && !ctx->trace;
+    // one frame goes as kernel parameters (see FrameCall), unless the launch is
+    // traced
+    const bool one = jobs.size() == 1 && !ctx->trace;
     const int slot = ctx->slot;
     if (!one) {
         ctx->slot = (ctx->slot + 1) % kSlots;
@@ -966,10 +966,12 @@ ft_status submit(ft_ctx *ctx, cudaStream_t stream, const ft_params &params, cons
         // a call's first kernel follows the stream's earlier work as any launch
         // does; only a kernel behind another of the same call may start early
         CallGuard guard(ctx, -1, stream);
+        if (pyr_frames > 0) FT_CUDA(launch_pyramids(call, pyr_blocks, stream));
         FT_CUDA(launch_fisheye(call, fish_blocks, stream));
-        if (items > 0) FT_CUDA(launch_fused(call, std::min(items, grid_max), stream, fish_blocks > 0));
+        if (items > 0)
+            FT_CUDA(launch_fused(call, std::min(items, grid_max), stream, pyr_frames > 0 || fish_blocks > 0));
         if (pose_frames > 0) FT_CUDA(launch_pose(call, stream));
-        ctx->launches += (items > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) + (fish_frames > 0 ? 1 : 0);
+        ctx->launches += (items > 0 ? 1 : 0) + (pyr_frames > 0 ? 1 : 0) + (pose_frames > 0 ? 1 : 0) + (fish_frames > 0 ? 1 : 0);
         return guard.end();
     }
     CallGuard guard(ctx, slot, stream);

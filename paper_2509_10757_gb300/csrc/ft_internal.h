@@ -286,6 +286,7 @@ cudaError_t launch_fused(const BatchHeader *dev_hdr, int grid, cudaStream_t stre
 cudaError_t launch_fused(const FrameCall &call, int grid, cudaStream_t stream, bool overlap);
 cudaError_t launch_pose(const FrameCall &call, cudaStream_t stream);
 cudaError_t launch_fisheye(const FrameCall &call, int blocks, cudaStream_t stream);
+cudaError_t launch_pyramids(const FrameCall &call, int tiles_per_image, cudaStream_t stream);
 // pose optimization of the frames with do_pose (one cluster per frame of the
 // first nframes; after the fused kernel on the same stream)
 cudaError_t launch_pose(const BatchHeader *dev_hdr, int nframes, cudaStream_t stream);

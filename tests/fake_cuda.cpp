@@ -370,6 +370,10 @@ cudaError_t launch_pyramids(const BatchHeader *h, int n, int, int, cudaStream_t 
 {
     return n > 0 ? kernel("pyramids", s, [=] { return frames_of(h); }) : cudaSuccess;
 }
+cudaError_t launch_pyramids(const FrameCall &, int, cudaStream_t s)
+{
+    return kernel("pyramids", s, [] { return std::string("one"); });
+}
 cudaError_t launch_orb(const OrbHeader *h, int n, int, int, int, cudaStream_t s)
 {
     return n > 0 ? kernel("orb", s, [=] { return std::to_string(h->nimages); }) : cudaSuccess;

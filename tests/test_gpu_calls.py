@@ -9,7 +9,7 @@ import pytest
 
 import oracle as orc
 from paper_2509_10757_gb300 import scenes
-from tests.gpu_common import assert_fisheye_equal, assert_search_equal
+from tests.gpu_common import assert_fisheye_equal, assert_search_equal, assert_stereo_equal
 from tests.test_gpu_parity import _shrink, _with_oracle_pyramids, check_frame
 from tests.test_gpu_pose import check_pose
 
@@ -146,3 +146,38 @@ def test_calls_captured_into_a_callers_graph(lib, kind, mode):
         assert c.sync_status() == 0
     finally:
         c.close()
+
+
+@pytest.mark.parametrize("W,H", [(752, 480), (401, 301), (64, 48)])
+def test_one_frame_with_its_pyramids_built(lib, W, H):
+    # one frame travels as kernel parameters, its pyramids' kernel included:
+    # levels, matches and pose, other calls of the context in between
+    from paper_2509_10757_gb300.batch import Context, PackedBatch, run_batch
+    fr = scenes.pinhole_frame(68, W=W, H=H, n_left=min(600, W * H // 60), n_map=800)
+    other = PackedBatch([scenes.single_pinhole(69), scenes.fisheye_frame(69)])
+    other.upload()
+    pb = PackedBatch([fr], device_pyramids=True, pose=True)
+    pb.upload()
+    c = Context(arena_bytes=256 << 20, max_frames=4)
+    try:
+        for _ in range(3):
+            pb.dev_pyr.fill_(0x5a)
+            pb.clear_outputs()
+            n = c.launches()
+            run_batch(c, pb)
+            assert c.launches() - n == 3
+            run_batch(c, other)
+        pb.download()
+        assert c.sync_status() == 0
+    finally:
+        c.close()
+    fr = _with_oracle_pyramids(fr)
+    for side, levels in (("L", fr.pyr_left), ("R", fr.pyr_right)):
+        for l in range(1, len(levels)):
+            assert np.array_equal(pb.device_level(0, side, l), levels[l]), (side, l)
+    st, se = orc.track_frame(P, fr)
+    out = pb.outputs(0)
+    assert_stereo_equal(out, st)
+    assert_search_equal(out, se, "l")
+    ref = orc.optimize_pose(P, fr.cam, fr.pose, fr.left, st["u_right"], fr.map.pos, se["mp_kp"])
+    check_pose(out, ref, f"{W}x{H}: ")

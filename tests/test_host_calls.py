@@ -99,3 +99,19 @@ lib.cudaStreamSynchronize(a)
 assert log() == ['fused 2'] * 6
 ctx.close()
 """)
+
+
+@pytest.mark.parametrize("pyramids,fisheye,pose,kernels", [
+    (False, 0, False, ["fused"]), (True, 0, False, ["pyramids", "fused"]), (True, 0, True, ["pyramids", "fused", "pose"]),
+    (False, 1, False, ["fisheye", "fused"])])
+def test_one_frame_travels_as_kernel_parameters(fake, pyramids, fisheye, pose, kernels):
+    run_against(fake, SETUP + f"""
+pb = batch({1 - fisheye}, 1, {pyramids}, {fisheye}, {pose})
+gate = lib.fake_gate(a)
+L.check(track(ctx, pb, a))
+assert lib.fake_table_kernels() == 0
+lib.fake_open(gate)
+lib.cudaStreamSynchronize(a)
+assert log() == [k + ' one' for k in {kernels}], log()
+ctx.close()
+""")
