@@ -523,12 +523,14 @@ ft_status ft_track_batch(ft_ctx *ctx, void *stream, const ft_params *params, con
  * fastest for the batch's bucket; *best receives it (may be NULL).  The
  * candidates: strip rows 16/32/64, search tile 256/512/1024, every count of
  * CTAs per SM up to the resident maximum, and the search in one pass or two
- * halves. */
+ * halves; and the shape an untuned call takes, which is kept if it is faster
+ * than the best of those by more than 2 %. */
 ft_status ft_autotune(ft_ctx *ctx, void *stream, const ft_params *params, const ft_batch *batch,
                       int iters, ft_tuning *best);
 
 /* Time candidate launch shapes for a stream of batches and keep the fastest
- * in every context for the batches' bucket.  A candidate runs as a sequence
+ * in every context for the batches' bucket.  A candidate (one of ft_autotune's
+ * lists, not the untuned shape) runs as a sequence
  * of launches taken by the n contexts in turn, context i on streams[i] with
  * batches[i] (each context with its own arena and each batch with its own
  * buffers, so later launches start while earlier ones' last frames finish);

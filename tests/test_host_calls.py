@@ -115,3 +115,29 @@ lib.cudaStreamSynchronize(a)
 assert log() == [k + ' one' for k in {kernels}], log()
 ctx.close()
 """)
+
+
+@pytest.mark.parametrize("ms,kept", [(0.9, "untuned"), (0.99, "listed"), (1.0, "listed"), (1.5, "listed")])
+def test_autotuner_meets_the_untuned_shape(fake, ms, kept):
+    # the launches' times by their strips: the shape an untuned call takes is
+    # kept where it is clearly the fastest
+    run_against(fake, SETUP + f"""
+pb = batch(1, 1)
+b = pb.batch()
+def tuning():
+    t = L.ft_tuning()
+    L.check(L.ft_get_tuning(ctx.ptr, C.byref(b), C.byref(t)))
+    return t
+free = tuning()
+assert free.strip_rows not in (16, 32, 64)
+lib.fake_fast_strip.argtypes = [C.c_int, C.c_double]
+lib.fake_fast_strip(free.strip_rows, {ms})
+best = L.ft_tuning()
+L.check(L.ft_autotune(ctx.ptr, a, None, C.byref(b), 2, C.byref(best)))
+for t in (best, tuning()):
+    if {kept == "untuned"}:
+        assert (t.strip_rows, t.search_tile) == (free.strip_rows, free.search_tile), t.strip_rows
+    else:
+        assert t.strip_rows in (16, 32, 64), t.strip_rows
+    assert t.ctas_per_sm in (1, 2, 3) and t.split_search in (1, -1)
+""")
