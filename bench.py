@@ -99,6 +99,32 @@ def progress(msg: str):
     sys.stderr.flush()
 
 
+def within(limit_s: float, run, finish):
+    """finish(run()); if run() has not returned after limit_s, every thread's
+    stack goes to stderr, finish gets the reason in its place, and the process
+    ends: a step that hangs costs its own result and no other."""
+    import faulthandler
+    lock, over = threading.Lock(), []
+
+    def give_up():
+        with lock:
+            if over:
+                return
+            over.append(True)
+            faulthandler.dump_traceback(file=sys.stderr, all_threads=True)
+            finish({"unavailable": f"not ended after {limit_s:g} s (the stacks are on stderr)"})
+            os._exit(0)
+
+    timer = threading.Timer(limit_s, give_up)
+    timer.daemon = True
+    timer.start()
+    result = run()
+    with lock:
+        over.append(True)
+        timer.cancel()
+        finish(result)
+
+
 class ClockSampler:
     """Samples nvidia-smi clocks and throttle reasons while running.  The
     sampler runs from before the warm-up to after the last timed form; mark()
@@ -564,11 +590,13 @@ def serve_load(frames, L, rate_hz: float, seconds: float, n_slots: int, max_batc
                 k = L.ft_server_poll(srv, buf, 512, 2000)
                 for i in range(k):
                     c = buf[i]
+                    if c.status:
+                        failed[0] += 1
                     done.append((c.stream_id, c.t_submit_us, c.t_done_us))
                 if stop.is_set() and k == 0 and time.time() > deadline[0]:
                     break
 
-        submitted, dropped, deadline = [0], [0], [0.0]
+        submitted, dropped, failed, deadline = [0], [0], [0], [0.0]
         th = threading.Thread(target=poller, daemon=True)
         th.start()
         t0 = time.perf_counter()
@@ -593,6 +621,7 @@ def serve_load(frames, L, rate_hz: float, seconds: float, n_slots: int, max_batc
         L.ft_server_get_stats(srv, C.byref(stats))
     finally:
         L.ft_server_destroy(srv)
+    assert failed[0] == 0, f"{failed[0]} requests failed"
     lat = np.array([(b - a) / 1e3 for _, a, b in done]) if done else np.zeros(1)
     t_last = max((b for _, _, b in done), default=0.0)
     t_first = min((a for _, a, _ in done), default=0.0)
@@ -677,6 +706,13 @@ def fisheye_pairs(frames) -> int:
     return n
 
 
+def tuning_of(t) -> dict:
+    """A launch shape as the report gives it."""
+    return {"strip_rows": t.strip_rows, "search_tile": t.search_tile, "fisheye_tile": t.fisheye_tile,
+            "ctas_per_sm": t.ctas_per_sm, "search_stage": "L2" if t.search_stage else "on chip if it fits",
+            "split_search": {1: "two halves", -1: "one pass"}.get(t.split_search, "automatic")}
+
+
 def time_batch(frames, steps: int, warmup: int, dev, local_rank: int, arena_bytes: int, lasts=None,
                pose: bool = False) -> dict:
     """One fused launch per step over `frames` (autotuned tiles,
@@ -724,10 +760,7 @@ def time_batch(frames, steps: int, warmup: int, dev, local_rank: int, arena_byte
            "value": (kp + mp) / mean_s, "unit": UNIT,
            "hbm": {"achieved_gbs": alg / mean_s / 1e9, "frac": alg / mean_s / 1e9 / peaks["hbm_gbs"],
                    "algorithmic_bytes": alg},
-           "tuning": {"strip_rows": best.strip_rows, "search_tile": best.search_tile,
-                      "fisheye_tile": best.fisheye_tile, "ctas_per_sm": best.ctas_per_sm,
-                      "search_stage": "L2" if best.search_stage else "on chip if it fits",
-                      "split_search": {1: "two halves", -1: "one pass"}.get(best.split_search, "automatic")}}
+           "tuning": tuning_of(best)}
     ctx.close()
     return out
 
@@ -1233,19 +1266,10 @@ def run_gpu(args, rank, world, local_rank):
         cpu = time_oracle(frames, budget_s=12.0)
         cpu["all_cores"] = time_oracle_all_cores(frames, budget_s=8.0)
         clocks.mark("cpu_baseline", False)
-    served = None
-    if rank == 0 and world == 1 and not args.no_served:
-        clocks.mark("served", True)
-        served = run_served(args, local_rank, seconds=4.0)
-        clocks.mark("served", False)
-    clk = clocks.stop()
-    def tuning_of(t):
-        return {"strip_rows": t.strip_rows, "search_tile": t.search_tile, "fisheye_tile": t.fisheye_tile,
-                "ctas_per_sm": t.ctas_per_sm, "search_stage": "L2" if t.search_stage else "on chip if it fits",
-                "split_search": {1: "two halves", -1: "one pass"}.get(t.split_search, "automatic")}
     ctx_tuning = tuning_of(best_stream)
     ctx.close()
     if rank != 0:
+        clocks.stop()
         return
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
@@ -1322,13 +1346,27 @@ def run_gpu(args, rank, world, local_rank):
         "pose_optimization": pose,
         "extraction": extraction,
         "gpu_launches": launches,
-        "clocks": clk,
     }
     if cpu is not None:
         line["cpu_baseline"] = cpu
-    if served is not None:
-        line["served"] = served
-    print(json.dumps(line), flush=True)
+
+    def finish(served):
+        line["clocks"] = clocks.stop()
+        if served is not None:
+            line["served"] = served
+        print(json.dumps(line), flush=True)
+
+    if world > 1 or args.no_served:
+        finish(None)
+        return
+    clocks.mark("served", True)
+
+    def sweep():
+        served = run_served(args, local_rank, seconds=4.0)
+        clocks.mark("served", False)
+        return served
+
+    within(float(os.environ.get("FT_BENCH_SERVED_LIMIT_S", "300")), sweep, finish)
 
 
 def main():
