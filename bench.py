@@ -708,8 +708,7 @@ def fisheye_pairs(frames) -> int:
 
 def tuning_of(t) -> dict:
     """A launch shape as the report gives it."""
-    return {"strip_rows": t.strip_rows, "search_tile": t.search_tile, "fisheye_tile": t.fisheye_tile,
-            "ctas_per_sm": t.ctas_per_sm, "search_stage": "L2" if t.search_stage else "on chip if it fits",
+    return {"strip_rows": t.strip_rows, "search_tile": t.search_tile, "ctas_per_sm": t.ctas_per_sm,
             "split_search": {1: "two halves", -1: "one pass"}.get(t.split_search, "automatic")}
 
 
@@ -889,8 +888,9 @@ def small_batch_result(steps: int, warmup: int, dev, local_rank: int) -> dict:
         for name, split in (("two_halves_ms", 1), ("one_pass_ms", -1)):
             ctx = Context(device=local_rank, arena_bytes=512 << 20, max_frames=16, use_graphs=True)
             b = pb.batch()
-            t = L.ft_tuning(strip_rows=32, search_tile=512, fisheye_tile=128, resolve_tile=2048, ctas_per_sm=0,
-                            search_stage=0, split_search=split)
+            t = L.ft_tuning()
+            L.check(ctx.lib.ft_get_tuning(ctx.ptr, C.byref(b), C.byref(t)), "ft_get_tuning")
+            t.split_search = split
             L.check(ctx.lib.ft_set_tuning(ctx.ptr, C.byref(b), C.byref(t)), "ft_set_tuning")
             for _ in range(warmup):
                 run_batch(ctx, pb)
@@ -910,7 +910,8 @@ def small_batch_result(steps: int, warmup: int, dev, local_rank: int) -> dict:
         out[str(n)] = row
     return {"frames": out, "steps": steps,
             "form": "one context, one stream, L2 flushed before each launch, median of launches "
-                    "timed alone; default launch shape with the search in two halves or in one pass"}
+                    "timed alone; the launch shape of an untuned call with the search in two halves (its own "
+                    "choice at these sizes) or in one pass"}
 
 
 def stress_result(n: int, steps: int, warmup: int, dev, local_rank: int) -> dict:
