@@ -234,8 +234,7 @@ ft_tuning shape_for(const std::vector<Job> &jobs, int slots)
         if (j.do_search) points += j.map.n;
     }
     if (rows > 0) {
-        t.strip_rows = (int)std::min<long long>(std::max<long long>(rows / 320, 4), 32);
-        if (rows / 48 > 600) t.strip_rows = 48;
+        t.strip_rows = strip_rows_for(rows);
     }
     if (points > 0) {
         t.search_tile = 256;
@@ -460,6 +459,14 @@ DevParams ft::make_dev_params(const ft_params &p)
         d.halo_c[o] = (int)std::ceil(d.band_r[std::min(o, std::max(p.nlevels - 1, 0))]) + 3;
     }
     return d;
+}
+
+// The strip height that suits a call of `rows` image rows over all its frames
+// (measured at shape_for).
+int ft::strip_rows_for(long long rows)
+{
+    if (rows / 48 > 600) return 48;
+    return (int)std::min<long long>(std::max<long long>(rows / 320, 4), 32);
 }
 
 // Strip height of the pinhole stereo items: at most `want` rows and the

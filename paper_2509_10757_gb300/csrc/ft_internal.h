@@ -315,5 +315,6 @@ void set_last_error(const char *msg);
 // host checks and derived tables shared by the entry points (ft_api.cu)
 ft_status check_params(const ft_params &p);   // FT_EINVAL + ft_last_error() text on a bad field
 DevParams make_dev_params(const ft_params &p);
+int strip_rows_for(long long rows);
 int stereo_strip_rows(int want, int H, int nr, int halo);
 }  // namespace ft

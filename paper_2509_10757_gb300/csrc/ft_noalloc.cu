@@ -233,8 +233,8 @@ ft_status ft_stereo_match_pinhole_noalloc(void *stream, const ft_params *params,
     F.ls_desc = reinterpret_cast<uint4 *>(d + o_lds);
     F.rs_kp = reinterpret_cast<float4 *>(d + o_rkp);
     F.rs_desc = reinterpret_cast<uint4 *>(d + o_rds);
-    // strips of 32 rows (the context's default), shortened by the same rule
-    const int sr = stereo_strip_rows(32, H, R.n, B.p.halo);
+    // strips as an untuned context call of one frame cuts them
+    const int sr = stereo_strip_rows(strip_rows_for(H), H, R.n, B.p.halo);
     F.strip_rows = sr;
     F.n_stereo_items = (H + sr - 1) / sr;
     F.rowsort = kRowSortItems;

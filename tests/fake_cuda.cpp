@@ -115,7 +115,7 @@ std::set<long> g_host;                          // host functions enqueued and n
 long g_next = 0;
 std::atomic<int> g_host_delay_us{0}, g_table_kernels{0};
 std::atomic<double> g_clock_ms{0};               // by the one-frame launches so far
-std::atomic<int> g_fast_strip{0};
+std::atomic<int> g_fast_strip{0}, g_last_strip{0};
 std::atomic<double> g_fast_ms{1};
 thread_local cudaError_t t_error = cudaSuccess;
 
@@ -171,6 +171,7 @@ void fake_fail(const char *name, int after)
 void fake_host_delay(int us) { g_host_delay_us = us; }
 // a one-frame launch takes 1 ms, with strips of `rows` rows `ms`
 void fake_fast_strip(int rows, double ms) { g_fast_strip = rows, g_fast_ms = ms; }
+int fake_last_strip() { return g_last_strip; }     // of the first frame of the last launch that ran
 int fake_table_kernels() { return g_table_kernels; }
 void *fake_gate(cudaStream_t s)                 // the stream stands here until the gate opens
 {
@@ -354,12 +355,12 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t, dim3, dim3, void **, size_t, cudaSt
 namespace ft {
 cudaError_t launch_fused(const BatchHeader *h, int, cudaStream_t s, bool)
 {
-    return kernel("fused", s, [=] { return frames_of(h); });
+    return kernel("fused", s, [=] { return g_last_strip = h->frames[0].strip_rows, frames_of(h); });
 }
 cudaError_t launch_fused(const FrameCall &call, int, cudaStream_t s, bool)
 {
     g_clock_ms = g_clock_ms + (call.f.strip_rows == g_fast_strip ? g_fast_ms.load() : 1.0);
-    return kernel("fused", s, [] { return std::string("one"); });
+    return kernel("fused", s, [n = call.f.strip_rows] { return g_last_strip = n, std::string("one"); });
 }
 cudaError_t launch_pose(const BatchHeader *h, int n, cudaStream_t s)
 {

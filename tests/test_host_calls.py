@@ -141,3 +141,22 @@ for t in (best, tuning()):
         assert t.strip_rows in (16, 32, 64), t.strip_rows
     assert t.ctas_per_sm in (1, 2, 3) and t.split_search in (1, -1)
 """)
+
+
+@pytest.mark.parametrize("W,H,right", [(752, 480, 1250), (640, 481, 600), (1280, 720, 4000), (320, 4000, 500), (64, 30, 9)])
+def test_allocation_free_stereo_cuts_the_contexts_strips(fake, W, H, right):
+    run_against(fake, SETUP + f"""
+from paper_2509_10757_gb300.batch import pinhole_struct
+pb = batch(1, 1)
+fr, st, out = pb.frames[0], pb.stereo_frame(0), pb.stereo_out(0)
+cam = pinhole_struct(fr.cam)
+cam.width, cam.height, st.right.n = {W}, {H}, {right}
+L.check(L.ft_stereo_match_pinhole(ctx.ptr, a, None, C.byref(cam), C.byref(st), C.byref(out)))
+lib.cudaStreamSynchronize(a)
+want = lib.fake_last_strip()
+assert 0 < want <= 32
+L.check(L.ft_stereo_match_pinhole_noalloc(a, None, C.byref(cam), C.byref(st), C.byref(out), None))
+lib.cudaStreamSynchronize(a)
+assert log() == ['fused one', 'fused 1'] and lib.fake_last_strip() == want
+ctx.close()
+""")
