@@ -678,12 +678,12 @@ ft_status ft_server_create(ft_server **out, const ft_server_desc *desc, const ft
 void ft_server_destroy(ft_server *s);
 /* Admit a stream (FT_EBUSY: the HBM budget cannot hold it now). */
 ft_status ft_server_open_stream(ft_server *s, const ft_stream_desc *d, int *stream_id);
-/* Release a stream's block (FT_EBUSY while it has requests queued or running). */
+/* Release a stream's block (FT_EBUSY while it has requests being submitted, queued or running). */
 ft_status ft_server_close_stream(ft_server *s, int stream_id);
 /* Upload a stream's resident pyramids / local map from host memory (synchronous). */
 ft_status ft_server_set_pyramids(ft_server *s, int stream_id, const ft_pyramid *left, const ft_pyramid *right);
 ft_status ft_server_set_map(ft_server *s, int stream_id, const ft_map_view *map);
-/* Queue one frame (FT_EBUSY: the stream already has two frames waiting). */
+/* Queue one frame (FT_EBUSY: the stream already has queue_depth frames waiting). */
 ft_status ft_server_submit(ft_server *s, const ft_request *req);
 /* Move up to max completions to out, waiting up to timeout_us for the first;
  * returns how many. */

@@ -567,7 +567,7 @@ __device__ __forceinline__ void write_stereo(const FrameDev &F, int i, int best,
     F.depth[i] = dep;
 }
 
-// Phase 1: the 8 lanes of a group scan the band candidates of one left
+// Phase 1: the kGroup lanes of a group scan the band candidates of one left
 // keypoint (consecutive candidates per lane, conflict-free shared loads) and
 // reduce to the smallest (distance, right index); lane 0 of the group queues
 // the match for refinement or writes the final "no match" outputs.

@@ -439,7 +439,7 @@ __device__ unsigned kth_key(const unsigned *list, int n, unsigned prefix, int fr
 // ranked by counting, all threads sharing the comparisons; more are sorted by
 // a bitonic network.  What bounds it is the chain of block-wide steps: four
 // histogram passes over device memory, a gather and a 45-step network took 24
-// us for two images' levels, this form 12 us.
+// us for two images' levels, this form 14 us.
 __global__ void __launch_bounds__(kOrbSelectThreads) orb_select_kernel(const OrbHeader *__restrict__ hdr)
 {
     __shared__ __align__(16) unsigned keys[kOrbMaxSlots];

@@ -129,7 +129,7 @@ struct PyrLevelInfo {
 };
 
 // A tile's output row of a level in the row table: its upper source row r0
-// (offset in floats of the staged tile; the lower one is the next staged
+// (offset in words of the staged tile; the lower one is the next staged
 // row), weights fy and 1 - fy, and the row's byte offset in the level.
 struct alignas(16) PyrRow {
     unsigned r0;
