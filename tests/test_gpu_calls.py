@@ -181,3 +181,28 @@ def test_one_frame_with_its_pyramids_built(lib, W, H):
     assert_search_equal(out, se, "l")
     ref = orc.optimize_pose(P, fr.cam, fr.pose, fr.left, st["u_right"], fr.map.pos, se["mp_kp"])
     check_pose(out, ref, f"{W}x{H}: ")
+
+
+@pytest.mark.parametrize("strip", [4, 24, 48])
+@pytest.mark.parametrize("tile", [256, 1024])
+@pytest.mark.parametrize("split", [1, -1])
+def test_shapes_of_untuned_calls(lib, strip, tile, split):
+    # the strip heights, search tiles and search forms the launch rule picks,
+    # on frames it does not pick them for
+    from paper_2509_10757_gb300.batch import Context, PackedBatch, run_batch
+    pb = PackedBatch([scenes.single_pinhole(70), scenes.fisheye_frame(70),
+                      scenes.pinhole_frame(70, W=1280, H=720, n_left=3000, n_map=5000)])
+    pb.upload()
+    pb.clear_outputs()
+    c = Context(arena_bytes=256 << 20, max_frames=4)
+    try:
+        b = pb.batch()
+        t = lib.ft_tuning(strip_rows=strip, search_tile=tile, resolve_tile=2048, split_search=split)
+        lib.check(lib.ft_set_tuning(c.ptr, C.byref(b), C.byref(t)), "ft_set_tuning")
+        run_batch(c, pb)
+        pb.download()
+        assert c.sync_status() == 0
+    finally:
+        c.close()
+    for f in range(3):
+        check_frame(pb, f, what=f"strips of {strip}, tiles of {tile}, split {split}")
